@@ -16,6 +16,20 @@ struct OwnerCode {
   int32_t *code = nullptr;
 };
 
+// What the lockstep ring sweeps need beside it (sweeps.cu), made on their
+// first use: chunk c is slots 32 c .. 32 c + 31 of the padded order, its plan
+// rows are coff[c] .. coff[c + 1] - 1 (the longest chain of the chunk), and
+// slot[32 r + lane] says where the input of that chain entry sits in the
+// order (or ~row when it lies too far back for the ring).
+struct LanePlan {
+  int64_t nch = 0;
+  int maxw = 0;                    // longest chain
+  const int64_t *coff = nullptr;   // int64[nch + 1]
+  const int64_t *first = nullptr;  // per slot: position in F of the chain's first entry
+  const int32_t *len = nullptr;    // per slot: chain length
+  const int32_t *slot = nullptr;
+};
+
 struct LevelOrder {
   int32_t *order = nullptr;   // levels padded to multiples of 32 slots (-1 fills)
   int64_t *lstart = nullptr;  // int64[nlev+1]: first slot of each level
@@ -24,6 +38,7 @@ struct LevelOrder {
   int32_t *corder = nullptr;  // the same rows without padding (clen = rows)
   int64_t clen = 0;
   OwnerCode owner[8];         // cache, see OwnerCode
+  LanePlan plan;
 };
 void level_order_free(LevelOrder &lo, cudaStream_t s);
 

@@ -272,5 +272,8 @@ void level_order_free(LevelOrder &lo, cudaStream_t s) {
   if (lo.lstart) cudaFreeAsync(lo.lstart, s);
   for (OwnerCode &oc : lo.owner)
     if (oc.code) cudaFreeAsync(oc.code, s);
+  for (const void *p : {(const void *)lo.plan.coff, (const void *)lo.plan.first,
+                        (const void *)lo.plan.len, (const void *)lo.plan.slot})
+    if (p) cudaFreeAsync(const_cast<void *>(p), s);
   lo = LevelOrder();
 }

@@ -20,15 +20,19 @@
 //    Suits deep, narrow DAGs, where the hand-off latency sets the time.
 //  * WARP_GRID: the same over all SMs with x in global memory (L2 hand-offs);
 //    suits wide DAGs, which need many SMs in flight.
-//  * FLAGS / SINGLE_CTA / CLUSTER: 32 rows of one level per warp in lockstep
-//    (all SMs through L2, one SM, or one cluster); they pack the FP64 work
-//    of 32 rows into each instruction but couple the rows of a warp.
+//  * FLAGS: 32 rows of one level per warp in lockstep over all SMs (L2
+//    hand-offs); packs the FP64 work of 32 rows into each instruction but
+//    couples the rows of a warp.
+//  * SINGLE_CTA / CLUSTER: the same on one SM or on a small cluster, x handed
+//    over through a ring in shared memory; for rows of at most 16 entries
+//    (longer ones run as WARP_GRID).  Suits narrow DAGs of short rows.
 // Rows are taken in level order (padded to warps for the lockstep kernels);
 // every wait is bounded.
 //
 // The transposed solve (L~U~)^-T p runs the same kernels on an explicit CSR
 // transpose T = F^T: forward with division by t_ii (U~^T), then backward with
 // unit diagonal (L~^T).
+#include <climits>
 #include <cstring>
 #include <mutex>
 
@@ -52,22 +56,14 @@ constexpr int kGridThreads = 256;
 constexpr unsigned long long kPending = 0x7FF0DEADBEEFCAFEull;
 constexpr unsigned long long kQuietNaN = 0x7FF8000000000000ull;
 
-template <bool GPU_SCOPE>
 __device__ __forceinline__ double ld_val(const double *p) {
   double v;
-  if (GPU_SCOPE)
-    asm volatile("ld.relaxed.gpu.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
-  else
-    asm volatile("ld.relaxed.cta.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+  asm volatile("ld.relaxed.gpu.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
   return v;
 }
 
-template <bool GPU_SCOPE>
 __device__ __forceinline__ void st_val(double *p, double v) {
-  if (GPU_SCOPE)
-    asm volatile("st.relaxed.gpu.global.f64 [%0], %1;" ::"l"(p), "d"(v) : "memory");
-  else
-    asm volatile("st.relaxed.cta.global.f64 [%0], %1;" ::"l"(p), "d"(v) : "memory");
+  asm volatile("st.relaxed.gpu.global.f64 [%0], %1;" ::"l"(p), "d"(v) : "memory");
 }
 
 __device__ __forceinline__ bool pending(double v) {
@@ -86,8 +82,8 @@ __device__ __forceinline__ bool pending(double v) {
 // few lanes it serves.  Each chain still runs left to right in its own lane.
 // `clear` (may alias `in`) gets kPending at position `row` once in[row] has
 // been read, which re-arms the buffer the next sweep writes.
-template <bool FORWARD, bool DIVIDE, bool GPU_SCOPE, int W>
-__global__ void __launch_bounds__(GPU_SCOPE ? kGridThreads : kCtaThreads)
+template <bool FORWARD, bool DIVIDE, int W>
+__global__ void __launch_bounds__(kGridThreads)
 k_sweep(const int32_t *__restrict__ order, int64_t len, const int64_t *__restrict__ rp,
         const int32_t *__restrict__ ci, const int64_t *__restrict__ dg,
         const double *__restrict__ v, const DivPrep *__restrict__ rd, const double *in,
@@ -141,7 +137,7 @@ k_sweep(const int32_t *__restrict__ order, int64_t len, const int64_t *__restric
       for (int u = 0; u < W; ++u) {
         const int e = q0 + u - off;
         if (e >= 0 && e < mylen) {
-          x[u] = ld_val<GPU_SCOPE>(&out[c[u]]);
+          x[u] = ld_val(&out[c[u]]);
           pend |= pending(x[u]);
         }
       }
@@ -157,7 +153,7 @@ k_sweep(const int32_t *__restrict__ order, int64_t len, const int64_t *__restric
           for (int u = 0; u < W; ++u) {
             const int e = q0 + u - off;
             if (e >= 0 && e < mylen && pending(x[u])) {
-              x[u] = ld_val<GPU_SCOPE>(&out[c[u]]);
+              x[u] = ld_val(&out[c[u]]);
               pend |= pending(x[u]);
             }
           }
@@ -170,7 +166,7 @@ k_sweep(const int32_t *__restrict__ order, int64_t len, const int64_t *__restric
           }
           if (__any_sync(FULL_MASK, pend)) {
             __nanosleep(backoff);
-            if (backoff < (GPU_SCOPE ? 256u : 128u)) backoff <<= 1;
+            if (backoff < 256u) backoff <<= 1;
           }
         }
         if (!__all_sync(FULL_MASK, ok)) break;
@@ -194,43 +190,37 @@ k_sweep(const int32_t *__restrict__ order, int64_t len, const int64_t *__restric
     if (row >= 0) {
       if ((unsigned long long)__double_as_longlong(s) == kPending)
         s = __longlong_as_double((long long)kQuietNaN);
-      st_val<GPU_SCOPE>(&out[row], s);
+      st_val(&out[row], s);
     }
   }
 }
 
 // ---------------------------------------------------------------------------
-// Cluster schedule: one thread-block cluster of C CTAs (C up to 16, one per
-// SM).  The sweep's output vector lives in the cluster's distributed shared
-// memory -- x_i in the shared memory of CTA (i mod C), slot i / C -- so a
-// dependency is handed from one SM to another through DSMEM (a few hundred
-// cycles) instead of L2, while the FP64 work spreads over C SMs.  Values are
-// again their own ready flags (kPending until written).  At the end each CTA
-// copies its slice to the global output.  Every CTA reaches the final cluster
-// barrier even after a failure, so no CTA leaves while others may still read
-// its shared memory.
+// The ring.  The SINGLE_CTA and CLUSTER sweeps hand x from row to row through
+// a ring in shared memory: every CTA of the launch holds a copy, slot p of the
+// walked order at entry p mod kRing, and a finished row stores its value into
+// all copies, so a waiting row polls its own SM's shared memory (~46 cycles a
+// look) and a hand-off costs one store's flight (probe, one warp per SM: ~205
+// cycles a hop within an SM, 230-370 pushed to another SM of the cluster,
+// 305-430 when the reader polls the other SM's memory, ~900 through L2).
+// An entry is the value and the slot it belongs to: two 64-bit words, each
+// half of the value beside the 32-bit tag slot + 1, so a reader that finds its
+// tag in both words has the whole value whatever the order the words landed
+// in, any bit pattern is a valid value, and an entry overwritten by a later
+// slot shows a later tag.  A reader then takes the value from the sweep's
+// output in global memory, where every row also stores its result (armed with
+// kPending on entry), and so does a row whose input lies kRingNear or more
+// slots back.  So the ring needs no flow control: it is a cache of the last
+// kRing results, and how far one warp runs ahead of another changes nothing
+// but speed.
 // ---------------------------------------------------------------------------
-// The cluster width C is a power of two (lg = log2 C), so owner and slot
-// are a mask and a shift: the address is computed once per value, off the
-// polling loop.
-__device__ __forceinline__ unsigned dsm_addr(unsigned base, int64_t i, int lg) {
-  unsigned a;
-  const unsigned rank = (unsigned)i & ((1u << lg) - 1u);
-  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(base), "r"(rank));
-  return a + ((unsigned)(i >> lg) << 3);
-}
-
-__device__ __forceinline__ double ld_dsm(unsigned a) {
-  unsigned long long v;
-  asm volatile("ld.relaxed.cluster.shared::cluster.b64 %0, [%1];" : "=l"(v) : "r"(a) : "memory");
-  return __longlong_as_double((long long)v);
-}
-
-__device__ __forceinline__ void st_dsm(unsigned a, double x) {
-  asm volatile("st.relaxed.cluster.shared::cluster.b64 [%0], %1;" ::"r"(a),
-               "l"((unsigned long long)__double_as_longlong(x))
-               : "memory");
-}
+constexpr int kRing = 8192;
+constexpr int kRingNear = kRing - 2048;
+constexpr int kLaneMaxThreads = 256;
+constexpr int kLaneW = 4;        // most entries of a window
+constexpr int kLaneMaxRow = 16;  // and of a row
+// the ring, a spare entry of no tag, and spare entries of every thread
+constexpr size_t kRingBytes = (size_t)(kRing + 1 + kLaneMaxThreads * kLaneW) * 16;
 
 __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
@@ -251,134 +241,320 @@ __device__ __forceinline__ bool cluster_launch_ok(unsigned C, int expect_c, int 
   return ok;
 }
 
-template <bool FORWARD, bool DIVIDE, int W>
-__global__ void __launch_bounds__(kCtaThreads, 1)
-k_sweep_cluster(const int32_t *__restrict__ order, int64_t len, int64_t n,
-                const int64_t *__restrict__ rp, const int32_t *__restrict__ ci,
-                const int64_t *__restrict__ dg, const double *__restrict__ v,
-                const DivPrep *__restrict__ rd, const double *in, double *out, double *clear,
-                DevErr *err, int64_t limit_ns, int expect_c) {
-  extern __shared__ __align__(16) double xs[];  // this CTA's slice of x
-  __shared__ int sfail;
-  unsigned rank, C;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
-  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(C));
-  const int lg = __ffs((int)C) - 1;  // C is a power of two
-  const int64_t slice = (n + C - 1) / C;
-  if (!cluster_launch_ok(C, expect_c, expect_c, (uint64_t)slice * sizeof(double), err)) return;
-  for (int64_t j = threadIdx.x; j < slice; j += blockDim.x)
-    xs[j] = __longlong_as_double((long long)kPending);
-  if (threadIdx.x == 0) sfail = 0;
-  const unsigned base = (unsigned)__cvta_generic_to_shared(xs);
-  cluster_sync_all();
+struct RingCtx {
+  unsigned rank, C, base;  // this CTA's rank and ring, the cluster's width
+};
 
-  const int lane = threadIdx.x & 31;
-  const int64_t gw = (int64_t)rank * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int64_t nw = (int64_t)C * (blockDim.x >> 5);
-  bool ok = true;
-  for (int64_t slot0 = gw * 32; slot0 < len && ok; slot0 += nw * 32) {
-    const int64_t row = order[slot0 + lane];
-    int64_t first = 0, d = 0;
-    int mylen = 0;
-    double s = 0.0;
-    DivPrep rr{0ull, 1.0};
-    if (row >= 0) {
-      d = dg[row];
-      if (DIVIDE) rr = rd[row];  // u_ii and its reciprocal, fetched off the chain
-      if (FORWARD) {
-        first = rp[row];
-        mylen = (int)(d - first);
-      } else {
-        first = rp[row + 1] - 1;
-        mylen = (int)(first - d);
-      }
-      s = in[row];
-      if (clear) clear[row] = __longlong_as_double((long long)kPending);
-    }
-    constexpr int64_t step = FORWARD ? 1 : -1;
-    const int maxlen = __reduce_max_sync(FULL_MASK, mylen);
-    const int off = maxlen - mylen;
-    for (int q0 = 0; q0 < maxlen; q0 += W) {
-      unsigned a[W];
-      double f[W], x[W];
-      bool pend = false;
+// Empty ring (tag 0 belongs to no slot); every CTA's ring is empty when this
+// returns.
+__device__ __forceinline__ void ring_start(const RingCtx &r, uint4 *ring) {
+  for (int j = threadIdx.x; j <= kRing; j += blockDim.x) ring[j] = make_uint4(0u, 0u, 0u, 0u);
+  cluster_sync_all();
+}
+
+__device__ __forceinline__ RingCtx ring_ctx(const uint4 *ring) {
+  RingCtx r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r.rank));
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r.C));
+  r.base = (unsigned)__cvta_generic_to_shared(ring);
+  return r;
+}
+
+// Value x of slot `sl` into the ring of CTA `cta`.
+__device__ __forceinline__ void ring_put(unsigned base, unsigned cta, int64_t sl, double x) {
+  unsigned a;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(base), "r"(cta));
+  a += ((unsigned)sl & (kRing - 1)) << 4;
+  const unsigned long long tag = (unsigned long long)((unsigned)sl + 1u) << 32;
+  asm volatile("st.relaxed.cluster.shared::cluster.v2.b64 [%0], {%1, %2};" ::"r"(a),
+               "l"(tag | (unsigned)__double2loint(x)), "l"(tag | (unsigned)__double2hiint(x))
+               : "memory");
+}
+
+__device__ __forceinline__ void ring_put_local(unsigned base, int64_t sl, double x) {
+  const unsigned tag = (unsigned)sl + 1u;
+  asm volatile("st.volatile.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(
+                   base + (((unsigned)sl & (kRing - 1)) << 4)),
+               "r"((unsigned)__double2loint(x)), "r"(tag), "r"((unsigned)__double2hiint(x)),
+               "r"(tag)
+               : "memory");
+}
+
+// How often (in polls) a waiting warp looks at the clock, the error word and
+// for overwritten entries: that is a round trip to L2, a poll is a shared-
+// memory load.
+constexpr unsigned kRingPolls = 256;
+
+// ---------------------------------------------------------------------------
+// Lockstep sweep on the ring: a warp takes a chunk, 32 rows of one level, a
+// row per lane, and the lanes advance their chains together, a window of
+// entries at a time (lane_take), so one FP64 warp instruction serves 32 rows.
+// An FP64 warp instruction holds its sub-partition's pipe ~76 cycles however
+// few lanes it serves, so on short rows this is what a level costs: the
+// hand-off, and the products and differences of the entries that arrive last.
+// The rows of a chunk are right-aligned, so those are the last NL of every
+// row.  Where an entry's input sits in the walked order comes from the order's
+// plan (LanePlan), its coefficient from F; both are loaded a whole chunk ahead
+// of their use, and the rows they belong to one chunk earlier.  Chunk c belongs
+// to CTA c mod C: neighbours of a level run on different SMs or
+// sub-partitions.
+// What bounds it: the latency of that chain, ~590 cycles a level forward.
+// 2D 64^2 grid, k = 2 (253 levels): one application 0.335 ms with a warp per
+// row on a cluster, 0.177 ms here on one SM; 2D 256^2 (1,021 levels) 1.49 ->
+// 0.85 ms; 3D 20^3, k = 1 (115 levels) 0.215 -> 0.150 ms on four SMs.  On
+// 3D 64^3, k = 2 (378 rows a level) it only equals the warp-per-row grid
+// (1.51 and 1.52 ms), and on 27-point grids it loses: their levels are too
+// wide for a few SMs' FP64 pipes.
+// Other forms measured slower: windows of up to 16 entries polled together
+// with the ready ones multiplied and subtracted as they came (the longer loop
+// body costs more than it saves, 1.6 ms on 256^2), and levels separated by
+// barriers instead of polled values with the loads of later levels between
+// them (2.0 ms: the barrier waits for the slowest warp's bookkeeping).
+// ---------------------------------------------------------------------------
+constexpr int kLaneThreads1 = 256;  // one CTA: more warps, to load further ahead
+constexpr int kLaneThreads = 128;   // a cluster: a warp per sub-partition
+
+struct LaneMeta {
+  int64_t first, coff;  // position of the chain's first entry; the chunk's plan rows
+  int32_t row, len, w;  // row (-1: padding), chain length, longest chain of the chunk
+};
+
+template <int W>
+struct LaneWin {
+  int sl[W];  // slot of the input; ~row: far, read from global memory; kNoSlot: none
+  double f[W];
+};
+constexpr int kNoSlot = INT_MAX;  // reads the spare entry
+
+__device__ __forceinline__ void lane_meta(LaneMeta &m, const int32_t *__restrict__ order,
+                                          const LanePlan &pl, int64_t c, int lane) {
+  m.row = -1;
+  m.len = m.w = 0;
+  m.first = m.coff = 0;
+  if (c < pl.nch) {
+    const int64_t slot = c * 32 + lane;
+    m.row = order[slot];
+    m.len = pl.len[slot];
+    m.first = pl.first[slot];
+    m.coff = pl.coff[c];
+    m.w = (int)(pl.coff[c + 1] - m.coff);
+  }
+}
+
+// Entries q0 .. q0 + W - 1 (those >= 0) of the chunk's right-aligned chains.
+template <bool FORWARD, int W>
+__device__ __forceinline__ void lane_window(LaneWin<W> &wn, const LaneMeta &m, int q0,
+                                            const int32_t *__restrict__ pslot,
+                                            const double *__restrict__ v, int lane) {
+  const int skip = m.w - m.len;
+  const int32_t *ps = pslot + m.coff * 32 + lane;
+  const double *pv = v + (FORWARD ? m.first - skip : m.first + skip);
 #pragma unroll
-      for (int u = 0; u < W; ++u) {
-        const int e = q0 + u - off;
-        if (e >= 0 && e < mylen) {
-          a[u] = dsm_addr(base, ci[first + step * e], lg);
-          f[u] = v[first + step * e];
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < W; ++u) {
-        const int e = q0 + u - off;
-        if (e >= 0 && e < mylen) {
-          x[u] = ld_dsm(a[u]);
-          pend |= pending(x[u]);
-        }
-      }
-      if (__any_sync(FULL_MASK, pend)) {
-        const uint64_t t0 = globaltimer_ns();
-        unsigned backoff = 8;
-        for (unsigned it = 0; __any_sync(FULL_MASK, pend); ++it) {
-          pend = false;
-#pragma unroll
-          for (int u = 0; u < W; ++u) {
-            const int e = q0 + u - off;
-            if (e >= 0 && e < mylen && pending(x[u])) {
-              x[u] = ld_dsm(a[u]);
-              pend |= pending(x[u]);
-            }
-          }
-          const bool stop = (it & 15u) == 15u &&
-                            (*((volatile int *)&sfail) || any_failed(err) ||
-                             (int64_t)(globaltimer_ns() - t0) > limit_ns);
-          if (__any_sync(FULL_MASK, stop)) {
-            ok = false;
-            break;
-          }
-          if (__any_sync(FULL_MASK, pend) && it >= 2) {
-            __nanosleep(backoff);
-            if (backoff < 64u) backoff <<= 1;
-          }
-        }
-        if (!__all_sync(FULL_MASK, ok)) {
-          ok = false;
-          break;
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < W; ++u) {
-        const int e = q0 + u - off;
-        if (e >= 0 && e < mylen) x[u] = __dmul_rn(f[u], x[u]);
-      }
-#pragma unroll
-      for (int u = 0; u < W; ++u) {
-        const int e = q0 + u - off;
-        if (e >= 0 && e < mylen) s = __dsub_rn(s, x[u]);
-      }
-    }
-    if (!ok) {
-      if (lane == 0) {
-        atomicExch(&sfail, 1);
-        if (row >= 0) set_err(err, row, ILUK_ETIMEOUT);
-        else set_err(err, n, ILUK_ETIMEOUT);
-      }
-      break;
-    }
-    if (DIVIDE && row >= 0) s = div_fin(s, rr);
-    if (row >= 0) {
-      if ((unsigned long long)__double_as_longlong(s) == kPending)
-        s = __longlong_as_double((long long)kQuietNaN);
-      st_dsm(dsm_addr(base, row, lg), s);
+  for (int u = 0; u < W; ++u) {
+    const int e = q0 + u;
+    wn.sl[u] = kNoSlot;
+    wn.f[u] = 0.0;
+    if (e >= skip && e >= 0) {
+      wn.sl[u] = ps[e * 32];
+      wn.f[u] = pv[FORWARD ? e : -e];
     }
   }
-  // Every CTA arrives here, so no shared memory is released while read.
+}
+
+// Waits until every lane has the window's inputs, multiplies and subtracts
+// them in order.  What follows the last arrival is on the sweep's critical
+// path, so the loop holds nothing but the loads, the tag comparison and a
+// vote, and the FP64 instructions come after it, unconditionally: one with
+// every lane predicated off would hold the FP64 pipe as long.  An input
+// that is not (or no longer) in the ring is copied from global memory into
+// this thread's own spare entry, and then looked for there.
+template <int W>
+__device__ __forceinline__ bool lane_take(const LaneWin<W> &wn, double &s, unsigned base,
+                                          unsigned own, const double *out,
+                                          const int32_t *__restrict__ order, DevErr *err,
+                                          int64_t limit_ns) {
+  unsigned a[W], want[W];
+  bool far = false;
+#pragma unroll
+  for (int u = 0; u < W; ++u) {
+    // a lane without an entry takes +0.0 from the spare entry of no tag, and
+    // subtracts 0 * 0, which changes no value
+    const bool none = wn.sl[u] == kNoSlot;
+    a[u] = base + ((none ? (unsigned)kRing : (unsigned)wn.sl[u] & (kRing - 1)) << 4);
+    want[u] = none ? 0u : (unsigned)wn.sl[u] + 1u;
+    far |= wn.sl[u] < 0;
+  }
+  double x[W];
+  uint64_t t0 = 0;
+  for (unsigned it = __any_sync(FULL_MASK, far) ? kRingPolls - 1 : 0;; ++it) {
+    uint4 r[W];
+    bool all = true;
+#pragma unroll
+    for (int u = 0; u < W; ++u)
+      asm volatile("ld.volatile.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                   : "=r"(r[u].x), "=r"(r[u].y), "=r"(r[u].z), "=r"(r[u].w)
+                   : "r"(a[u]));
+#pragma unroll
+    for (int u = 0; u < W; ++u) {
+      all = all && r[u].y == want[u] && r[u].w == want[u];
+      x[u] = __hiloint2double((int)r[u].z, (int)r[u].x);
+    }
+    if (__all_sync(FULL_MASK, all)) break;
+    if ((it & (kRingPolls - 1)) == kRingPolls - 1) {
+      if (t0 == 0) t0 = globaltimer_ns();
+      const bool stop = any_failed(err) || (int64_t)(globaltimer_ns() - t0) > limit_ns;
+      if (__any_sync(FULL_MASK, stop)) return false;  // the whole warp gives up together
+      bool again = false;
+#pragma unroll
+      for (int u = 0; u < W; ++u) {
+        if (wn.sl[u] == kNoSlot || (r[u].y == want[u] && r[u].w == want[u])) continue;
+        const bool is_far = wn.sl[u] < 0;
+        if (!is_far && r[u].y <= want[u] && r[u].w <= want[u]) continue;  // not there yet
+        const double g = ld_val(&out[is_far ? ~wn.sl[u] : order[wn.sl[u]]]);
+        if (pending(g)) {
+          again = true;
+          continue;
+        }
+        a[u] = own + u * 16u;
+        asm volatile("st.volatile.shared.v4.u32 [%0], {%1, %2, %3, %2};" ::"r"(a[u]),
+                     "r"((unsigned)__double2loint(g)), "r"(want[u]),
+                     "r"((unsigned)__double2hiint(g)));
+      }
+      if (__any_sync(FULL_MASK, again)) --it;
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < W; ++u) x[u] = __dmul_rn(wn.f[u], x[u]);
+#pragma unroll
+  for (int u = 0; u < W; ++u) s = __dsub_rn(s, x[u]);
+  return true;
+}
+
+// A row's entries sit right-aligned in EN early windows of PW and a last one
+// of NL (a row has at most EN * PW + NL), all loaded a whole chunk ahead of
+// their use.
+template <int PW, int EN, int NL>
+struct LaneChunk {
+  LaneMeta m;
+  LaneWin<PW> win[EN];
+  LaneWin<NL> last;
+  double s;
+};
+
+template <bool FORWARD, int PW, int EN, int NL>
+__device__ __forceinline__ void lane_chunk(LaneChunk<PW, EN, NL> &ch,
+                                           const int32_t *__restrict__ pslot,
+                                           const double *__restrict__ v, const double *in,
+                                           int lane) {
+#pragma unroll
+  for (int w = 0; w < EN; ++w)
+    lane_window<FORWARD, PW>(ch.win[w], ch.m, ch.m.w - NL - (EN - w) * PW, pslot, v, lane);
+  lane_window<FORWARD, NL>(ch.last, ch.m, ch.m.w - NL, pslot, v, lane);
+  ch.s = ch.m.row >= 0 ? in[ch.m.row] : 0.0;
+}
+
+template <bool FORWARD, bool DIVIDE, int PW, int EN, int NL>
+__global__ void __launch_bounds__(kLaneMaxThreads, 1)
+k_sweep_lane(const int32_t *__restrict__ order, LanePlan pl, const double *__restrict__ v,
+             const DivPrep *__restrict__ rd, const double *in, double *out, double *clear,
+             DevErr *err, int64_t limit_ns, int expect_c) {
+  extern __shared__ __align__(16) uint4 ring[];
+  const RingCtx rc = ring_ctx(ring);
+  if (!cluster_launch_ok(rc.C, expect_c, expect_c, kRingBytes, err)) return;
+  ring_start(rc, ring);
+  const int lane = threadIdx.x & 31;
+  const unsigned own = rc.base + (unsigned)(kRing + 1 + threadIdx.x * kLaneW) * 16u;
+  const int64_t step = (int64_t)rc.C * (blockDim.x >> 5);
+  int64_t c = (int64_t)rc.rank + (int64_t)rc.C * (threadIdx.x >> 5);
+  LaneChunk<PW, EN, NL> cur, nxt;
+  lane_meta(cur.m, order, pl, c, lane);
+  lane_meta(nxt.m, order, pl, c + step, lane);
+  lane_chunk<FORWARD, PW, EN, NL>(cur, pl.slot, v, in, lane);
+  bool ok = true;
+  for (; c < pl.nch; c += step) {
+    LaneMeta far;  // the rows of the chunk after the next one
+    lane_meta(far, order, pl, c + 2 * step, lane);
+    lane_chunk<FORWARD, PW, EN, NL>(nxt, pl.slot, v, in, lane);
+    const int32_t row = cur.m.row;
+    DivPrep rr{0ull, 1.0};
+    if (DIVIDE && row >= 0) rr = rd[row];
+    if (clear && row >= 0) clear[row] = __longlong_as_double((long long)kPending);
+    double s = cur.s;
+#pragma unroll
+    for (int w = 0; w < EN; ++w)
+      if (cur.m.w > NL + (EN - 1 - w) * PW && ok)
+        ok = lane_take<PW>(cur.win[w], s, rc.base, own, out, order, err, limit_ns);
+    if (ok) ok = lane_take<NL>(cur.last, s, rc.base, own, out, order, err, limit_ns);
+    if (!ok) {
+      if (row >= 0) set_err(err, row, ILUK_ETIMEOUT);
+      break;
+    }
+    // (a padding lane has no divisor)
+    if (DIVIDE && row >= 0) s = div_fin(s, rr);
+    const int64_t slot = c * 32 + lane;
+    if (rc.C == 1) {
+      ring_put_local(rc.base, slot, s);
+    } else {
+      for (unsigned k = 1; k <= rc.C; ++k)
+        ring_put(rc.base, (rc.rank + k) & (rc.C - 1), slot, s);
+    }
+    // (s comes from a subtraction or a division, never the signalling marker)
+    if (row >= 0) st_val(&out[row], s);
+    cur = nxt;
+    nxt.m = far;
+  }
+  // every CTA arrives here: no shared memory is released while written to
+  __syncwarp();
   cluster_sync_all();
-  for (int64_t j = threadIdx.x; j < slice; j += blockDim.x) {
-    const int64_t i = j * C + rank;
-    if (i < n) out[i] = xs[j];
+}
+
+// Plan of a padded order (LanePlan, internal.h).  Chain entry e of a row is
+// its e-th in subtraction order.
+template <bool FORWARD>
+__global__ void k_lane_rows(const int32_t *__restrict__ order, int64_t nch,
+                            const int64_t *__restrict__ rp, const int64_t *__restrict__ dg,
+                            int32_t *slot_of, int64_t *first, int32_t *len, int32_t *w,
+                            int32_t *maxw) {
+  const int lane = threadIdx.x & 31;
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t c = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; c < nch; c += nw) {
+    const int64_t slot = c * 32 + lane;
+    const int32_t row = order[slot];
+    int64_t f = 0;
+    int l = 0;
+    if (row >= 0) {
+      slot_of[row] = (int32_t)slot;
+      const int64_t d = dg[row];
+      f = FORWARD ? rp[row] : rp[row + 1] - 1;
+      l = (int)(FORWARD ? d - f : f - d);
+    }
+    first[slot] = f;
+    len[slot] = l;
+    const int m = __reduce_max_sync(FULL_MASK, l);
+    if (lane == 0) {
+      w[c] = m;
+      atomicMax(maxw, m);
+    }
+  }
+}
+
+template <bool FORWARD>
+__global__ void k_lane_slots(LanePlan pl, const int32_t *__restrict__ slot_of,
+                             const int32_t *__restrict__ ci, int32_t *pslot) {
+  const int lane = threadIdx.x & 31;
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t c = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; c < pl.nch; c += nw) {
+    const int64_t slot = c * 32 + lane, f = pl.first[slot], off = pl.coff[c];
+    const int len = pl.len[slot], w = (int)(pl.coff[c + 1] - off), skip = w - len;
+    for (int e = 0; e < w; ++e) {
+      int32_t v = 0;
+      if (e >= skip) {
+        const int32_t col = ci[FORWARD ? f + (e - skip) : f - (e - skip)];
+        const int32_t sl = slot_of[col];
+        v = slot - sl < kRingNear ? sl : ~col;
+      }
+      pslot[(off + e) * 32 + lane] = v;
+    }
   }
 }
 
@@ -392,11 +568,23 @@ k_sweep_cluster(const int32_t *__restrict__ order, int64_t len, int64_t n,
 // therefore pays, after its last dependency arrives, only for the rest of its
 // own chain.  SCOPE 0: values in global memory, any number of SMs (a
 // co-resident cooperative grid); SCOPE 1: values in the distributed shared
-// memory of one thread-block cluster (as k_sweep_cluster).
+// memory of one thread-block cluster.
 // ---------------------------------------------------------------------------
+__device__ __forceinline__ double ld_dsm(unsigned a) {
+  unsigned long long v;
+  asm volatile("ld.relaxed.cluster.shared::cluster.b64 %0, [%1];" : "=l"(v) : "r"(a) : "memory");
+  return __longlong_as_double((long long)v);
+}
+
+__device__ __forceinline__ void st_dsm(unsigned a, double x) {
+  asm volatile("st.relaxed.cluster.shared::cluster.b64 [%0], %1;" ::"r"(a),
+               "l"((unsigned long long)__double_as_longlong(x))
+               : "memory");
+}
+
 template <int SCOPE>
 __device__ __forceinline__ double wpr_load(const double *out, unsigned da, int64_t i) {
-  if (SCOPE == 0) return ld_val<true>(&out[i]);
+  if (SCOPE == 0) return ld_val(&out[i]);
   return ld_dsm(da);
 }
 
@@ -432,7 +620,7 @@ __device__ void sweep_prefixes(const int32_t *__restrict__ order, int64_t len,
         const double *pa = &xg[order[ps]];
         const uint64_t t0 = globaltimer_ns();
         for (unsigned it = 0;; ++it) {
-          if (!pending(ld_val<true>(pa))) break;
+          if (!pending(ld_val(pa))) break;
           if ((it & 15u) == 15u &&
               (any_failed(err) || (int64_t)(globaltimer_ns() - t0) > limit_ns)) {
             ok = false;
@@ -444,7 +632,7 @@ __device__ void sweep_prefixes(const int32_t *__restrict__ order, int64_t len,
       if (!__shfl_sync(FULL_MASK, ok ? 1 : 0, 0)) return;  // stop helping
     }
     const int64_t row = order[slot];
-    if (!pending(ld_val<true>(&xg[row]))) continue;  // the row is done already
+    if (!pending(ld_val(&xg[row]))) continue;  // the row is done already
     const int64_t d = dg[row];
     const int64_t first = FORWARD ? rp[row] : rp[row + 1] - 1;
     const int mylen = (int)(FORWARD ? d - first : first - d);
@@ -457,7 +645,7 @@ __device__ void sweep_prefixes(const int32_t *__restrict__ order, int64_t len,
       double prod = 0.0;
       bool have = e >= mylen;
       if (e < mylen) {
-        const double x = ld_val<true>(&xg[ci[first + step * e]]);
+        const double x = ld_val(&xg[ci[first + step * e]]);
         if (!pending(x)) {
           prod = __dmul_rn(v[first + step * e], x);
           have = true;
@@ -548,7 +736,7 @@ sweep_wpr_body(const int32_t *__restrict__ order, int64_t len, int64_t n,
       if ((unsigned)(pk >> 32) == epoch) {
         __threadfence();  // the difference was written before the count
         k0 = (int)(pk & 0xffffffffu);
-        s = ld_val<true>(&pre_s[row]);
+        s = ld_val(&pre_s[row]);
       }
     }
     // where x_row goes: this CTA's slot for the warp's current row
@@ -618,10 +806,10 @@ sweep_wpr_body(const int32_t *__restrict__ order, int64_t len, int64_t n,
               if ((unsigned long long)__double_as_longlong(r) == kPending)
                 r = __longlong_as_double((long long)kQuietNaN);
               if (SCOPE == 0) {
-                st_val<true>(&out[row], r);
+                st_val(&out[row], r);
               } else {
                 st_dsm(sa, r);
-                if (help) st_val<true>(&out[row], r);  // the helpers' copy
+                if (help) st_val(&out[row], r);  // the helpers' copy
               }
             }
           }
@@ -663,10 +851,10 @@ sweep_wpr_body(const int32_t *__restrict__ order, int64_t len, int64_t n,
       s = __longlong_as_double((long long)kQuietNaN);
     if (lane == 0) {
       if (SCOPE == 0) {
-        st_val<true>(&out[row], s);
+        st_val(&out[row], s);
       } else {
         st_dsm(sa, s);
-        if (help) st_val<true>(&out[row], s);  // the helpers' copy
+        if (help) st_val(&out[row], s);  // the helpers' copy
       }
     }
     __syncwarp();
@@ -770,6 +958,82 @@ static const int32_t *owner_codes(const LevelOrder &lo_c, int64_t n, int C, int 
   return slot->code;
 }
 
+static unsigned row_blocks(int64_t n) {
+  int64_t b = (n + 255) / 256;
+  const int64_t cap = (int64_t)num_sms() * 8;
+  return (unsigned)(b > cap ? cap : b < 1 ? 1 : b);
+}
+
+// What the ring kernels need beside a level order, built once per order and
+// kept with it.  Nothing is built while `s` is being captured.
+static std::mutex g_plan_mu;
+
+static bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  cudaStreamIsCapturing(s, &cs);
+  return cs != cudaStreamCaptureStatusNone;
+}
+
+template <bool FORWARD>
+static bool ensure_lane_plan(const LevelOrder &lo_c, int64_t n, const int64_t *rp,
+                             const int32_t *ci, const int64_t *dg, cudaStream_t s) {
+  LevelOrder &lo = const_cast<LevelOrder &>(lo_c);  // a cache of the order
+  std::lock_guard<std::mutex> lk(g_plan_mu);
+  if (lo.plan.slot) return true;
+  if (!lo.order || lo.plan.maxw > kLaneMaxRow || capturing(s)) return false;
+  LanePlan pl;
+  pl.nch = lo.len / 32;
+  int32_t *slot_of = nullptr, *w = nullptr, *len = nullptr, *pslot = nullptr;
+  int64_t *first = nullptr, *coff = nullptr, *scan_tmp = nullptr;
+  auto free_all = [&](bool keep) {
+    for (void *p : {(void *)slot_of, (void *)w, (void *)scan_tmp})
+      if (p) cudaFreeAsync(p, s);
+    if (!keep) {
+      for (void *p : {(void *)len, (void *)first, (void *)coff, (void *)pslot})
+        if (p) cudaFreeAsync(p, s);
+      cudaGetLastError();
+    }
+    return keep;
+  };
+  const size_t nch = (size_t)pl.nch;
+  if (cudaMallocAsync((void **)&slot_of, (size_t)n * 4, s) != cudaSuccess ||
+      cudaMallocAsync((void **)&w, (nch + 1) * 4, s) != cudaSuccess ||
+      cudaMemsetAsync(w + nch, 0, 4, s) != cudaSuccess ||
+      cudaMallocAsync((void **)&len, nch * 32 * 4, s) != cudaSuccess ||
+      cudaMallocAsync((void **)&first, nch * 32 * 8, s) != cudaSuccess ||
+      cudaMallocAsync((void **)&coff, (nch + 1) * 8, s) != cudaSuccess ||
+      cudaMallocAsync((void **)&scan_tmp, (size_t)scan_tmp_elems(pl.nch) * 8, s) != cudaSuccess)
+    return free_all(false);
+  k_lane_rows<FORWARD><<<row_blocks(lo.len), 256, 0, s>>>(lo.order, pl.nch, rp, dg, slot_of,
+                                                          first, len, w, w + nch);
+  note_launch();
+  int64_t rows = 0;
+  int32_t maxw = 0;
+  if (launch_scan_lengths(pl.nch, w, coff, scan_tmp, s) != cudaSuccess ||
+      cudaMemcpyAsync(&rows, coff + nch, 8, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+      cudaMemcpyAsync(&maxw, w + nch, 4, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+      cudaStreamSynchronize(s) != cudaSuccess)
+    return free_all(false);
+  pl.maxw = maxw;
+  if (maxw > kLaneMaxRow) {  // not for these sweeps: remembered by maxw
+    lo.plan = LanePlan();
+    lo.plan.maxw = maxw;
+    return free_all(false);
+  }
+  if (cudaMallocAsync((void **)&pslot, (size_t)(rows > 0 ? rows : 1) * 32 * 4, s) != cudaSuccess)
+    return free_all(false);
+  pl.len = len;
+  pl.first = first;
+  pl.coff = coff;
+  k_lane_slots<FORWARD><<<row_blocks(lo.len), 256, 0, s>>>(pl, slot_of, ci, pslot);
+  note_launch();
+  // complete before another stream's sweep may find it
+  if (cudaStreamSynchronize(s) != cudaSuccess) return free_all(false);
+  pl.slot = pslot;
+  lo.plan = pl;
+  return free_all(true);
+}
+
 __global__ void k_fill_pending(int64_t n, double *x, unsigned long long bits) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x)
@@ -816,17 +1080,19 @@ cudaError_t launch_div_check(int64_t n, const double *a, const double *b, double
   return cudaGetLastError();
 }
 
-// Cluster width for n rows: the largest of 16, 8, 4, 2 whose slices fit in
-// one CTA's shared memory and that the device can schedule (0 when none).
+// Cluster width for n rows: the largest of 16, 8, 4, 2 (at most `widest`)
+// whose slices of x, or `fixed` bytes, fit in one CTA's shared memory and that
+// the device can schedule (0 when none).
 template <typename K>
-static int cluster_width(int64_t n, K kern) {
-  static int cached[64][2] = {};
+static int cluster_width(int64_t n, K kern, size_t fixed = 0, int widest = 16) {
+  static int cached[64][2] = {};  // per kernel type, as every static of a template
   static std::mutex mu;
   int dev = 0;
   cudaGetDevice(&dev);
   const size_t budget = (size_t)max_smem_optin() - 1024;
   for (int C : {16, 8, 4, 2}) {
-    const size_t smem = (size_t)((n + C - 1) / C) * sizeof(double);
+    if (C > widest) continue;
+    const size_t smem = fixed ? fixed : (size_t)((n + C - 1) / C) * sizeof(double);
     if (smem > budget) continue;
     {
       std::lock_guard<std::mutex> lk(mu);
@@ -842,7 +1108,7 @@ static int cluster_width(int64_t n, K kern) {
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)C);
-    cfg.blockDim = dim3(kCtaThreads);
+    cfg.blockDim = dim3(fixed ? kLaneMaxThreads : kCtaThreads);
     cfg.dynamicSmemBytes = smem;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -865,7 +1131,12 @@ static int cluster_width(int64_t n, K kern) {
   return 0;
 }
 
-int cluster_size_for(int64_t n) { return cluster_width(n, k_sweep_cluster<true, false, 4>); }
+// Cluster width of the lockstep ring sweep on this device: four SMs, enough for
+// the levels it suits (eight or sixteen measured the same or slower: every
+// result goes to each CTA's ring), or two (0 when neither can be scheduled).
+static int ring_cluster() {
+  return cluster_width((int64_t)0, k_sweep_lane<true, false, 4, 3, 4>, kRingBytes, 4);
+}
 
 template <typename K, typename... Args>
 static cudaError_t launch_on_cluster(K kern, int C, int threads, size_t smem, cudaStream_t s,
@@ -931,68 +1202,61 @@ static cudaError_t run_sweep(int64_t n, const LevelOrder &lo, const int64_t *rp,
   ProfScope prof_scope(FORWARD ? ILUK_PROF_SWEEP : ILUK_PROF_SWEEP_BWD, s);
   // an empty order: nothing to sweep (n = 0, or a direction the caller skips)
   if (n == 0 || (!lo.order && !lo.corder)) return cudaSuccess;
-  // the helped kind needs its scratch; without it, the plain cluster kind
-  if ((sched & 0xf) == ILUK_SCHED_WARP_CLUSTER_HELP && (!aux || !aux->pre_s || aux->n < n))
-    sched = (sched & ~0xf) | ILUK_SCHED_WARP_CLUSTER;
-  const bool helped = (sched & 0xf) == ILUK_SCHED_WARP_CLUSTER_HELP;
-  if (helped) sched = (sched & ~0xf) | ILUK_SCHED_WARP_CLUSTER;
-  // the lockstep kinds walk the padded level order; an index order (a
-  // factorization that has not built its level orders) has only the plain one
-  const int kind0 = sched & 0xf;
-  const bool padded = kind0 != ILUK_SCHED_WARP_GRID && kind0 != ILUK_SCHED_WARP_CLUSTER;
-  if (padded && !lo.order) return cudaErrorInvalidValue;
-  if (!padded && !lo.corder) return cudaErrorInvalidValue;
   int64_t limit = wait_limit();
-  const int32_t *order = lo.order;
-  int64_t len = lo.len;
   const int w = (sched >> 4) & 0xf;  // CTA width / 128 of the warp-per-row kinds
   const int threads = w ? w * 128 : kCtaThreads;
-  sched &= 0xf;
-  if (sched == ILUK_SCHED_SINGLE_CTA) {
-    k_sweep<FORWARD, DIVIDE, false, 4><<<1, kCtaThreads, 0, s>>>(order, len, rp, ci, dg, v, rd,
-                                                                in, out, clear, err, limit);
-    note_launch();
-    return cudaGetLastError();
+  int kind = sched & 0xf;
+  if (kind == ILUK_SCHED_SINGLE_CTA || kind == ILUK_SCHED_CLUSTER) {
+    if (!lo.order) return cudaErrorInvalidValue;  // an index order: no levels to walk
+    if (ensure_lane_plan<FORWARD>(lo, n, rp, ci, dg, s)) {
+      const bool one = kind == ILUK_SCHED_SINGLE_CTA;
+      const int C = one ? 1 : ring_cluster();
+      const auto kern = lo.plan.maxw <= 4   ? k_sweep_lane<FORWARD, DIVIDE, 2, 1, 2>
+                        : lo.plan.maxw <= 8 ? k_sweep_lane<FORWARD, DIVIDE, 4, 1, 4>
+                                            : k_sweep_lane<FORWARD, DIVIDE, 4, 3, 4>;
+      return launch_on_cluster(kern, C, one ? kLaneThreads1 : kLaneThreads, kRingBytes, s,
+                               (const int32_t *)lo.order, lo.plan, v, rd, in, out, clear, err,
+                               limit, C);
+    }
+    // rows too long for a lane, or no plan (a capture before the first use)
+    kind = ILUK_SCHED_WARP_GRID;
   }
-  if (sched == ILUK_SCHED_WARP_GRID || sched == ILUK_SCHED_WARP_CLUSTER) {
+  if (kind == ILUK_SCHED_WARP_CLUSTER || kind == ILUK_SCHED_WARP_CLUSTER_HELP) {
+    if (!lo.corder) return cudaErrorInvalidValue;
     // one warp per row needs no warp-aligned levels: the unpadded order keeps
     // every warp's next row further ahead and wastes no slot loads
-    order = lo.corder;
-    len = lo.clen;
-  }
-  if (sched == ILUK_SCHED_CLUSTER || sched == ILUK_SCHED_WARP_CLUSTER) {
-    const bool wpr = sched == ILUK_SCHED_WARP_CLUSTER;
-    const int C = wpr ? cluster_width(n, k_sweep_wpr<FORWARD, DIVIDE, 1>)
-                      : cluster_width(n, k_sweep_cluster<FORWARD, DIVIDE, 4>);
+    const int32_t *order = lo.corder;
+    const int64_t len = lo.clen;
+    const int C = cluster_width(n, k_sweep_wpr<FORWARD, DIVIDE, 1>);
     if (C == 0) return cudaErrorInvalidConfiguration;
-    if (wpr) {
-      const int wpc = threads / 32;
-      const int64_t nwc = (int64_t)C * wpc;
-      const size_t wsmem = (size_t)((len + nwc - 1) / nwc * wpc) * sizeof(double);
-      if (wsmem > (size_t)max_smem_optin()) return cudaErrorInvalidConfiguration;
-      const int32_t *owner = owner_codes(lo, n, C, threads, s);
-      if (!owner) return cudaErrorMemoryAllocation;
-      double *no_ps = nullptr;
-      unsigned long long *no_pk = nullptr;
-      unsigned *no_words = nullptr;
-      if (helped && C == kHelpCluster) {  // a second cluster of prefix helpers
-        const int64_t lag = (FORWARD ? kHelpLagFwd : kHelpLagBwd) + nwc;
-        const cudaError_t e =
-            launch_help(k_sweep_wpr_help<FORWARD, DIVIDE>, threads, wsmem, s, order, len, n, rp,
-                        ci, dg, v, rd, in, out, clear, err, limit, owner, aux->pre_s, aux->pre_k,
-                        aux->words, lag, C, 2 * C);
-        if (e == cudaSuccess) return e;
-        cudaGetLastError();  // cannot hold both clusters at once: the plain kind
-      }
-      return launch_on_cluster(k_sweep_wpr<FORWARD, DIVIDE, 1>, C, threads, wsmem, s, order, len,
-                               n, rp, ci, dg, v, rd, in, out, clear, err, limit, owner, no_ps,
-                               no_pk, no_words, (int64_t)0, C, C);
+    const int wpc = threads / 32;
+    const int64_t nwc = (int64_t)C * wpc;
+    const size_t wsmem = (size_t)((len + nwc - 1) / nwc * wpc) * sizeof(double);
+    if (wsmem > (size_t)max_smem_optin()) return cudaErrorInvalidConfiguration;
+    const int32_t *owner = owner_codes(lo, n, C, threads, s);
+    if (!owner) return cudaErrorMemoryAllocation;
+    double *no_ps = nullptr;
+    unsigned long long *no_pk = nullptr;
+    unsigned *no_words = nullptr;
+    // the helped kind needs its scratch; without it, the plain cluster kind
+    if (kind == ILUK_SCHED_WARP_CLUSTER_HELP && aux && aux->pre_s && aux->n >= n &&
+        C == kHelpCluster) {  // a second cluster of prefix helpers
+      const int64_t lag = (FORWARD ? kHelpLagFwd : kHelpLagBwd) + nwc;
+      const cudaError_t e =
+          launch_help(k_sweep_wpr_help<FORWARD, DIVIDE>, threads, wsmem, s, order, len, n, rp,
+                      ci, dg, v, rd, in, out, clear, err, limit, owner, aux->pre_s, aux->pre_k,
+                      aux->words, lag, C, 2 * C);
+      if (e == cudaSuccess) return e;
+      cudaGetLastError();  // cannot hold both clusters at once: the plain kind
     }
-    const size_t smem = (size_t)((n + C - 1) / C) * sizeof(double);
-    return launch_on_cluster(k_sweep_cluster<FORWARD, DIVIDE, 4>, C, kCtaThreads, smem, s, order,
-                             len, n, rp, ci, dg, v, rd, in, out, clear, err, limit, C);
+    return launch_on_cluster(k_sweep_wpr<FORWARD, DIVIDE, 1>, C, threads, wsmem, s, order, len,
+                             n, rp, ci, dg, v, rd, in, out, clear, err, limit, owner, no_ps,
+                             no_pk, no_words, (int64_t)0, C, C);
   }
-  if (sched == ILUK_SCHED_WARP_GRID) {
+  if (kind == ILUK_SCHED_WARP_GRID) {
+    if (!lo.corder) return cudaErrorInvalidValue;
+    const int32_t *order = lo.corder;
+    int64_t len = lo.clen;
     auto kern = k_sweep_wpr<FORWARD, DIVIDE, 0>;
     int bps = 1;  // an explicit width means one CTA of that width per SM
     if (w == 0) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, kCtaThreads, 0);
@@ -1017,11 +1281,15 @@ static cudaError_t run_sweep(int64_t n, const LevelOrder &lo, const int64_t *rp,
     note_launch();
     return e;
   }
-  // Multi-SM: every block must be resident (rows wait on rows of other
-  // blocks), so the grid is launched cooperatively and sized by occupancy.
+  // FLAGS.  Multi-SM: every block must be resident (rows wait on rows of
+  // other blocks), so the grid is launched cooperatively and sized by
+  // occupancy.
+  if (!lo.order) return cudaErrorInvalidValue;
+  const int32_t *order = lo.order;
+  int64_t len = lo.len;
   int bps = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_sweep<FORWARD, DIVIDE, true, 8>,
-                                                kGridThreads, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_sweep<FORWARD, DIVIDE, 8>, kGridThreads,
+                                                0);
   if (bps > 2) bps = 2;
   if (bps < 1) bps = 1;
   int64_t grid = (int64_t)bps * num_sms();
@@ -1030,7 +1298,7 @@ static cudaError_t run_sweep(int64_t n, const LevelOrder &lo, const int64_t *rp,
   void *args[] = {(void *)&order, (void *)&len, (void *)&rp, (void *)&ci, (void *)&dg,
                   (void *)&v, (void *)&rd, (void *)&in, (void *)&out, (void *)&clear,
                   (void *)&err, (void *)&limit};
-  cudaError_t e = cudaLaunchCooperativeKernel((const void *)k_sweep<FORWARD, DIVIDE, true, 8>,
+  cudaError_t e = cudaLaunchCooperativeKernel((const void *)k_sweep<FORWARD, DIVIDE, 8>,
                                               dim3((unsigned)grid), dim3(kGridThreads), args, 0, s);
   note_launch();
   return e;
@@ -1042,9 +1310,10 @@ static cudaError_t run_sweep(int64_t n, const LevelOrder &lo, const int64_t *rp,
 static int usable_sched(int64_t n, int sc) {
   int kind = sc & 0xf, w = (sc >> 4) & 0xf;
   if (kind < ILUK_SCHED_FLAGS || kind > ILUK_SCHED_WARP_CLUSTER_HELP) kind = ILUK_SCHED_WARP_GRID;
-  const bool clustered = kind == ILUK_SCHED_CLUSTER || kind == ILUK_SCHED_WARP_CLUSTER ||
-                         kind == ILUK_SCHED_WARP_CLUSTER_HELP;
-  if (clustered && cluster_size_for(n) == 0) kind = ILUK_SCHED_WARP_GRID;
+  if (kind == ILUK_SCHED_CLUSTER && ring_cluster() == 0) kind = ILUK_SCHED_WARP_GRID;
+  if ((kind == ILUK_SCHED_WARP_CLUSTER || kind == ILUK_SCHED_WARP_CLUSTER_HELP) &&
+      cluster_width(n, k_sweep_wpr<true, false, 1>) == 0)
+    kind = ILUK_SCHED_WARP_GRID;
   const bool per_row = kind == ILUK_SCHED_WARP_GRID || kind == ILUK_SCHED_WARP_CLUSTER ||
                        kind == ILUK_SCHED_WARP_CLUSTER_HELP;
   if (!per_row || w < 2 || w > 8) w = 0;
