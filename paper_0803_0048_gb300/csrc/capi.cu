@@ -293,13 +293,17 @@ void iluk_sym_destroy(iluk_sym *S) {
   delete S;
 }
 
-int iluk_symbolic(const iluk_pattern *A, int k, iluk_sym **out, iluk_info *info, void *stream) {
+static int symbolic_impl(const iluk_pattern *A, int k, iluk_sym **out, iluk_info *info,
+                         void *stream, bool validated) {
   info_init(info);
   if (!out) return fail(info, ILUK_EINVAL);
   *out = nullptr;
   if (k < 0 || k > 250) return fail(info, ILUK_EINVAL);
-  int st = iluk_validate(A, info, stream);
-  if (st != ILUK_OK) return st;
+  int st = ILUK_OK;
+  if (!validated) {
+    st = iluk_validate(A, info, stream);
+    if (st != ILUK_OK) return st;
+  }
   cudaStream_t s = (cudaStream_t)stream;
   const int64_t n = A->n, nnz = A->nnz;
 
@@ -333,6 +337,57 @@ int iluk_symbolic(const iluk_pattern *A, int k, iluk_sym **out, iluk_info *info,
   } while (0)
 
   CKS(dalloc(&err, 1, s));
+  int32_t *maxrow = nullptr;
+  auto drop_maxrow = at_scope_exit([&] { dfree(maxrow, s); });
+  CKS(dalloc(&maxrow, 1, s));
+  CKS(cudaMemsetAsync(maxrow, 0, sizeof(int32_t), s));
+  // what follows F's pattern: the A -> F map and the pivot table
+  auto finish = [&]() -> cudaError_t {
+    cudaError_t e = dalloc(&S->a2f, nnz, s);
+    if (e == cudaSuccess) e = dalloc(&S->arowptr, n + 1, s);
+    if (e == cudaSuccess)
+      e = launch_a2f(n, A->rowptr, A->colind, S->rowptr, S->colind, S->a2f, s);
+    if (e == cudaSuccess) e = dalloc(&S->pinfo, S->nnz, s);
+    if (e == cudaSuccess)
+      e = launch_pivot_info(n, S->rowptr, S->colind, S->diag, S->pinfo, s);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(S->arowptr, A->rowptr, (n + 1) * sizeof(int64_t),
+                          cudaMemcpyDeviceToDevice, s);
+    int32_t mr = 0;
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(&mr, maxrow, sizeof(int32_t), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    S->max_row = mr;
+    return e;
+  };
+  // The levels of fill one after another, without waits (fill.cu); the walk
+  // below takes the patterns whose window they do not, and the compared
+  // variants of k <= 1.
+  if (n > 0 && (k >= 2 || symbolic_variant() == 0)) {
+    const int64_t cols = fill_window(n, A->rowptr, A->colind, s);
+    if (cols > 0) {
+      FillPattern fp;
+      const int64_t row_max = max_smem_optin() / 5 / 32 * 32;
+      CKS(launch_fill_err(err, s));
+      CKS(build_fill_pattern(n, nnz, A->rowptr, A->colind, k, cols, &fp, maxrow, err, row_max, s));
+      S->nnz = fp.nnz;
+      S->rowptr = fp.rowptr;
+      S->colind = fp.colind;
+      S->level = fp.level;
+      S->diag = fp.diag;
+      int64_t row;
+      uint64_t need = 0;
+      st = read_err(err, s, &row, &need);
+      if (st == ILUK_OK) CKS(finish());
+      cleanup();
+      if (st != ILUK_OK) {
+        iluk_sym_destroy(S);
+        return fail(info, st, row, (int64_t)need);
+      }
+      *out = S;
+      return fail(info, ILUK_OK);
+    }
+  }
   CKS(dalloc(&ar.row_off, n, s));
   CKS(dalloc(&ar.row_len, n, s));
   CKS(dalloc(&ar.row_ust, n, s));
@@ -422,24 +477,11 @@ int iluk_symbolic(const iluk_pattern *A, int k, iluk_sym **out, iluk_info *info,
   CKS(cudaMemcpyAsync(&nnzF, S->rowptr + n, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
   CKS(cudaStreamSynchronize(s));
   S->nnz = nnzF;
-  int32_t *maxrow = nullptr;
   CKS(dalloc(&S->colind, nnzF, s));
   CKS(dalloc(&S->level, nnzF, s));
   CKS(dalloc(&S->diag, n, s));
-  CKS(dalloc(&S->a2f, nnz, s));
-  CKS(dalloc(&S->arowptr, n + 1, s));
-  CKS(dalloc(&maxrow, 1, s));
-  CKS(cudaMemsetAsync(maxrow, 0, sizeof(int32_t), s));
   CKS(launch_symbolic_compact(n, ar, S->rowptr, S->colind, S->level, S->diag, maxrow, s));
-  CKS(launch_a2f(n, A->rowptr, A->colind, S->rowptr, S->colind, S->a2f, s));
-  CKS(dalloc(&S->pinfo, nnzF, s));
-  CKS(launch_pivot_info(n, S->rowptr, S->colind, S->diag, S->pinfo, s));
-  CKS(cudaMemcpyAsync(S->arowptr, A->rowptr, (n + 1) * sizeof(int64_t), cudaMemcpyDeviceToDevice, s));
-  int32_t mr = 0;
-  CKS(cudaMemcpyAsync(&mr, maxrow, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-  CKS(cudaStreamSynchronize(s));
-  S->max_row = mr;
-  dfree(maxrow, s);
+  CKS(finish());
   cleanup();
   // The level orders of the two sweeps depend only on the pattern; they are
   // built by the first numeric phase, on a second stream while the
@@ -449,13 +491,18 @@ int iluk_symbolic(const iluk_pattern *A, int k, iluk_sym **out, iluk_info *info,
   return fail(info, ILUK_OK);
 }
 
-// Build the sweeps' level orders of S once (synchronous on `s`).
+int iluk_symbolic(const iluk_pattern *A, int k, iluk_sym **out, iluk_info *info, void *stream) {
+  return symbolic_impl(A, k, out, info, stream, false);
+}
+
+// Build the sweeps' level orders of S once (synchronous on `s`), unless a DAG
+// is deeper than `cap` levels (kLevelsTooDeep: no orders).
 static std::mutex g_levels_mu;
-static int ensure_levels(const iluk_sym *Sc, cudaStream_t s) {
+static int ensure_levels(const iluk_sym *Sc, cudaStream_t s, int64_t cap = INT32_MAX) {
   iluk_sym *S = const_cast<iluk_sym *>(Sc);  // the level orders are a cache of the pattern
   std::lock_guard<std::mutex> lk(g_levels_mu);
   if (S->levels_built) return ILUK_OK;
-  const int st = build_levels_pair(S->n, S->rowptr, S->colind, S->diag, &S->lord, &S->uord, s);
+  const int st = build_levels_pair(S->n, S->rowptr, S->colind, S->diag, &S->lord, &S->uord, (int)cap, s);
   if (st != ILUK_OK) return st;
   S->depth_lower = S->lord.nlev;
   S->depth_upper = S->uord.nlev;
@@ -521,21 +568,31 @@ void iluk_fac_destroy(iluk_fac *F) {
   delete F;
 }
 
+// v0 (may be null): also L x = v0 into F->tmp, which must be pending.
 static int numeric_into(iluk_fac *F, const double *A_val, iluk_info *info, cudaStream_t s,
-                        bool build_levels = true, int32_t *depth = nullptr,
-                        unsigned *maxdepth = nullptr) {
+                        bool build_levels = true, const double *v0 = nullptr) {
   const iluk_sym *S = F->S;
+  // The first factorization of this pattern builds the sweeps' level orders,
+  // first, so that its rows are taken in level order too (3D 64^3, k = 2: 0.8 +
+  // 2.7 ms; in index order beside the build the rows took 17.4 ms); a DAG
+  // deeper than kFirstLevels and narrower than kFirstRows rows a level is not
+  // worth waiting for: its orders are built on a second stream while its rows
+  // go in index order, which costs them little (random band, k = 2: 15,777
+  // levels, 10 rows each).
+  constexpr int64_t kFirstLevels = 2048, kFirstRows = 64;
+  int lst = ILUK_OK;
+  if (build_levels && !S->levels_built) {
+    const int64_t cap = std::max(kFirstLevels, S->n / kFirstRows);
+    lst = ensure_levels(S, s, cap);
+    if (lst != ILUK_OK && lst != kLevelsTooDeep) return fail(info, lst);
+  }
   // the numeric phase's row ticket lives in the handle's scratch
   CK(cudaMemsetAsync(F->sync, 0, sweep_sync_ints(S->n) * sizeof(int), s));
   CK(launch_fill_err(F->err, s));
-  // the numeric phase also fills the reciprocals of the diagonal (after the factorization)
+  // the numeric phase also fills the reciprocals of the diagonal
   CK(launch_numeric(S, A_val, F->val, F->rdiag, reinterpret_cast<unsigned long long *>(F->sync),
-                    F->err, depth, maxdepth, s));
-  // First factorization of this pattern: build the sweeps' level orders on a
-  // second stream meanwhile (they read only the pattern; the numeric kernel
-  // leaves room on every SM for the two level-building CTAs).
-  int lst = ILUK_OK;
-  if (build_levels && !S->levels_built) {
+                    F->err, v0, v0 ? F->tmp : nullptr, s));
+  if (lst == kLevelsTooDeep) {
     cudaStream_t side = nullptr;
     if (cudaStreamCreateWithFlags(&side, cudaStreamNonBlocking) == cudaSuccess) {
       prof_override = ILUK_PROF_OVERLAPPED;
@@ -587,14 +644,6 @@ int iluk_numeric(const iluk_sym *S, const double *A_val, iluk_fac **out, iluk_in
   return ILUK_OK;
 }
 
-// iluk_symbolic + iluk_numeric with the two phases overlapped (k >= 2): one
-// cooperative launch in which some CTAs walk the symbolic rows and the others
-// factor each row as soon as its pattern is final (see k_factor_fused).  The
-// results are those of the two calls bit for bit.  The sweeps of the returned
-// factorization walk index orders until level orders are built (by a later
-// iluk_numeric/iluk_refactor on S, or iluk_sym_depth).  Falls back to the two
-// calls for k <= 1 (rows need no other rows' patterns) and whenever the fused
-// launch cannot run or reports an error (the two calls then report it).
 }  // extern "C"
 
 // A factorization made without level orders (iluk_factor) measured the
@@ -609,16 +658,16 @@ static int levels_if_wide(const iluk_sym *S, const unsigned *maxdepth, iluk_info
   return ensure_levels(S, s);
 }
 
-// iluk_factor, with two additions for iluk_solve: `validated` skips the
-// pattern check the caller has made, and a non-null v0 asks the one-launch
-// path to solve L x = v0 beside its numeric phase (each row's entry of x as
-// soon as the row is factored).  Then *fwd_done tells whether it did: F->tmp
-// holds x and must be consumed by a backward sweep before any other apply.
-// The fallbacks (k <= 1, the two separate phases) leave *fwd_done false and
-// F->tmp pending, as iluk_factor does.
+// iluk_factor, with three additions for iluk_solve: `validated` skips the
+// pattern check of the one-launch path (the caller has made it), `solving` says
+// that sweeps follow, and a non-null v0 asks for L x = v0 beside the numeric
+// phase (each row's entry of x as soon as the row is factored).  Then
+// *fwd_done tells whether it was made: F->tmp holds x and must be consumed by
+// a backward sweep before any other apply.  The fallback to the two calls
+// leaves *fwd_done false and F->tmp pending, as iluk_factor does.
 static int factor_impl(const iluk_pattern *A, const double *A_val, int k, iluk_sym **S_out,
                        iluk_fac **F_out, iluk_info *info, void *stream, bool validated,
-                       const double *v0, bool *fwd_done) {
+                       bool solving, const double *v0, bool *fwd_done) {
   info_init(info);
   if (fwd_done) *fwd_done = false;
   if (!S_out || !F_out || !A || (!A_val && A->nnz > 0)) return fail(info, ILUK_EINVAL);
@@ -639,36 +688,36 @@ static int factor_impl(const iluk_pattern *A, const double *A_val, int k, iluk_s
     *F_out = F2;
     return ILUK_OK;
   };
-  // k <= 1: rows need no other rows' patterns, so the two phases simply run
-  // one after the other, without the level orders (index orders instead)
+  // The two phases one after the other, each over the whole GPU.  Level orders
+  // come between them where the DAG is wide (kWideSweepRows) or a solve's
+  // sweeps gain from them (kSolveSweepRows); else the sweeps walk index orders.
   auto serial = [&]() -> int {
     cudaStream_t s2 = (cudaStream_t)stream;
     iluk_sym *S2 = nullptr;
-    int st2 = iluk_symbolic(A, k, &S2, info, stream);
+    int st2 = symbolic_impl(A, k, &S2, info, stream, validated);
     if (st2 != ILUK_OK) return st2;
     iluk_fac *F2 = new iluk_fac();
     F2->S = S2;
-    cudaError_t e2 = build_index_orders(S2->n, &S2->xlord, &S2->xuord, s2);
+    int64_t levels = S2->n / kWideSweepRows;
+    if (solving)
+      levels = std::max(S2->n / kSolveSweepRows,
+                        S2->max_row <= kRingMaxRow ? kRingLevels : kSolveLevels);
+    st2 = levels > 0 ? ensure_levels(S2, s2, levels) : kLevelsTooDeep;
+    cudaError_t e2 = cudaSuccess;
+    if (st2 == kLevelsTooDeep) e2 = build_index_orders(S2->n, &S2->xlord, &S2->xuord, s2);
     if (e2 == cudaSuccess) e2 = dalloc(&F2->val, S2->nnz, s2);
     if (e2 == cudaSuccess) e2 = dalloc(&F2->sync, sweep_sync_ints(S2->n), s2);
     if (e2 == cudaSuccess) e2 = dalloc(&F2->tmp, S2->n, s2);
     if (e2 == cudaSuccess) e2 = dalloc(&F2->rdiag, S2->n, s2);
     if (e2 == cudaSuccess) e2 = dalloc(&F2->err, 2, s2);
     if (e2 == cudaSuccess) e2 = launch_fill_pending(S2->n, F2->tmp, s2);
-    int32_t *depth = nullptr;
-    unsigned *maxdepth = nullptr;
-    auto depth_bufs = at_scope_exit([&] { dfree(depth, s2); dfree(maxdepth, s2); });
-    if (e2 == cudaSuccess) e2 = dalloc(&depth, S2->n, s2);
-    if (e2 == cudaSuccess) e2 = dalloc(&maxdepth, 1, s2);
-    if (e2 == cudaSuccess) e2 = cudaMemsetAsync(depth, 0, (size_t)S2->n * sizeof(int32_t), s2);
-    if (e2 == cudaSuccess) e2 = cudaMemsetAsync(maxdepth, 0, sizeof(unsigned), s2);
     if (e2 != cudaSuccess) {
-      iluk_fac_destroy(F2);
-      iluk_sym_destroy(S2);
-      return fail(info, e2 == cudaErrorMemoryAllocation ? ILUK_ENOMEM : ILUK_ECUDA);
+      st2 = fail(info, e2 == cudaErrorMemoryAllocation ? ILUK_ENOMEM : ILUK_ECUDA);
+    } else if (st2 == ILUK_OK || st2 == kLevelsTooDeep) {
+      st2 = numeric_into(F2, A_val, info, s2, false, v0);
+    } else {
+      fail(info, st2);
     }
-    st2 = numeric_into(F2, A_val, info, s2, false, depth, maxdepth);
-    if (st2 == ILUK_OK) st2 = levels_if_wide(S2, maxdepth, info, s2);
     if (st2 != ILUK_OK) {
       iluk_fac_destroy(F2);
       iluk_sym_destroy(S2);
@@ -676,15 +725,21 @@ static int factor_impl(const iluk_pattern *A, const double *A_val, int k, iluk_s
     }
     *S_out = S2;
     *F_out = F2;
+    if (fwd_done) *fwd_done = v0 != nullptr && S2->n > 0;
     return ILUK_OK;
   };
-  if (k <= 1 || A->n == 0) return serial();
+  // k >= 2 on a pattern whose rows must wait for one another's patterns
+  // (fill_window): both phases in one launch (k_factor_fused), falling back to
+  // the two calls whenever that cannot run or reports an error.
+  if (k <= 1 || A->n <= 0 || !pattern_args_ok(A)) return serial();
   if (!validated) {
     int st = iluk_validate(A, info, stream);
     if (st != ILUK_OK) return st;
+    validated = true;
   }
   cudaStream_t s = (cudaStream_t)stream;
   const int64_t n = A->n, nnz = A->nnz;
+  if (fill_window(n, A->rowptr, A->colind, s) > 0) return serial();
 
   SymArena ar{};
   DevErr *err = nullptr;
@@ -845,7 +900,7 @@ extern "C" {
 
 int iluk_factor(const iluk_pattern *A, const double *A_val, int k, iluk_sym **S_out,
                 iluk_fac **F_out, iluk_info *info, void *stream) {
-  return factor_impl(A, A_val, k, S_out, F_out, info, stream, false, nullptr, nullptr);
+  return factor_impl(A, A_val, k, S_out, F_out, info, stream, false, false, nullptr, nullptr);
 }
 
 int iluk_refactor(iluk_fac *F, const double *A_val, iluk_info *info, void *stream) {
@@ -909,7 +964,8 @@ static int ensure_transpose(iluk_fac *F, cudaStream_t s) {
   dfree(cursor, s);
   dfree(scan_tmp, s);
   if (!F->tlord.order && S->n) {
-    int st = build_levels_pair(S->n, F->trowptr, F->tcolind, F->tdiag, &F->tlord, &F->tuord, s);
+    int st = build_levels_pair(S->n, F->trowptr, F->tcolind, F->tdiag, &F->tlord, &F->tuord, INT32_MAX,
+                               s);
     if (st != ILUK_OK) return st;
   }
   return ILUK_OK;
@@ -1789,7 +1845,7 @@ int iluk_solve(const iluk_pattern *A, const double *A_val, int k, const double *
     iluk_sym *S = nullptr;
     iluk_fac *F = nullptr;
     int operator()(const double *v1, iluk_fac **Fo, bool *fwd_done, iluk_info *finfo) override {
-      int st2 = factor_impl(A, A_val, k, &S, &F, finfo, stream, true, v1, fwd_done);
+      int st2 = factor_impl(A, A_val, k, &S, &F, finfo, stream, true, true, v1, fwd_done);
       if (st2 == ILUK_OK) st2 = iluk_set_schedule(F, sched);
       if (st2 != ILUK_OK) {
         if (F) iluk_fac_destroy(F);
@@ -1814,8 +1870,8 @@ int iluk_solve(const iluk_pattern *A, const double *A_val, int k, const double *
     // GMRES ended before its first application (b = 0, or x = 0 already
     // within rtol): the factorization still runs, and its failures count
     iluk_info finfo;
-    const int fst = factor_impl(A, A_val, k, &hook.S, &hook.F, &finfo, stream, true, nullptr,
-                                nullptr);
+    const int fst = factor_impl(A, A_val, k, &hook.S, &hook.F, &finfo, stream, true, true,
+                                nullptr, nullptr);
     if (fst != ILUK_OK) {
       if (info) *info = finfo;
       return fst;

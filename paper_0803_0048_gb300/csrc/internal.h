@@ -115,13 +115,23 @@ namespace iluk {
 // Average rows per forward level from which the row kernels (numeric phase,
 // TPIILU build) walking level order leave out the column map for more warps.
 constexpr int64_t kWideLevelRows = 300;
-// Average rows per forward level from which a factorization made without
-// level orders builds them for its sweeps: on DAGs this wide the sweeps in
-// index order starve (C3, 378 rows a level: one application 8.7 ms in index
-// order, 1.5 ms in level order; 27-point 90^3, 1,168 a level: 22.1 / 2.2 ms),
-// on narrower ones index order is as fast or faster (2D 256^2, 64 a level:
-// 1.06 / 1.35 ms; the random band, 10 a level: 15.1 / 15.3 ms).
+// Average rows per forward level from which a factorization in one call
+// builds level orders for its numeric phase and its sweeps: on DAGs this wide
+// index order starves both (C3, 378 rows a level: one application 8.7 ms in
+// index order, 1.5 ms in level order; 27-point 90^3, 1,168 a level: 22.1 / 2.2
+// ms), on narrower ones it is as fast or faster (the random band, 10 a level:
+// 15.1 / 15.3 ms).
 constexpr int64_t kWideSweepRows = 128;
+// A one-call solve, whose sweeps follow, builds them from half that width (27-
+// point 30^3 k = 1, 71 rows a level: one application 0.68 ms in level order,
+// 0.92 in index order) or up to kSolveLevels levels, and up to kRingLevels where
+// F's rows are short enough for the lockstep ring sweeps (sweeps.cu), which need
+// them: building costs ~0.7 us a level, a ring sweep saves ~0.3 us a level of
+// every application (2D 64^2, 16 rows a level: 0.335 -> 0.177 ms).
+constexpr int64_t kSolveSweepRows = 64;
+constexpr int64_t kSolveLevels = 600;
+constexpr int64_t kRingLevels = 8192;
+constexpr int kRingMaxRow = 2 * 16 + 1;
 
 int64_t wait_limit();
 void note_launch();              // counts kernel launches (iluk_launch_count)
@@ -193,19 +203,33 @@ cudaError_t launch_symbolic_compact(int64_t n, const SymArena &ar, const int64_t
 cudaError_t launch_a2f(int64_t n, const int64_t *arp, const int32_t *aci, const int64_t *frp,
                        const int32_t *fci, int32_t *a2f, cudaStream_t s);
 
+// Symbolic phase without waits (fill.cu)
+struct FillPattern {
+  int64_t nnz = 0;
+  int64_t *rowptr = nullptr;
+  int32_t *colind = nullptr;
+  uint8_t *level = nullptr;
+  int64_t *diag = nullptr;
+};
+int64_t fill_window(int64_t n, const int64_t *arp, const int32_t *aci, cudaStream_t s);
+cudaError_t build_fill_pattern(int64_t n, int64_t nnz, const int64_t *arp, const int32_t *aci,
+                               int k, int64_t cols, FillPattern *fp, int32_t *maxrow, DevErr *err,
+                               int64_t max_row, cudaStream_t s);
+
 // Levels (levels.cu): synchronous; allocates both orders on success.
+constexpr int kLevelsTooDeep = -1;
 int build_levels_pair(int64_t n, const int64_t *rp, const int32_t *ci, const int64_t *dg,
-                      LevelOrder *fwd, LevelOrder *bwd, cudaStream_t s);
+                      LevelOrder *fwd, LevelOrder *bwd, int cap, cudaStream_t s);
 
 // Numeric (numeric.cu)
 // The factor values double as ready flags (numeric.cu); fval is overwritten.
 cudaError_t launch_pivot_info(int64_t n, const int64_t *frp, const int32_t *fci,
                               const int64_t *fdiag, int64_t *pinfo, cudaStream_t s);
-// depth/maxdepth (may be null): each row's forward depth and the DAG's
-// depth, zeroed by the caller.
+// v0, xf (may be null): also L x = v0 into xf, which holds the pending marker
+// in every entry, each row's entry as soon as the row is factored.
 cudaError_t launch_numeric(const iluk_sym *S, const double *aval, double *fval, DivPrep *rdiag,
-                           unsigned long long *ticket, DevErr *err, int32_t *depth,
-                           unsigned *maxdepth, cudaStream_t s);
+                           unsigned long long *ticket, DevErr *err, const double *v0, double *xf,
+                           cudaStream_t s);
 cudaError_t launch_numeric_batched(const iluk_sym *S, int64_t nbatch, const double *avals,
                                    double *fvals, unsigned long long *ticket, DevErr *errs,
                                    cudaStream_t s);

@@ -12,72 +12,116 @@
 namespace iluk {
 
 constexpr int kDepthThreads = 512;
+constexpr int kDepthBatch = 4;  // inputs a lane looks at together
 
-// One warp per row, rows claimed in sweep order through a global ticket per
-// direction; depth[] doubles as the ready flag (0 until the row is final),
-// handed over through L2.  A warp claims a row only while it runs, and every
-// row it reads holds an earlier ticket, so the waits end whether or not all
-// CTAs are resident: the launch can share the GPU with the numeric phase, and
-// wide DAGs (thousands of rows per level) get thousands of warps.
+// One row per lane: a warp claims the next 32 rows in sweep order through a
+// global ticket per direction, and its lanes walk their rows' inputs, nearest
+// last, kDepthBatch at a time; a lane that finds an input without a depth yet
+// looks at it again in the warp's next round, while the others go on.
+// depth[] doubles as the ready flag (0 until the row is final), handed over
+// through L2.  A warp claims rows only while it runs, and every row it reads
+// holds an earlier ticket or belongs to the same warp, so the waits end whether
+// or not all CTAs are resident.
+// What bounds it: one L2 round trip (~900 cycles) a level.  With a warp per
+// row the rows in flight (one per warp) covered only a part of a wide DAG's
+// wavefront: 3D 64^3, k = 2 (694 levels) 5.8 ms for both directions.
+// A row deeper than `cap` ends the launch (fail = 2): the caller wants no
+// orders for a DAG that deep.
 template <bool FORWARD>
 __device__ void depth_rows(int64_t n, const int64_t *__restrict__ rp,
                            const int32_t *__restrict__ ci, const int64_t *__restrict__ dg,
                            int32_t *depth, int32_t *maxdepth, DevErr *err, int64_t limit_ns,
-                           unsigned long long *ticket, int *fail) {
+                           unsigned long long *ticket, int *fail, int cap) {
   const int lane = threadIdx.x & 31;
   int dmax_local = 0;
   for (;;) {
     unsigned long long tk = 0;
-    if (lane == 0) tk = atomicAdd(ticket, 1ull);
-    const int64_t t = (int64_t)__shfl_sync(FULL_MASK, tk, 0);
-    if (t >= n) break;
+    if (lane == 0) tk = atomicAdd(ticket, 32ull);
+    const int64_t t = (int64_t)__shfl_sync(FULL_MASK, tk, 0) + lane;
+    if (t - lane >= n) break;
+    if (__any_sync(FULL_MASK, *((volatile int *)fail) != 0)) break;
+    const bool mine = t < n;
     const int64_t row = FORWARD ? t : n - 1 - t;
-    const int64_t d = dg[row];
-    const int64_t b0 = FORWARD ? rp[row] : d + 1;
-    const int64_t b1 = FORWARD ? d : rp[row + 1];
-    int dm = 0;
-    bool ok = true;
-    for (int64_t base = b0; base < b1; base += 32) {
-      const int64_t q = base + lane;
-      int v = 1;
-      const int32_t *src = nullptr;
-      if (q < b1) {
-        src = &depth[ci[q]];
-        asm volatile("ld.relaxed.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(src));
-      }
-      if (__any_sync(FULL_MASK, v == 0)) {
-        const uint64_t t0 = globaltimer_ns();
-        unsigned backoff = 16;
-        for (unsigned it = 0; __any_sync(FULL_MASK, v == 0); ++it) {
-          if (v == 0) asm volatile("ld.relaxed.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(src));
-          const bool stop = (it & 15u) == 15u &&
-                            (*((volatile int *)fail) || (int64_t)(globaltimer_ns() - t0) > limit_ns);
-          if (__any_sync(FULL_MASK, stop)) {  // the whole warp gives up together
-            ok = false;
-            break;
-          }
-          if (it >= 4) {
-            __nanosleep(backoff);
-            if (backoff < 64u) backoff <<= 1;
+    // inputs q = 0 .. len - 1, the nearest row last
+    int64_t first = 0;
+    int len = 0;
+    if (mine) {
+      const int64_t d = dg[row];
+      first = FORWARD ? rp[row] : rp[row + 1] - 1;
+      len = (int)(FORWARD ? d - first : first - d);
+    }
+    int q = 0, dm = 0;
+    bool done = !mine;
+    const uint64_t t0 = globaltimer_ns();
+    unsigned backoff = 16;
+    bool gone = false;
+    for (unsigned it = 0;; ++it) {
+      bool moved = false;
+      if (!done) {
+        int v[kDepthBatch];
+#pragma unroll
+        for (int u = 0; u < kDepthBatch; ++u) {
+          v[u] = 1;
+          if (q + u < len) {
+            const int32_t *src = &depth[ci[FORWARD ? first + q + u : first - q - u]];
+            asm volatile("ld.relaxed.gpu.global.b32 %0, [%1];" : "=r"(v[u]) : "l"(src));
           }
         }
+        bool go = true;
+        int adv = 0;
+#pragma unroll
+        for (int u = 0; u < kDepthBatch; ++u) {
+          go = go && v[u] != 0;
+          if (go && q + u < len) {
+            if (v[u] > dm) dm = v[u];
+            ++adv;
+          }
+        }
+        q += adv;
+        moved = adv > 0;
+        if (q >= len) {
+          ++dm;
+          asm volatile("st.relaxed.gpu.global.b32 [%0], %1;" ::"l"(&depth[row]), "r"(dm)
+                       : "memory");
+          if (dm > dmax_local) dmax_local = dm;
+          if (dm > cap) atomicExch(fail, 2);
+          done = moved = true;
+        }
       }
-      if (!__all_sync(FULL_MASK, ok)) break;
-      if (q < b1 && v > dm) dm = v;
-    }
-    if (!__all_sync(FULL_MASK, ok)) {
-      if (lane == 0) {
-        atomicExch(fail, 1);
-        set_err(err, t, ILUK_ETIMEOUT);
+      if (__all_sync(FULL_MASK, done)) break;
+      if ((it & 15u) == 15u) {
+        const bool late = (int64_t)(globaltimer_ns() - t0) > limit_ns;
+        const bool stop = *((volatile int *)fail) != 0 || late;
+        if (__any_sync(FULL_MASK, stop)) {  // the whole warp gives up together
+          if (late && !done) {
+            atomicCAS(fail, 0, 1);
+            set_err(err, t, ILUK_ETIMEOUT);
+          }
+          gone = true;
+          break;
+        }
       }
-      return;
+      if (!__any_sync(FULL_MASK, moved)) {
+        // far from its inputs: only the first waiting lane looks, at its first
+        // missing input, so that the waiting warps leave L2 to the others
+        const unsigned waiting = __ballot_sync(FULL_MASK, !done);
+        const bool leader = lane == __ffs(waiting) - 1;
+        const int32_t *src = nullptr;
+        if (leader) src = &depth[ci[FORWARD ? first + q : first - q]];
+        for (int k = 0; k < 8; ++k) {
+          __nanosleep(backoff);
+          int v = 0;
+          if (leader) asm volatile("ld.relaxed.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(src));
+          if (__any_sync(FULL_MASK, v != 0)) break;
+        }
+        if (backoff < 256u) backoff <<= 1;
+      } else {
+        backoff = 16;
+      }
     }
-    dm = __reduce_max_sync(FULL_MASK, dm) + 1;
-    if (lane == 0) {
-      asm volatile("st.relaxed.gpu.global.b32 [%0], %1;" ::"l"(&depth[row]), "r"(dm) : "memory");
-      if (dm > dmax_local) dmax_local = dm;
-    }
+    if (gone) break;
   }
+  dmax_local = __reduce_max_sync(FULL_MASK, dmax_local);
   if (lane == 0 && dmax_local) atomicMax(maxdepth, dmax_local);
 }
 
@@ -86,12 +130,12 @@ __device__ void depth_rows(int64_t n, const int64_t *__restrict__ rp,
 __global__ void __launch_bounds__(kDepthThreads)
 k_depth_pair(int64_t n, const int64_t *__restrict__ rp, const int32_t *__restrict__ ci,
              const int64_t *__restrict__ dg, int32_t *depth_f, int32_t *depth_b, int32_t *mx,
-             DevErr *err, unsigned long long *ctl, int64_t limit_ns) {
+             DevErr *err, unsigned long long *ctl, int64_t limit_ns, int cap) {
   int *fail = reinterpret_cast<int *>(ctl + 2);
   if ((blockIdx.x & 1) == 0)
-    depth_rows<true>(n, rp, ci, dg, depth_f, mx, err, limit_ns, ctl, fail);
+    depth_rows<true>(n, rp, ci, dg, depth_f, mx, err, limit_ns, ctl, fail, cap);
   else
-    depth_rows<false>(n, rp, ci, dg, depth_b, mx + 1, err + 1, limit_ns, ctl + 1, fail + 1);
+    depth_rows<false>(n, rp, ci, dg, depth_b, mx + 1, err + 1, limit_ns, ctl + 1, fail + 1, cap);
 }
 
 __global__ void k_level_count(int64_t n, const int32_t *__restrict__ depth, int32_t *cnt) {
@@ -180,11 +224,12 @@ static int order_from_depth(int64_t n, const int32_t *depth, int32_t nlev, Level
   return ILUK_OK;
 }
 
-// Synchronous: the depths of both sweep DAGs (one launch, one block each),
-// then the two padded level orders.  On success fwd->order / bwd->order (and
-// their level starts) are new device allocations.
+// Synchronous: the depths of both sweep DAGs (one launch), then the two padded
+// level orders.  On success fwd->order / bwd->order (and their level starts)
+// are new device allocations.  kLevelsTooDeep (and no orders) when a DAG is
+// deeper than cap.
 int build_levels_pair(int64_t n, const int64_t *rp, const int32_t *ci, const int64_t *dg,
-                      LevelOrder *fwd, LevelOrder *bwd, cudaStream_t s) {
+                      LevelOrder *fwd, LevelOrder *bwd, int cap, cudaStream_t s) {
   ProfScope prof_scope(ILUK_PROF_DEPTH, s);
   *fwd = LevelOrder();
   *bwd = LevelOrder();
@@ -209,14 +254,16 @@ int build_levels_pair(int64_t n, const int64_t *rp, const int32_t *ci, const int
     cleanup();
     return ILUK_ECUDA;
   }
-  // one forward and one backward CTA per SM: 1024 threads, which leaves room
-  // beside the numeric phase's 256-thread CTA when both run at once
-  int64_t grid = 2 * (int64_t)num_sms();
-  const int64_t want = 2 * ((n * 32 + kDepthThreads - 1) / kDepthThreads);
+  // all the rows in flight that the SMs take: half the CTAs of each direction
+  int bps = 0;
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_depth_pair, kDepthThreads, 0);
+  if (bps < 1) bps = 1;
+  int64_t grid = ((int64_t)bps * num_sms() + 1) / 2 * 2;
+  const int64_t want = 2 * ((n + kDepthThreads - 1) / kDepthThreads);
   if (grid > want) grid = want;
   if (grid < 2) grid = 2;
   k_depth_pair<<<(unsigned)grid, kDepthThreads, 0, s>>>(n, rp, ci, dg, depth, depth + n, mx, err,
-                                                        ctl, wait_limit());
+                                                        ctl, wait_limit(), cap);
   note_launch();
   DevErr herr[2];
   int32_t nlev[2] = {0, 0};
@@ -232,6 +279,10 @@ int build_levels_pair(int64_t n, const int64_t *rp, const int32_t *ci, const int
       cleanup();
       return (int)(herr[d].key & 0xff);
     }
+  if (nlev[0] > cap || nlev[1] > cap) {
+    cleanup();
+    return kLevelsTooDeep;
+  }
   int st = order_from_depth(n, depth, nlev[0], fwd, s);
   if (st == ILUK_OK) st = order_from_depth(n, depth + n, nlev[1], bwd, s);
   cleanup();

@@ -373,6 +373,69 @@ __device__ __forceinline__ bool apply_pivots(int dp, double *rv, const int64_t *
   return __all_sync(FULL_MASK, ok);
 }
 
+// The forward substitution L x = v0 (L unit lower triangular, its strictly
+// lower part the multipliers f_ih of Eq. 1) for one row, taken by the warp that
+// has just factored that row: x_i = v0_i - sum over h in L(i), ascending, of
+// f_ih * x_h, each product and each difference rounded once, in the order of
+// the stand-alone forward sweep, so the result is bit for bit the sweep's.
+// The row's multipliers and columns are still in the warp's shared memory.
+// x lives in global memory, filled with kPendingF before the launch; x_h is
+// polled until it leaves that state (the rows that own x_h were claimed
+// earlier and are resident, so every wait ends).  A value that would equal
+// the marker is stored as a quiet NaN, as the sweep does.  Warp-uniform;
+// false on time-out or when a row before `row` has failed.
+__device__ __forceinline__ bool forward_entry(int64_t row, int dp, const double *lmul,
+                                              const int32_t *lcol, const double *v0, double *x,
+                                              const DevErr *err, int64_t limit_ns, int lane) {
+  double s = v0[row];
+  for (int b = 0; b < dp; b += 32) {
+    const int e = b + lane;
+    const bool act = e < dp;
+    const int cnt = dp - b < 32 ? dp - b : 32;
+    double f = 0.0, prod = 0.0;
+    int32_t c = 0;
+    bool have = !act;
+    if (act) {
+      c = lcol[e];
+      f = lmul[e];
+      const double xh = ld_gpu(&x[c]);
+      if (!pend_f(xh)) {
+        prod = __dmul_rn(f, xh);
+        have = true;
+      }
+    }
+    int done = 0;
+    const uint64_t t0 = globaltimer_ns();
+    unsigned backoff = 16;
+    for (unsigned it = 0;; ++it) {
+      // subtract the ready products in order, up to the first missing one
+      const unsigned ready = __ballot_sync(FULL_MASK, have);
+      const unsigned rest = ~(ready >> done);
+      const int run = rest == 0u ? 32 - done : __ffs(rest) - 1;
+      const int upto = done + run < cnt ? done + run : cnt;
+      for (int j = done; j < upto; ++j) s = __dsub_rn(s, __shfl_sync(FULL_MASK, prod, j));
+      done = upto;
+      if (done >= cnt) break;
+      const bool stop = (it & 15u) == 15u &&
+                        (earlier_failed(err, row) || (int64_t)(globaltimer_ns() - t0) > limit_ns);
+      if (__any_sync(FULL_MASK, stop)) return false;
+      __nanosleep(backoff);
+      if (backoff < 128u) backoff <<= 1;
+      if (!have) {
+        const double xh = ld_gpu(&x[c]);
+        if (!pend_f(xh)) {
+          prod = __dmul_rn(f, xh);
+          have = true;
+        }
+      }
+    }
+  }
+  if ((unsigned long long)__double_as_longlong(s) == kPendingF)
+    s = __longlong_as_double((long long)0x7FF8000000000000ll);
+  if (lane == 0) asm volatile("st.relaxed.gpu.global.f64 [%0], %1;" ::"l"(x + row), "d"(s) : "memory");
+  return true;
+}
+
 // Pivot facts per lower entry (i, h) of F: position of row h's diagonal and
 // the length of its strictly upper part, packed for the numeric phase.
 __global__ void k_pivot_info(int64_t n, const int64_t *__restrict__ frp,
@@ -415,7 +478,7 @@ k_numeric(int64_t n, int64_t nbatch, const int64_t *__restrict__ arp,
           const int64_t *__restrict__ fdiag, const int64_t *__restrict__ pinfo, double *fval,
           int64_t fstride, const int32_t *__restrict__ order,
           unsigned long long *ticket, DevErr *errs, int cap, int map_cap, int64_t limit_ns,
-          int64_t hold, DivPrep *rdiag, int32_t *depth, unsigned *maxdepth) {
+          int64_t hold, DivPrep *rdiag, const double *v0, double *xf) {
   // per warp: values, pivot infos (cap each), columns, then the column map
   extern __shared__ __align__(16) unsigned char smem[];
   const int lane = threadIdx.x & 31;
@@ -509,7 +572,11 @@ k_numeric(int64_t n, int64_t nbatch, const int64_t *__restrict__ arp,
         }
       }
       if (rdiag && lane == 0) publish_recip(&rdiag[row], svals[dp]);
-      if (depth) note_depth(row, dp, rc, depth, maxdepth, err, limit_ns, lane);
+      __syncwarp();
+      // the row's entry of L x = v0, when the launch carries a right-hand side
+      if (xf && !forward_entry(row, dp, svals, scols, v0, xf, err, limit_ns, lane)) {
+        if (lane == 0 && !earlier_failed(err, row)) set_err(err, row, ILUK_ETIMEOUT);
+      }
     }
     __syncwarp();
   }
@@ -558,69 +625,6 @@ __device__ __forceinline__ bool wait_word(const unsigned long long *p, unsigned 
       if (backoff < kPollSleepMax) backoff <<= 1;
     }
   }
-}
-
-// The forward substitution L x = v0 (L unit lower triangular, its strictly
-// lower part the multipliers f_ih of Eq. 1) for one row, taken by the warp that
-// has just factored that row: x_i = v0_i - sum over h in L(i), ascending, of
-// f_ih * x_h, each product and each difference rounded once, in the order of
-// the stand-alone forward sweep, so the result is bit for bit the sweep's.
-// The row's multipliers and columns are still in the warp's shared memory.
-// x lives in global memory, filled with kPendingF before the launch; x_h is
-// polled until it leaves that state (the rows that own x_h were claimed
-// earlier and are resident, so every wait ends).  A value that would equal
-// the marker is stored as a quiet NaN, as the sweep does.  Warp-uniform;
-// false on time-out or when a row before `row` has failed.
-__device__ __forceinline__ bool forward_entry(int64_t row, int dp, const double *lmul,
-                                              const int32_t *lcol, const double *v0, double *x,
-                                              const DevErr *err, int64_t limit_ns, int lane) {
-  double s = v0[row];
-  for (int b = 0; b < dp; b += 32) {
-    const int e = b + lane;
-    const bool act = e < dp;
-    const int cnt = dp - b < 32 ? dp - b : 32;
-    double f = 0.0, prod = 0.0;
-    int32_t c = 0;
-    bool have = !act;
-    if (act) {
-      c = lcol[e];
-      f = lmul[e];
-      const double xh = ld_gpu(&x[c]);
-      if (!pend_f(xh)) {
-        prod = __dmul_rn(f, xh);
-        have = true;
-      }
-    }
-    int done = 0;
-    const uint64_t t0 = globaltimer_ns();
-    unsigned backoff = 16;
-    for (unsigned it = 0;; ++it) {
-      // subtract the ready products in order, up to the first missing one
-      const unsigned ready = __ballot_sync(FULL_MASK, have);
-      const unsigned rest = ~(ready >> done);
-      const int run = rest == 0u ? 32 - done : __ffs(rest) - 1;
-      const int upto = done + run < cnt ? done + run : cnt;
-      for (int j = done; j < upto; ++j) s = __dsub_rn(s, __shfl_sync(FULL_MASK, prod, j));
-      done = upto;
-      if (done >= cnt) break;
-      const bool stop = (it & 15u) == 15u &&
-                        (earlier_failed(err, row) || (int64_t)(globaltimer_ns() - t0) > limit_ns);
-      if (__any_sync(FULL_MASK, stop)) return false;
-      __nanosleep(backoff);
-      if (backoff < 128u) backoff <<= 1;
-      if (!have) {
-        const double xh = ld_gpu(&x[c]);
-        if (!pend_f(xh)) {
-          prod = __dmul_rn(f, xh);
-          have = true;
-        }
-      }
-    }
-  }
-  if ((unsigned long long)__double_as_longlong(s) == kPendingF)
-    s = __longlong_as_double((long long)0x7FF8000000000000ll);
-  if (lane == 0) asm volatile("st.relaxed.gpu.global.f64 [%0], %1;" ::"l"(x + row), "d"(s) : "memory");
-  return true;
 }
 
 __device__ void numeric_arena_rows(int64_t n, const int64_t *__restrict__ arp,
@@ -799,7 +803,7 @@ static int numeric_cap(const iluk_sym *S, size_t static_smem, bool wide, int *wa
 
 static cudaError_t launch_numeric_impl(const iluk_sym *S, int64_t nbatch, const double *avals,
                                        double *fvals, DivPrep *rdiag, unsigned long long *ticket,
-                                       DevErr *errs, int32_t *depth, unsigned *maxdepth,
+                                       DevErr *errs, const double *v0, double *xf,
                                        cudaStream_t s) {
   // the forward level order, once built, is a valid and better-spread order
   const int32_t *order = S->levels_built ? S->lord.corder : nullptr;
@@ -841,8 +845,8 @@ static cudaError_t launch_numeric_impl(const iluk_sym *S, int64_t nbatch, const 
   }
   kern<<<(unsigned)grid, warps * 32, smem, s>>>(
       S->n, nbatch, S->arowptr, S->a2f, avals, S->nnzA, S->rowptr, S->colind, S->diag, S->pinfo,
-      fvals, S->nnz, order, ticket, errs, cap, map_cap, wait_limit(), hold_row(), rdiag, depth,
-      maxdepth);
+      fvals, S->nnz, order, ticket, errs, cap, map_cap, wait_limit(), hold_row(), rdiag, v0,
+      xf);
   note_launch();
   return cudaGetLastError();
 }
@@ -903,9 +907,9 @@ cudaError_t launch_factor_fused(int64_t n, int64_t nnz_a, const int64_t *arp,
 }
 
 cudaError_t launch_numeric(const iluk_sym *S, const double *aval, double *fval, DivPrep *rdiag,
-                           unsigned long long *ticket, DevErr *err, int32_t *depth,
-                           unsigned *maxdepth, cudaStream_t s) {
-  return launch_numeric_impl(S, 1, aval, fval, rdiag, ticket, err, depth, maxdepth, s);
+                           unsigned long long *ticket, DevErr *err, const double *v0, double *xf,
+                           cudaStream_t s) {
+  return launch_numeric_impl(S, 1, aval, fval, rdiag, ticket, err, v0, xf, s);
 }
 
 cudaError_t launch_numeric_batched(const iluk_sym *S, int64_t nbatch, const double *avals,
