@@ -112,7 +112,7 @@ typedef struct iiluk iiluk;        /* TPIILU incomplete inverses              */
 enum { ILUK_PREC_NONE = 0, ILUK_PREC_ILU = 1, ILUK_PREC_IILU = 2 };
 /* Sweep schedules (all give bit-identical results): rows of a level in
  * lockstep warps over all SMs (FLAGS), on one SM (SINGLE_CTA) or on a small
- * thread-block cluster (CLUSTER; both for sweeps whose rows hold at most 16
+ * thread-block cluster (CLUSTER; both for sweeps whose rows hold at most 8
  * entries, longer rows run as WARP_GRID); one warp per row over all SMs
  * (WARP_GRID) or on one cluster (WARP_CLUSTER).  AUTO times them and keeps the fastest;
  * the pick is remembered by the symbolic handle, and later factorizations of

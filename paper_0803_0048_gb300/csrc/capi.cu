@@ -1001,6 +1001,40 @@ static const SweepAux *sweep_aux(iluk_fac *F, int sched, cudaStream_t s) {
   return &F->aux;
 }
 
+// The schedule of a one-call solve, from the shape of F's DAG alone: timing
+// the kinds takes several applications each, more than such a solve makes
+// (random band, n = 160,000, k = 2: 710 ms of timing in a 790 ms call; 2D 64^2:
+// 8 of 18 ms).  `e`: entries of L a level, `r`: rows a level.  Where the lines
+// lie (one application, the kinds timed over 37 grids and bands of 576 to
+// 373,248 rows, k = 0..2; the pick is within ~10 % of the best on all):
+//  * rows of at most 8 entries a side (kRingMaxRow), orders built: one SM up
+//    to 320 entries a level (2D 256^2, e = 287: 0.85 ms, four SMs 0.87; 2D
+//    300^2, e = 337: 1.10 / 1.01), four SMs up to 1,000 (3D 30^3 k = 1, e = 957:
+//    0.28 ms, warp-per-row grid 0.34; k = 0, e = 1,043: 0.196 / 0.192);
+//  * longer rows: a warp per row on a cluster up to 850 entries a level (3D
+//    20^3 k = 2, e = 394: 0.30 ms, grid 0.36; 27-point 20^3 k = 1, e = 868: 0.46
+//    / 0.44), with helpers where rows hold 60 entries or more;
+//  * else the warp-per-row grid.
+// Without level orders the depth is unknown, but above n / 64 (see factor_impl):
+// narrow.
+static int shape_schedule(const iluk_sym *S) {
+  if (S->n == 0) return ILUK_SCHED_WARP_GRID;
+  const double rows = (double)S->nnz / (double)S->n;
+  const int wc = rows >= 60.0 ? ILUK_SCHED_WARP_CLUSTER_HELP : ILUK_SCHED_WARP_CLUSTER;
+  auto pair = [](int f, int b) { return f | (b << 8); };
+  if (!S->levels_built)
+    return pair(ILUK_SCHED_WIDTH(wc, 512), ILUK_SCHED_WIDTH(wc, 384));
+  const double depth = std::max(S->depth_lower, 1);
+  const double e = ((double)S->nnz - (double)S->n) / 2.0 / depth, r = (double)S->n / depth;
+  if (S->max_row <= kRingMaxRow && e <= 1000.0)
+    return e <= 320.0 ? ILUK_SCHED_SINGLE_CTA : ILUK_SCHED_CLUSTER;
+  if (e <= 850.0) {
+    const int w = r >= 20.0 ? 512 : 384;
+    return ILUK_SCHED_WIDTH(wc, w);
+  }
+  return ILUK_SCHED_WIDTH(ILUK_SCHED_WARP_GRID, e < 2000.0 ? 256 : 512);
+}
+
 // Autotuner: time every sweep schedule (the warp-per-row ones at several CTA
 // widths) on this factorization, forward and backward sweeps separately, and
 // keep the fastest of each (packed as forward | backward << 8); the sweeps of
@@ -1041,21 +1075,23 @@ static int pick_schedule(iluk_fac *F, cudaStream_t s, bool transpose = false) {
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
   cudaEventCreate(&e2);
-  // the warp-per-row kinds at several CTA widths: fewer warps keep fewer
-  // rows in flight (less polling), more warps start each row earlier
-  const int candidates[] = {ILUK_SCHED_FLAGS,
-                            ILUK_SCHED_SINGLE_CTA,
-                            ILUK_SCHED_CLUSTER,
-                            ILUK_SCHED_WARP_GRID,
-                            ILUK_SCHED_WIDTH(ILUK_SCHED_WARP_GRID, 512),
-                            ILUK_SCHED_WIDTH(ILUK_SCHED_WARP_GRID, 256),
-                            ILUK_SCHED_WARP_CLUSTER,
-                            ILUK_SCHED_WIDTH(ILUK_SCHED_WARP_CLUSTER, 768),
-                            ILUK_SCHED_WIDTH(ILUK_SCHED_WARP_CLUSTER, 512),
-                            ILUK_SCHED_WIDTH(ILUK_SCHED_WARP_CLUSTER, 384),
-                            ILUK_SCHED_WIDTH(ILUK_SCHED_WARP_CLUSTER, 256),
-                            ILUK_SCHED_WIDTH(ILUK_SCHED_WARP_CLUSTER_HELP, 512),
-                            ILUK_SCHED_WIDTH(ILUK_SCHED_WARP_CLUSTER_HELP, 384)};
+  // The warp-per-row kinds at several CTA widths: fewer warps keep fewer rows
+  // in flight (less polling), more warps start each row earlier.  Where the
+  // orders tell a wide DAG (over 2,500 entries of L a level), the kinds that
+  // keep to a few SMs are left out: there they take 2 to 20 times the grid's
+  // time, most of all in these trials.
+  const bool wide = S->levels_built && S->nnz / 2 > 2500 * (int64_t)S->depth_lower;
+  std::vector<int> candidates = {ILUK_SCHED_FLAGS, ILUK_SCHED_WARP_GRID,
+                                 ILUK_SCHED_WIDTH(ILUK_SCHED_WARP_GRID, 512),
+                                 ILUK_SCHED_WIDTH(ILUK_SCHED_WARP_GRID, 256)};
+  if (!wide)
+    for (int c : {(int)ILUK_SCHED_SINGLE_CTA, (int)ILUK_SCHED_CLUSTER,
+                  ILUK_SCHED_WIDTH(ILUK_SCHED_WARP_CLUSTER, 768),
+                  ILUK_SCHED_WIDTH(ILUK_SCHED_WARP_CLUSTER, 512),
+                  ILUK_SCHED_WIDTH(ILUK_SCHED_WARP_CLUSTER, 384),
+                  ILUK_SCHED_WIDTH(ILUK_SCHED_WARP_CLUSTER_HELP, 512),
+                  ILUK_SCHED_WIDTH(ILUK_SCHED_WARP_CLUSTER_HELP, 384)})
+      candidates.push_back(c);
   for (int sched : candidates) {
     float mf = 1e30f, mb = 1e30f;
     for (int rep = 0; rep < 3; ++rep) {
@@ -1711,7 +1747,8 @@ static int gmres_impl(const iluk_pattern *A, const double *A_val, int prec_kind,
           if (info) *info = finfo;
           return hst;
         }
-        sched = pick_schedule(F, s);
+        if (F->sched == ILUK_SCHED_AUTO) F->sched = shape_schedule(F->S);
+        sched = F->sched;
         const int ost = orders_for(F, sched, s);
         if (ost != ILUK_OK) return fail(info, ost);
       }

@@ -131,7 +131,7 @@ constexpr int64_t kWideSweepRows = 128;
 constexpr int64_t kSolveSweepRows = 64;
 constexpr int64_t kSolveLevels = 600;
 constexpr int64_t kRingLevels = 8192;
-constexpr int kRingMaxRow = 2 * 16 + 1;
+constexpr int kRingMaxRow = 2 * 8 + 1;
 
 int64_t wait_limit();
 void note_launch();              // counts kernel launches (iluk_launch_count)

@@ -24,7 +24,7 @@
 //    hand-offs); packs the FP64 work of 32 rows into each instruction but
 //    couples the rows of a warp.
 //  * SINGLE_CTA / CLUSTER: the same on one SM or on a small cluster, x handed
-//    over through a ring in shared memory; for rows of at most 16 entries
+//    over through a ring in shared memory; for rows of at most 8 entries
 //    (longer ones run as WARP_GRID).  Suits narrow DAGs of short rows.
 // Rows are taken in level order (padded to warps for the lockstep kernels);
 // every wait is bounded.
@@ -218,7 +218,7 @@ constexpr int kRing = 8192;
 constexpr int kRingNear = kRing - 2048;
 constexpr int kLaneMaxThreads = 256;
 constexpr int kLaneW = 4;        // most entries of a window
-constexpr int kLaneMaxRow = 16;  // and of a row
+constexpr int kLaneMaxRow = 8;   // and of a row
 // the ring, a spare entry of no tag, and spare entries of every thread
 constexpr size_t kRingBytes = (size_t)(kRing + 1 + kLaneMaxThreads * kLaneW) * 16;
 
@@ -288,11 +288,11 @@ constexpr unsigned kRingPolls = 256;
 // ---------------------------------------------------------------------------
 // Lockstep sweep on the ring: a warp takes a chunk, 32 rows of one level, a
 // row per lane, and the lanes advance their chains together, a window of
-// entries at a time (lane_take), so one FP64 warp instruction serves 32 rows.
+// two or four entries at a time (lane_take), so one FP64 warp instruction serves 32 rows.
 // An FP64 warp instruction holds its sub-partition's pipe ~76 cycles however
 // few lanes it serves, so on short rows this is what a level costs: the
 // hand-off, and the products and differences of the entries that arrive last.
-// The rows of a chunk are right-aligned, so those are the last NL of every
+// The rows of a chunk are right-aligned, so those are the last window of every
 // row.  Where an entry's input sits in the walked order comes from the order's
 // plan (LanePlan), its coefficient from F; both are loaded a whole chunk ahead
 // of their use, and the rows they belong to one chunk earlier.  Chunk c belongs
@@ -301,10 +301,10 @@ constexpr unsigned kRingPolls = 256;
 // What bounds it: the latency of that chain, ~590 cycles a level forward.
 // 2D 64^2 grid, k = 2 (253 levels): one application 0.335 ms with a warp per
 // row on a cluster, 0.177 ms here on one SM; 2D 256^2 (1,021 levels) 1.49 ->
-// 0.85 ms; 3D 20^3, k = 1 (115 levels) 0.215 -> 0.150 ms on four SMs.  On
-// 3D 64^3, k = 2 (378 rows a level) it only equals the warp-per-row grid
-// (1.51 and 1.52 ms), and on 27-point grids it loses: their levels are too
-// wide for a few SMs' FP64 pipes.
+// 0.85 ms; 3D 20^3, k = 1 (115 levels) 0.215 -> 0.150 ms on four SMs.  Rows of
+// more than 8 entries ran no faster than a warp per row at any size tried (three
+// early windows: 3D 20^3, k = 2 0.37 / 0.30 ms; 64^3 1.51 / 1.52; 27-point grids
+// lose by 1.1 to 2 times), so they do not take this.
 // Other forms measured slower: windows of up to 16 entries polled together
 // with the ready ones multiplied and subtracted as they came (the longer loop
 // body costs more than it saves, 1.6 ms on 256^2), and levels separated by
@@ -430,30 +430,25 @@ __device__ __forceinline__ bool lane_take(const LaneWin<W> &wn, double &s, unsig
   return true;
 }
 
-// A row's entries sit right-aligned in EN early windows of PW and a last one
-// of NL (a row has at most EN * PW + NL), all loaded a whole chunk ahead of
-// their use.
-template <int PW, int EN, int NL>
+// A row's entries (at most 2 W) sit right-aligned in two windows, both loaded a
+// whole chunk ahead of their use.
+template <int W>
 struct LaneChunk {
   LaneMeta m;
-  LaneWin<PW> win[EN];
-  LaneWin<NL> last;
+  LaneWin<W> early, last;
   double s;
 };
 
-template <bool FORWARD, int PW, int EN, int NL>
-__device__ __forceinline__ void lane_chunk(LaneChunk<PW, EN, NL> &ch,
-                                           const int32_t *__restrict__ pslot,
+template <bool FORWARD, int W>
+__device__ __forceinline__ void lane_chunk(LaneChunk<W> &ch, const int32_t *__restrict__ pslot,
                                            const double *__restrict__ v, const double *in,
                                            int lane) {
-#pragma unroll
-  for (int w = 0; w < EN; ++w)
-    lane_window<FORWARD, PW>(ch.win[w], ch.m, ch.m.w - NL - (EN - w) * PW, pslot, v, lane);
-  lane_window<FORWARD, NL>(ch.last, ch.m, ch.m.w - NL, pslot, v, lane);
+  lane_window<FORWARD, W>(ch.early, ch.m, ch.m.w - 2 * W, pslot, v, lane);
+  lane_window<FORWARD, W>(ch.last, ch.m, ch.m.w - W, pslot, v, lane);
   ch.s = ch.m.row >= 0 ? in[ch.m.row] : 0.0;
 }
 
-template <bool FORWARD, bool DIVIDE, int PW, int EN, int NL>
+template <bool FORWARD, bool DIVIDE, int W>
 __global__ void __launch_bounds__(kLaneMaxThreads, 1)
 k_sweep_lane(const int32_t *__restrict__ order, LanePlan pl, const double *__restrict__ v,
              const DivPrep *__restrict__ rd, const double *in, double *out, double *clear,
@@ -466,25 +461,22 @@ k_sweep_lane(const int32_t *__restrict__ order, LanePlan pl, const double *__res
   const unsigned own = rc.base + (unsigned)(kRing + 1 + threadIdx.x * kLaneW) * 16u;
   const int64_t step = (int64_t)rc.C * (blockDim.x >> 5);
   int64_t c = (int64_t)rc.rank + (int64_t)rc.C * (threadIdx.x >> 5);
-  LaneChunk<PW, EN, NL> cur, nxt;
+  LaneChunk<W> cur, nxt;
   lane_meta(cur.m, order, pl, c, lane);
   lane_meta(nxt.m, order, pl, c + step, lane);
-  lane_chunk<FORWARD, PW, EN, NL>(cur, pl.slot, v, in, lane);
+  lane_chunk<FORWARD, W>(cur, pl.slot, v, in, lane);
   bool ok = true;
   for (; c < pl.nch; c += step) {
     LaneMeta far;  // the rows of the chunk after the next one
     lane_meta(far, order, pl, c + 2 * step, lane);
-    lane_chunk<FORWARD, PW, EN, NL>(nxt, pl.slot, v, in, lane);
+    lane_chunk<FORWARD, W>(nxt, pl.slot, v, in, lane);
     const int32_t row = cur.m.row;
     DivPrep rr{0ull, 1.0};
     if (DIVIDE && row >= 0) rr = rd[row];
     if (clear && row >= 0) clear[row] = __longlong_as_double((long long)kPending);
     double s = cur.s;
-#pragma unroll
-    for (int w = 0; w < EN; ++w)
-      if (cur.m.w > NL + (EN - 1 - w) * PW && ok)
-        ok = lane_take<PW>(cur.win[w], s, rc.base, own, out, order, err, limit_ns);
-    if (ok) ok = lane_take<NL>(cur.last, s, rc.base, own, out, order, err, limit_ns);
+    if (cur.m.w > W) ok = lane_take<W>(cur.early, s, rc.base, own, out, order, err, limit_ns);
+    if (ok) ok = lane_take<W>(cur.last, s, rc.base, own, out, order, err, limit_ns);
     if (!ok) {
       if (row >= 0) set_err(err, row, ILUK_ETIMEOUT);
       break;
@@ -1135,7 +1127,7 @@ static int cluster_width(int64_t n, K kern, size_t fixed = 0, int widest = 16) {
 // the levels it suits (eight or sixteen measured the same or slower: every
 // result goes to each CTA's ring), or two (0 when neither can be scheduled).
 static int ring_cluster() {
-  return cluster_width((int64_t)0, k_sweep_lane<true, false, 4, 3, 4>, kRingBytes, 4);
+  return cluster_width((int64_t)0, k_sweep_lane<true, false, 4>, kRingBytes, 4);
 }
 
 template <typename K, typename... Args>
@@ -1211,9 +1203,8 @@ static cudaError_t run_sweep(int64_t n, const LevelOrder &lo, const int64_t *rp,
     if (ensure_lane_plan<FORWARD>(lo, n, rp, ci, dg, s)) {
       const bool one = kind == ILUK_SCHED_SINGLE_CTA;
       const int C = one ? 1 : ring_cluster();
-      const auto kern = lo.plan.maxw <= 4   ? k_sweep_lane<FORWARD, DIVIDE, 2, 1, 2>
-                        : lo.plan.maxw <= 8 ? k_sweep_lane<FORWARD, DIVIDE, 4, 1, 4>
-                                            : k_sweep_lane<FORWARD, DIVIDE, 4, 3, 4>;
+      const auto kern = lo.plan.maxw <= 4 ? k_sweep_lane<FORWARD, DIVIDE, 2>
+                                          : k_sweep_lane<FORWARD, DIVIDE, 4>;
       return launch_on_cluster(kern, C, one ? kLaneThreads1 : kLaneThreads, kRingBytes, s,
                                (const int32_t *)lo.order, lo.plan, v, rd, in, out, clear, err,
                                limit, C);

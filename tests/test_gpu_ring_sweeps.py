@@ -1,7 +1,7 @@
 """The lockstep sweeps on the shared-memory ring (SINGLE_CTA and CLUSTER)
 against the oracle, bit for bit, at the sizes where they can go wrong: one
 row, one chunk of 32 rows and its edges, rows of exactly the window sizes and
-one beyond (2 + 2, 4 + 4, 16 entries, and longer ones that run warp-per-row),
+one beyond (2 + 2, 4 + 4, and longer ones that run warp-per-row),
 levels wider than the warps, and orders long enough that inputs lie beyond the
 ring or are overwritten in it (more than 8,192 slots back)."""
 import numpy as np
