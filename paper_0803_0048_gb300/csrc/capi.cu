@@ -1647,7 +1647,10 @@ static int gmres_impl(const iluk_pattern *A, const double *A_val, int prec_kind,
   double *V = nullptr, *Z = nullptr, *w = nullptr, *u = nullptr, *Hd = nullptr, *dsc = nullptr,
          *dy = nullptr;
   DotScratch ds{};
+  MgsScratch ms{};
+  unsigned char *xchg = nullptr;
   auto scratch = at_scope_exit([&] {
+    dfree(xchg, s);
     dfree(cursor, s); dfree(scan_tmp, s); dfree(trp, s); dfree(tci, s); dfree(tv, s);
     dfree(V, s); dfree(Z, s); dfree(w, s); dfree(u, s); dfree(Hd, s); dfree(dsc, s);
     dfree(dy, s); dfree(ds.partial, s); dfree(ds.counter, s);
@@ -1679,7 +1682,12 @@ static int gmres_impl(const iluk_pattern *A, const double *A_val, int prec_kind,
   CK(dalloc(&Z, store_z ? (size_t)ldv * m : (size_t)ldv, s));
   CK(dalloc(&w, ldv, s));
   CK(dalloc(&u, ldv, s));
-  CK(dalloc(&Hd, (size_t)(m + 1) * m, s));
+  CK(dalloc(&Hd, (size_t)m + 2, s));  // a column of H, then the orthogonalisation's status
+  CK(dalloc(&xchg, mgs_scratch_bytes(), s));
+  CK(cudaMemsetAsync(xchg, 0, mgs_scratch_bytes(), s));
+  CK(cudaMemsetAsync(Hd, 0, ((size_t)m + 2) * sizeof(double), s));
+  ms.xchg = xchg;
+  ms.fail = reinterpret_cast<int *>(Hd + m + 1);
   CK(dalloc(&dsc, 4, s));
   CK(dalloc(&dy, m, s));
   CK(dalloc(&ds.partial, kDotP, s));
@@ -1695,6 +1703,7 @@ static int gmres_impl(const iluk_pattern *A, const double *A_val, int prec_kind,
     if (st != ILUK_OK) return fail(info, st);
   }
   bool fwd_ready = false;  // F->tmp holds L^-1 v_1 (made by the factorization)
+  bool one_launch = true;  // the Gram-Schmidt steps of an iteration in one launch (mgs.cu)
   // an exit before the backward sweep consumed it leaves F->tmp armed again,
   // as every later application expects
   auto rearm = at_scope_exit([&] {
@@ -1754,10 +1763,10 @@ static int gmres_impl(const iluk_pattern *A, const double *A_val, int prec_kind,
       }
       gv[0] = beta;
       int jend = -1;
-      bool bad = false;
+      bool bad = false, timed_out = false;
       for (int j = 0; j < m; ++j) {
         double *vj = V + (size_t)j * ldv;
-        double *hc = Hd + (size_t)j * (m + 1);  // column j of H
+        double *hc = Hd;  // column j of H
         double *zj = store_z ? Z + (size_t)j * ldv : Z;
         if (fwd_ready) {  // z_1 from the forward sweep the factorization made
           fwd_ready = false;
@@ -1768,17 +1777,31 @@ static int gmres_impl(const iluk_pattern *A, const double *A_val, int prec_kind,
           CK(precond(vj, zj));
         }
         CK(launch_spmv(n, orp, oci, ov, zj, w, nullptr, s));
-        CK(launch_dot(n, w, V, hc + 0, 0, ds, s));
-        for (int i = 0; i <= j; ++i) {
-          const double *vi = V + (size_t)i * ldv;
-          if (i < j)
-            CK(launch_mgs_step(n, w, vi, hc + i, V + (size_t)(i + 1) * ldv, hc + i + 1, 0, ds, s));
-          else
-            CK(launch_mgs_step(n, w, vi, hc + i, w, hc + j + 1, 1, ds, s));
+        const cudaError_t me =
+            one_launch ? launch_mgs(n, w, V, ldv, j, hc, V + (size_t)(j + 1) * ldv, &ms, s)
+                       : cudaErrorInvalidConfiguration;
+        if (me == cudaErrorInvalidConfiguration) {  // the same, one inner product a launch
+          one_launch = false;
+          CK(launch_dot(n, w, V, hc + 0, 0, ds, s));
+          for (int i = 0; i <= j; ++i) {
+            const double *vi = V + (size_t)i * ldv;
+            if (i < j)
+              CK(launch_mgs_step(n, w, vi, hc + i, V + (size_t)(i + 1) * ldv, hc + i + 1, 0, ds,
+                                 s));
+            else
+              CK(launch_mgs_step(n, w, vi, hc + i, w, hc + j + 1, 1, ds, s));
+          }
+          CK(launch_scale_div(n, w, hc + j + 1, V + (size_t)(j + 1) * ldv, s));
+        } else {
+          CK(me);
         }
-        CK(launch_scale_div(n, w, hc + j + 1, V + (size_t)(j + 1) * ldv, s));
-        CK(cudaMemcpyAsync(col.data(), hc, (j + 2) * sizeof(double), cudaMemcpyDeviceToHost, s));
+        CK(cudaMemcpyAsync(col.data(), hc, (m + 2) * sizeof(double), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
+        if (col[m + 1] != 0.0) {
+          status = ILUK_ETIMEOUT;
+          timed_out = true;
+          break;
+        }
         for (int i = 0; i <= j + 1; ++i) H[(size_t)i * m + j] = col[i];
         const double hn = col[j + 1];
         for (int i = 0; i < j; ++i) {  // previous rotations
@@ -1803,6 +1826,7 @@ static int gmres_impl(const iluk_pattern *A, const double *A_val, int prec_kind,
         const bool breakdown = hn == 0.0;
         if (std::fabs(gv[j + 1]) / bnorm <= rtol || iters >= maxit || breakdown) break;
       }
+      if (timed_out) break;
       if (bad) { status = ILUK_EINVAL; break; }
       for (int i = jend; i >= 0; --i) {
         double sacc = gv[i];

@@ -276,6 +276,15 @@ cudaError_t launch_dot(int64_t n, const double *x, const double *y, double *out,
 cudaError_t launch_mgs_step(int64_t n, double *w, const double *vi, const double *hij,
                             const double *vnext, double *out, int take_sqrt,
                             const DotScratch &ds, cudaStream_t s);
+// One Arnoldi step's Gram-Schmidt in one launch (mgs.cu)
+struct MgsScratch {
+  void *xchg = nullptr;  // mgs_scratch_bytes(), zeroed before the first launch
+  int *fail = nullptr;   // device word: a bounded wait ran out
+  unsigned tag = 1;      // next unused tag
+};
+size_t mgs_scratch_bytes();
+cudaError_t launch_mgs(int64_t n, const double *w, const double *V, int64_t ldv, int j, double *hc,
+                       double *vout, MgsScratch *ms, cudaStream_t s);
 cudaError_t launch_scale_div(int64_t n, const double *x, const double *den, double *y,
                              cudaStream_t s);
 cudaError_t launch_combine(int64_t n, const double *V, int64_t ldv, const double *y, int cnt,
