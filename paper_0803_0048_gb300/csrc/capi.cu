@@ -1032,7 +1032,7 @@ static int shape_schedule(const iluk_sym *S) {
     const int w = r >= 20.0 ? 512 : 384;
     return ILUK_SCHED_WIDTH(wc, w);
   }
-  return ILUK_SCHED_WIDTH(ILUK_SCHED_WARP_GRID, e < 2000.0 ? 256 : 512);
+  return ILUK_SCHED_WIDTH(ILUK_SCHED_WARP_GRID, 512);
 }
 
 // Autotuner: time every sweep schedule (the warp-per-row ones at several CTA

@@ -558,9 +558,8 @@ __global__ void k_lane_slots(LanePlan pl, const int32_t *__restrict__ slot_of,
 // then subtracts the longest ready prefix of the chain, in order, and goes
 // back to polling only if the prefix stopped at a still-pending entry.  A row
 // therefore pays, after its last dependency arrives, only for the rest of its
-// own chain.  SCOPE 0: values in global memory, any number of SMs (a
-// co-resident cooperative grid); SCOPE 1: values in the distributed shared
-// memory of one thread-block cluster.
+// own chain.  Below: values in the distributed shared memory of one
+// thread-block cluster; k_sweep_grid: in global memory, over all SMs.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ double ld_dsm(unsigned a) {
   unsigned long long v;
@@ -572,12 +571,6 @@ __device__ __forceinline__ void st_dsm(unsigned a, double x) {
   asm volatile("st.relaxed.cluster.shared::cluster.b64 [%0], %1;" ::"r"(a),
                "l"((unsigned long long)__double_as_longlong(x))
                : "memory");
-}
-
-template <int SCOPE>
-__device__ __forceinline__ double wpr_load(const double *out, unsigned da, int64_t i) {
-  if (SCOPE == 0) return ld_val(&out[i]);
-  return ld_dsm(da);
 }
 
 // Prefix helpers (ILUK_SCHED_WARP_CLUSTER_HELP).  The FP64 pipes of the
@@ -661,7 +654,7 @@ __device__ void sweep_prefixes(const int32_t *__restrict__ order, int64_t len,
   }
 }
 
-template <bool FORWARD, bool DIVIDE, int SCOPE>
+template <bool FORWARD, bool DIVIDE>
 __device__ __forceinline__ void
 sweep_wpr_body(const int32_t *__restrict__ order, int64_t len, int64_t n,
                const int64_t *__restrict__ rp, const int32_t *__restrict__ ci,
@@ -670,7 +663,7 @@ sweep_wpr_body(const int32_t *__restrict__ order, int64_t len, int64_t n,
                DevErr *err, int64_t limit_ns, const int32_t *__restrict__ owner, double *pre_s,
                unsigned long long *pre_k, unsigned *aux_words, int64_t lag, int expect_c,
                int expect_grid) {
-  // SCOPE 1: x_i lives in the shared memory of the CTA whose warp computes
+  // x_i lives in the shared memory of the CTA whose warp computes
   // row i, at slot (k * wpc + warp) for the warp's k-th row; owner[i] holds
   // (rank << 26 | slot), so the producer's store stays on its own SM and only
   // the dependants' polls cross SMs.  With prefix helpers (pre_s non-null) the
@@ -679,28 +672,22 @@ sweep_wpr_body(const int32_t *__restrict__ order, int64_t len, int64_t n,
   extern __shared__ __align__(16) double xs[];
   unsigned rank = 0, C = 1, base = 0;
   const int wpc = blockDim.x >> 5;  // warps per CTA
-  const bool help = SCOPE == 1 && pre_s != nullptr;
+  const bool help = pre_s != nullptr;
   const unsigned epoch = help ? *((volatile unsigned *)aux_words) : 0u;
-  int64_t slice = 0;
-  if (SCOPE == 1) {
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
-    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(C));
-    const int64_t nwc = (int64_t)C * wpc;
-    slice = (len + nwc - 1) / nwc * wpc;
-    if (!cluster_launch_ok(C, expect_c, expect_grid, (uint64_t)slice * sizeof(double), err))
-      return;
-    for (int64_t j = threadIdx.x; j < slice; j += blockDim.x)
-      xs[j] = __longlong_as_double((long long)kPending);
-    base = (unsigned)__cvta_generic_to_shared(xs);
-    cluster_sync_all();
-  }
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(C));
+  const int64_t nw = (int64_t)C * wpc;
+  const int64_t slice = (len + nw - 1) / nw * wpc;
+  if (!cluster_launch_ok(C, expect_c, expect_grid, (uint64_t)slice * sizeof(double), err)) return;
+  for (int64_t j = threadIdx.x; j < slice; j += blockDim.x)
+    xs[j] = __longlong_as_double((long long)kPending);
+  base = (unsigned)__cvta_generic_to_shared(xs);
+  cluster_sync_all();
   const int lane = threadIdx.x & 31;
-  const int64_t gw = SCOPE == 1 ? (int64_t)rank * wpc + (threadIdx.x >> 5)
-                                : ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t nw = SCOPE == 1 ? (int64_t)C * wpc : ((int64_t)gridDim.x * blockDim.x) >> 5;
-  unsigned own_slot = 0;  // SCOPE 1: the slot of this warp's current row
+  const int64_t gw = (int64_t)rank * wpc + (threadIdx.x >> 5);
+  unsigned own_slot = 0;  // the slot of this warp's current row
   unsigned own_base = 0;
-  if (SCOPE == 1) asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(own_base) : "r"(base), "r"(rank));
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(own_base) : "r"(base), "r"(rank));
   bool ok = true;
   if (help && blockIdx.x >= C) {  // a helper CTA: no rows of its own
     const int hw = (int)(blockDim.x >> 5);
@@ -732,7 +719,7 @@ sweep_wpr_body(const int32_t *__restrict__ order, int64_t len, int64_t n,
       }
     }
     // where x_row goes: this CTA's slot for the warp's current row
-    const unsigned sa = SCOPE == 1 ? own_base + ((own_slot + (threadIdx.x >> 5)) << 3) : 0u;
+    const unsigned sa = own_base + ((own_slot + (threadIdx.x >> 5)) << 3);
     if (clear && lane == 0) clear[row] = __longlong_as_double((long long)kPending);
     bool stored = false;  // the last-entry path below stored x_row already
     for (int b = k0; b < mylen && ok; b += 32) {
@@ -747,13 +734,11 @@ sweep_wpr_body(const int32_t *__restrict__ order, int64_t len, int64_t n,
       if (act) {
         c = ci[first + step * e];
         f = v[first + step * e];
-        if (SCOPE == 1) {
-          const unsigned oc = (unsigned)owner[c];
-          unsigned a;
-          asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(base), "r"(oc >> 26));
-          da = a + ((oc & ((1u << 26) - 1u)) << 3);
-        }
-        x = wpr_load<SCOPE>(out, da, c);
+        const unsigned oc = (unsigned)owner[c];
+        unsigned a;
+        asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(base), "r"(oc >> 26));
+        da = a + ((oc & ((1u << 26) - 1u)) << 3);
+        x = ld_dsm(da);
         if (!pending(x)) {
           prod = __dmul_rn(f, x);
           have = true;
@@ -761,7 +746,6 @@ sweep_wpr_body(const int32_t *__restrict__ order, int64_t len, int64_t n,
       }
       int done = 0;
       const uint64_t t0 = globaltimer_ns();
-      unsigned backoff = 8;
       for (unsigned it = 0;; ++it) {
         const unsigned ready = __ballot_sync(FULL_MASK, have);
         const unsigned rest = ~(ready >> done);  // first not-ready lane at or after `done`
@@ -779,7 +763,7 @@ sweep_wpr_body(const int32_t *__restrict__ order, int64_t len, int64_t n,
           bool gave_up = false;
           if (lane == done) {
             for (unsigned jt = 0; !have; ++jt) {
-              x = wpr_load<SCOPE>(out, da, c);
+              x = ld_dsm(da);
               if (!pending(x)) {
                 prod = __dmul_rn(f, x);
                 have = true;
@@ -787,9 +771,6 @@ sweep_wpr_body(const int32_t *__restrict__ order, int64_t len, int64_t n,
                          (any_failed(err) || (int64_t)(globaltimer_ns() - t0) > limit_ns)) {
                 gave_up = true;
                 break;
-              } else if (SCOPE == 0) {
-                __nanosleep(backoff);
-                if (backoff < 128u) backoff <<= 1;
               }
             }
             if (!gave_up) {
@@ -797,12 +778,8 @@ sweep_wpr_body(const int32_t *__restrict__ order, int64_t len, int64_t n,
               if (DIVIDE) r = div_fin(r, rr);
               if ((unsigned long long)__double_as_longlong(r) == kPending)
                 r = __longlong_as_double((long long)kQuietNaN);
-              if (SCOPE == 0) {
-                st_val(&out[row], r);
-              } else {
-                st_dsm(sa, r);
-                if (help) st_val(&out[row], r);  // the helpers' copy
-              }
+              st_dsm(sa, r);
+              if (help) st_val(&out[row], r);  // the helpers' copy
             }
           }
           ok = __shfl_sync(FULL_MASK, gave_up ? 0 : 1, done) != 0;
@@ -815,14 +792,9 @@ sweep_wpr_body(const int32_t *__restrict__ order, int64_t len, int64_t n,
           ok = false;
           break;
         }
-        // grid: back off (L2 polls compete with the stores they wait for);
-        // cluster: spin, a DSMEM poll is cheap and sleeping measured slower
-        if (SCOPE == 0) {
-          __nanosleep(backoff);
-          if (backoff < 128u) backoff <<= 1;
-        }
+        // spin: a DSMEM poll is cheap and sleeping measured slower
         if (!have) {
-          x = wpr_load<SCOPE>(out, da, c);
+          x = ld_dsm(da);
           if (!pending(x)) {
             prod = __dmul_rn(f, x);
             have = true;
@@ -842,33 +814,27 @@ sweep_wpr_body(const int32_t *__restrict__ order, int64_t len, int64_t n,
     if ((unsigned long long)__double_as_longlong(s) == kPending)
       s = __longlong_as_double((long long)kQuietNaN);
     if (lane == 0) {
-      if (SCOPE == 0) {
-        st_val(&out[row], s);
-      } else {
-        st_dsm(sa, s);
-        if (help) st_val(&out[row], s);  // the helpers' copy
-      }
+      st_dsm(sa, s);
+      if (help) st_val(&out[row], s);  // the helpers' copy
     }
     __syncwarp();
   }
-  if (SCOPE == 1) {
-    cluster_sync_all();
-    if (!help)  // with helpers every row already wrote its x to out
-      for (int64_t j = threadIdx.x; j < slice; j += blockDim.x) {
-        const int64_t pos = (j / wpc) * nw + (int64_t)rank * wpc + j % wpc;
-        if (pos < len) out[order[pos]] = xs[j];
-      }
-    if (help) {
-      // the last CTA to finish advances the epoch: every CTA read it at its
-      // start and published its last prefix before arriving here
-      __syncthreads();
-      if (threadIdx.x == 0) {
+  cluster_sync_all();
+  if (!help)  // with helpers every row already wrote its x to out
+    for (int64_t j = threadIdx.x; j < slice; j += blockDim.x) {
+      const int64_t pos = (j / wpc) * nw + (int64_t)rank * wpc + j % wpc;
+      if (pos < len) out[order[pos]] = xs[j];
+    }
+  if (help) {
+    // the last CTA to finish advances the epoch: every CTA read it at its
+    // start and published its last prefix before arriving here
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      __threadfence();
+      if (atomicAdd(&aux_words[1], 1u) == gridDim.x - 1) {
+        aux_words[1] = 0u;
         __threadfence();
-        if (atomicAdd(&aux_words[1], 1u) == gridDim.x - 1) {
-          aux_words[1] = 0u;
-          __threadfence();
-          aux_words[0] = epoch + 1u == 0xffffffffu ? 0u : epoch + 1u;
-        }
+        aux_words[0] = epoch + 1u == 0xffffffffu ? 0u : epoch + 1u;
       }
     }
   }
@@ -885,11 +851,10 @@ sweep_wpr_body(const int32_t *__restrict__ order, int64_t len, int64_t n,
   order, len, n, rp, ci, dg, v, rd, in, out, clear, err, limit_ns, owner, pre_s, pre_k,     \
       aux_words, lag, expect_c, expect_grid
 
-// Warp-per-row sweeps: SCOPE 0 on a grid, SCOPE 1 on one cluster whose width
-// the launch gives.
-template <bool FORWARD, bool DIVIDE, int SCOPE>
+// Warp-per-row sweeps on one cluster whose width the launch gives.
+template <bool FORWARD, bool DIVIDE>
 __global__ void __launch_bounds__(kCtaThreads, 1) k_sweep_wpr(ILUK_WPR_PARAMS) {
-  sweep_wpr_body<FORWARD, DIVIDE, SCOPE>(ILUK_WPR_ARGS);
+  sweep_wpr_body<FORWARD, DIVIDE>(ILUK_WPR_ARGS);
 }
 
 // The helped form: a cooperative launch of two clusters of kHelpCluster CTAs,
@@ -899,10 +864,175 @@ constexpr int kHelpCluster = 16;
 template <bool FORWARD, bool DIVIDE>
 __global__ void __cluster_dims__(kHelpCluster, 1, 1) __launch_bounds__(kCtaThreads, 1)
     k_sweep_wpr_help(ILUK_WPR_PARAMS) {
-  sweep_wpr_body<FORWARD, DIVIDE, 1>(ILUK_WPR_ARGS);
+  sweep_wpr_body<FORWARD, DIVIDE>(ILUK_WPR_ARGS);
 }
 #undef ILUK_WPR_PARAMS
 #undef ILUK_WPR_ARGS
+
+// ---------------------------------------------------------------------------
+// Warp-per-row sweep over all SMs (WARP_GRID), x in global memory.  A row costs
+// four dependent loads before its first look at x (its index, its position, its
+// entries, x), and only a few levels' rows are in flight, so while a warp
+// waits for one row's inputs it loads the next row's: index two rows ahead,
+// position, right-hand side and divisor one row ahead, the entries once those
+// are there.  What bounds it: an L2 hand-off a level (~1,900 cycles a level with
+// the rest of the chain), and on the widest DAGs the FP64 unit, one warp
+// instruction an entry (27-point 90^3).  One application, without the loads
+// ahead -> with them: 3D 64^3 k = 2 1.48 -> 1.35 ms, 72^3 k = 0 0.72 -> 0.50, 27-point
+// 90^3 k = 0 2.22 -> 1.88, 50^3 k = 1 1.39 -> 1.32 ms.  Tried and slower or no
+// faster: a row per lane (32 rows wait for the slowest of their inputs: 64^3
+// 1.75 ms, 90^3 1.90), two rows a warp (64^3 1.48 ms; 90^3 1.69).
+// ---------------------------------------------------------------------------
+constexpr unsigned kGridSleep = 32u;  // longest pause between looks, ns
+
+struct GridRow {
+  int64_t row, first;
+  int len;
+  double s;
+  DivPrep rr;
+};
+
+template <bool FORWARD, bool DIVIDE>
+__device__ __forceinline__ void grid_row(GridRow &g, int64_t row, const int64_t *__restrict__ rp,
+                                         const int64_t *__restrict__ dg,
+                                         const DivPrep *__restrict__ rd, const double *in) {
+  g.row = row;
+  g.first = 0;
+  g.len = 0;
+  g.s = 0.0;
+  g.rr = DivPrep{0ull, 1.0};
+  if (row >= 0) {
+    const int64_t d = dg[row];
+    g.first = FORWARD ? rp[row] : rp[row + 1] - 1;
+    g.len = (int)(FORWARD ? d - g.first : g.first - d);
+    if (DIVIDE) g.rr = rd[row];
+    g.s = in[row];
+  }
+}
+
+template <bool FORWARD, bool DIVIDE>
+__global__ void __launch_bounds__(kCtaThreads, 1)
+k_sweep_grid(const int32_t *__restrict__ order, int64_t len, const int64_t *__restrict__ rp,
+             const int32_t *__restrict__ ci, const int64_t *__restrict__ dg,
+             const double *__restrict__ v, const DivPrep *__restrict__ rd, const double *in,
+             double *out, double *clear, DevErr *err, int64_t limit_ns) {
+  const int lane = threadIdx.x & 31;
+  const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  constexpr int64_t step = FORWARD ? 1 : -1;
+  auto index = [&](int64_t slot) { return slot < len ? (int64_t)order[slot] : (int64_t)-1; };
+  GridRow cur, nxt;
+  grid_row<FORWARD, DIVIDE>(cur, index(gw), rp, dg, rd, in);
+  int64_t r1 = index(gw + nw);
+  int32_t c = 0, cn = 0;
+  double f = 0.0, fn = 0.0;
+  if (lane < cur.len) {
+    c = ci[cur.first + step * lane];
+    f = v[cur.first + step * lane];
+  }
+  for (int64_t slot = gw; slot < len; slot += nw) {
+    const int64_t r2 = index(slot + 2 * nw);
+    grid_row<FORWARD, DIVIDE>(nxt, r1, rp, dg, rd, in);
+    if (clear && lane == 0) clear[cur.row] = __longlong_as_double((long long)kPending);
+    double s = cur.s, res = 0.0;
+    bool fetched = false;  // the next row's entries are on their way
+    auto fetch = [&]() {
+      fetched = true;
+      if (lane < nxt.len) {
+        cn = ci[nxt.first + step * lane];
+        fn = v[nxt.first + step * lane];
+      }
+    };
+    bool ok = true, stored = false;
+    for (int b = 0; b < cur.len && ok; b += 32) {
+      const int e = b + lane;
+      const bool act = e < cur.len;
+      const int cnt = (cur.len - b) < 32 ? cur.len - b : 32;
+      const bool last_batch = b + 32 >= cur.len;
+      if (b > 0 && act) {
+        c = ci[cur.first + step * e];
+        f = v[cur.first + step * e];
+      }
+      double x = 0.0, prod = 0.0;
+      bool have = !act;
+      auto look = [&]() {
+        x = ld_val(&out[c]);
+        if (!pending(x)) {
+          prod = __dmul_rn(f, x);
+          have = true;
+        }
+      };
+      if (act) look();
+      if (!fetched) fetch();
+      int done = 0;
+      const uint64_t t0 = globaltimer_ns();
+      unsigned backoff = 8;
+      for (unsigned it = 0;; ++it) {
+        const unsigned ready = __ballot_sync(FULL_MASK, have);
+        const unsigned rest = ~(ready >> done);  // first not-ready lane at or after `done`
+        const int run = rest == 0u ? 32 - done : __ffs(rest) - 1;
+        const int upto = done + run < cnt ? done + run : cnt;
+        for (int j = done; j < upto; ++j) s = __dsub_rn(s, __shfl_sync(FULL_MASK, prod, j));
+        done = upto;
+        if (done >= cnt) break;
+        if (last_batch && done == cnt - 1) {
+          // only the row's last entry is missing: the lane that owns it
+          // finishes the row alone, with no vote or shuffle in between
+          bool gave_up = false;
+          if (lane == done) {
+            for (unsigned jt = 0; !have; ++jt) {
+              look();
+              if (have) break;
+              if ((jt & 15u) == 15u &&
+                  (any_failed(err) || (int64_t)(globaltimer_ns() - t0) > limit_ns)) {
+                gave_up = true;
+                break;
+              }
+              __nanosleep(backoff);
+              if (backoff < kGridSleep) backoff <<= 1;
+            }
+            if (!gave_up) {
+              res = __dsub_rn(s, prod);
+              if (DIVIDE) res = div_fin(res, cur.rr);
+              if ((unsigned long long)__double_as_longlong(res) == kPending)
+                res = __longlong_as_double((long long)kQuietNaN);
+              st_val(&out[cur.row], res);
+            }
+          }
+          ok = __shfl_sync(FULL_MASK, gave_up ? 0 : 1, done) != 0;
+          stored = ok;
+          break;
+        }
+        const bool stop = (it & 15u) == 15u &&
+                          (any_failed(err) || (int64_t)(globaltimer_ns() - t0) > limit_ns);
+        if (__any_sync(FULL_MASK, stop)) {
+          ok = false;
+          break;
+        }
+        // back off: L2 polls compete with the stores they wait for
+        __nanosleep(backoff);
+        if (backoff < kGridSleep) backoff <<= 1;
+        if (!have) look();
+      }
+    }
+    if (!ok) {
+      if (lane == 0) set_err(err, cur.row, ILUK_ETIMEOUT);
+      return;
+    }
+    if (!fetched) fetch();
+    if (!stored) {
+      if (DIVIDE) s = div_fin(s, cur.rr);
+      if ((unsigned long long)__double_as_longlong(s) == kPending)
+        s = __longlong_as_double((long long)kQuietNaN);
+      if (lane == 0) st_val(&out[cur.row], s);
+    }
+    __syncwarp();
+    cur = nxt;
+    c = cn;
+    f = fn;
+    r1 = r2;
+  }
+}
 
 // owner[order[pos]] = (rank << 26 | slot) for the CTA layout above.
 __global__ void k_owner_codes(const int32_t *__restrict__ order, int64_t len, int C, int wpc,
@@ -1218,7 +1348,7 @@ static cudaError_t run_sweep(int64_t n, const LevelOrder &lo, const int64_t *rp,
     // every warp's next row further ahead and wastes no slot loads
     const int32_t *order = lo.corder;
     const int64_t len = lo.clen;
-    const int C = cluster_width(n, k_sweep_wpr<FORWARD, DIVIDE, 1>);
+    const int C = cluster_width(n, k_sweep_wpr<FORWARD, DIVIDE>);
     if (C == 0) return cudaErrorInvalidConfiguration;
     const int wpc = threads / 32;
     const int64_t nwc = (int64_t)C * wpc;
@@ -1240,7 +1370,7 @@ static cudaError_t run_sweep(int64_t n, const LevelOrder &lo, const int64_t *rp,
       if (e == cudaSuccess) return e;
       cudaGetLastError();  // cannot hold both clusters at once: the plain kind
     }
-    return launch_on_cluster(k_sweep_wpr<FORWARD, DIVIDE, 1>, C, threads, wsmem, s, order, len,
+    return launch_on_cluster(k_sweep_wpr<FORWARD, DIVIDE>, C, threads, wsmem, s, order, len,
                              n, rp, ci, dg, v, rd, in, out, clear, err, limit, owner, no_ps,
                              no_pk, no_words, (int64_t)0, C, C);
   }
@@ -1248,25 +1378,16 @@ static cudaError_t run_sweep(int64_t n, const LevelOrder &lo, const int64_t *rp,
     if (!lo.corder) return cudaErrorInvalidValue;
     const int32_t *order = lo.corder;
     int64_t len = lo.clen;
-    auto kern = k_sweep_wpr<FORWARD, DIVIDE, 0>;
+    auto kern = k_sweep_grid<FORWARD, DIVIDE>;
     int bps = 1;  // an explicit width means one CTA of that width per SM
     if (w == 0) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, kCtaThreads, 0);
     if (bps < 1) bps = 1;
     int64_t grid = (int64_t)bps * num_sms();
     const int64_t want = (len + (threads / 32) - 1) / (threads / 32);
     if (grid > want) grid = want;
-    const int64_t nn = n;
-    const int32_t *no_owner = nullptr;
-    double *no_ps = nullptr;
-    unsigned long long *no_pk = nullptr;
-    unsigned *no_words = nullptr;
-    int64_t no_lag = 0;
-    int no_c = 0;
-    void *args[] = {(void *)&order, (void *)&len, (void *)&nn, (void *)&rp, (void *)&ci,
-                    (void *)&dg, (void *)&v, (void *)&rd, (void *)&in, (void *)&out,
-                    (void *)&clear, (void *)&err, (void *)&limit, (void *)&no_owner,
-                    (void *)&no_ps, (void *)&no_pk, (void *)&no_words, (void *)&no_lag,
-                    (void *)&no_c, (void *)&no_c};
+    void *args[] = {(void *)&order, (void *)&len, (void *)&rp, (void *)&ci, (void *)&dg,
+                    (void *)&v, (void *)&rd, (void *)&in, (void *)&out, (void *)&clear,
+                    (void *)&err, (void *)&limit};
     cudaError_t e = cudaLaunchCooperativeKernel((const void *)kern, dim3((unsigned)grid),
                                                 dim3((unsigned)threads), args, 0, s);
     note_launch();
@@ -1303,7 +1424,7 @@ static int usable_sched(int64_t n, int sc) {
   if (kind < ILUK_SCHED_FLAGS || kind > ILUK_SCHED_WARP_CLUSTER_HELP) kind = ILUK_SCHED_WARP_GRID;
   if (kind == ILUK_SCHED_CLUSTER && ring_cluster() == 0) kind = ILUK_SCHED_WARP_GRID;
   if ((kind == ILUK_SCHED_WARP_CLUSTER || kind == ILUK_SCHED_WARP_CLUSTER_HELP) &&
-      cluster_width(n, k_sweep_wpr<true, false, 1>) == 0)
+      cluster_width(n, k_sweep_wpr<true, false>) == 0)
     kind = ILUK_SCHED_WARP_GRID;
   const bool per_row = kind == ILUK_SCHED_WARP_GRID || kind == ILUK_SCHED_WARP_CLUSTER ||
                        kind == ILUK_SCHED_WARP_CLUSTER_HELP;
