@@ -286,6 +286,10 @@ void iluk_sym_destroy(iluk_sym *S) {
   dfree(S->a2f, s);
   dfree(S->pinfo, s);
   dfree(S->tinfo, s);
+  dfree(S->stage.off, s);
+  dfree(S->stage.src, s);
+  dfree(S->stage.pos, s);
+  dfree(S->stage.first, s);
   level_order_free(S->lord, s);
   level_order_free(S->uord, s);
   level_order_free(S->xlord, s);

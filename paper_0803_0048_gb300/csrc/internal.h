@@ -42,6 +42,17 @@ struct LevelOrder {
 };
 void level_order_free(LevelOrder &lo, cudaStream_t s);
 
+// The numeric phase's updates per row, in pivot order (k_numeric_staged,
+// numeric.cu): row i's are src/pos[off[i] .. off[i + 1]), those of its lower
+// entry p start at first[p].
+struct StagePlan {
+  int state = 0;  // 0 not tried, 1 there, -1 the pattern does not suit it
+  int32_t most = 0;
+  int64_t *off = nullptr;
+  uint32_t *src = nullptr;
+  uint16_t *pos = nullptr, *first = nullptr;
+};
+
 // Handle layouts (opaque in the public header).
 struct iluk_sym {
   int64_t n = 0, nnz = 0, nnzA = 0;
@@ -58,6 +69,7 @@ struct iluk_sym {
   int32_t max_row = 0;
   int32_t depth_lower = -1, depth_upper = -1;
   LevelOrder lord, uord;       // forward / backward sweep level orders
+  StagePlan stage;             // made on first use
   bool levels_built = false;   // lord/uord are built by the first numeric phase
   LevelOrder xlord, xuord;     // index orders (iluk_factor), for the sweeps until lord/uord exist
   // the sweep schedules the autotuner picked for a factorization of this

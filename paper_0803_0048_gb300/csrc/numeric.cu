@@ -19,12 +19,15 @@
 //
 // k_factor_fused runs this phase beside the symbolic one in one launch, each
 // row starting as soon as its pattern is final (see the section below).
+#include <mutex>
+
 #include "internal.h"
 #include "symbolic_body.cuh"
 
 namespace iluk {
 
 constexpr int kNumThreads = 256;
+constexpr int kStagedThreads = 1024;  // k_numeric_staged, at most
 // Static shared memory of the numeric kernels (apply_pivots' per-warp
 // bitmaps), left out of the dynamic shared memory's budget.
 constexpr int kTouchedWords = 16;  // bitmap words per warp: rows of up to 512 entries
@@ -583,6 +586,299 @@ k_numeric(int64_t n, int64_t nbatch, const int64_t *__restrict__ arp,
 }
 
 // ---------------------------------------------------------------------------
+// Rows with an update plan (wide DAGs of short rows: grids).  The plan lists,
+// per row and in pivot order, every update f_ij <- f_ij - f_ih f_hj inside the
+// pattern: where f_hj lies in F and which position of the row it updates.  It
+// depends on the pattern only, is made once with the level orders (StagePlan,
+// two passes in which no row waits), and spares the numeric rows the column
+// reads and searches, most of a row's time.  A row's warp loads the values of
+// all its updates before the first pivot; when a pivot's are missing it looks
+// again at those of the next kStageAhead pivots together, so pivots that become
+// final at about the same time cost one round trip to L2, not one each.  Each
+// entry sees its updates in the same order as above.
+// What bounds it: per level one hand-off through L2, then multiplier (div_fin)
+// and update of the trailing pivots one after the other (~550 cycles each).
+// Refactorization: 27-point 50^3 k = 1 4.15 -> 2.71 ms, 90^3 k = 0 5.92 -> 3.05, 30^3
+// k = 1 1.43 -> 1.00, 3D 64^3 k = 2 2.70 -> 2.06, 72^3 k = 0 1.27 -> 0.79, 2D 256^2 k = 2
+// 1.68 -> 1.52; making the plan for 64^3 0.35 ms.  On narrower DAGs (below
+// kStageLevelRows) the early publishing above is worth more: random band k = 1,
+// 38 rows a level, 4.41 ms there and 5.61 here.  Tried and slower: the
+// multipliers of all pivots that do not update each other at once (27-point 50^3
+// 3.56 ms: neighbouring pivots mostly do), finding the updates anew in every
+// factorization (3.64 ms).
+// ---------------------------------------------------------------------------
+constexpr int64_t kStageLevelRows = 48;
+constexpr int kStageAhead = 6;
+constexpr int kStageLook = 4;  // updates a lane watches while it waits
+
+// One row's updates: calls add(t, q, from, pos) for the t-th (in order), found
+// by pivot q (row-relative) at F's position `from`, for position pos; then
+// bound(q, first) with the first update of every pivot.  rc: the row's columns
+// in shared memory.  Returns the number of updates.  Warp-uniform.
+template <class Add, class Bound>
+__device__ __forceinline__ int stage_row(const int32_t *__restrict__ fci,
+                                         const int64_t *__restrict__ pinfo, int64_t b0, int m,
+                                         int dp, const int32_t *rc, int lane, Add add,
+                                         Bound bound) {
+  int total = 0;
+  for (int base = 0; base < dp; base += 32) {
+    // the upper parts of 32 pivots as one list of candidates
+    const int q = base + lane;
+    int64_t hd = 0;
+    int len = 0;
+    if (q < dp) {
+      const int64_t pi = pinfo[b0 + q];
+      hd = pi >> kUlenBits;
+      len = (int)(pi & ((1ll << kUlenBits) - 1));
+    }
+    int incl = len;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(FULL_MASK, incl, o);
+      if (lane >= o) incl += y;
+    }
+    const int raw = __shfl_sync(FULL_MASK, incl, 31), excl = incl - len;
+    int mine = total;  // updates before pivot q's first
+    for (int r0 = 0; r0 < raw; r0 += 32) {
+      const int r = r0 + lane;
+      int s = 0;  // the candidate's pivot: the last lane with excl <= r
+#pragma unroll
+      for (int o = 16; o >= 1; o >>= 1) {
+        const int e = __shfl_sync(FULL_MASK, excl, s + o);
+        if (e <= r) s += o;
+      }
+      const int64_t from =
+          __shfl_sync(FULL_MASK, hd, s) + 1 + (r - __shfl_sync(FULL_MASK, excl, s));
+      int ps = -1;
+      if (r < raw) {
+        const int32_t j = fci[from];
+        const int lo = lower_bound_i(rc, base + s + 1, m, j);
+        if (lo < m && rc[lo] == j) ps = lo;
+      }
+      const unsigned hit = __ballot_sync(FULL_MASK, ps >= 0);
+      if (ps >= 0) add(total + __popc(hit & ((1u << lane) - 1u)), from, ps);
+      // every hit among candidates before pivot q's first precedes its updates
+      const int before = excl - r0;
+      if (before > 0) mine += __popc(before >= 32 ? hit : hit & ((1u << before) - 1u));
+      total += __popc(hit);
+    }
+    if (q < dp) bound(q, mine);
+  }
+  return total;
+}
+
+template <bool WRITE>
+__global__ void __launch_bounds__(256)
+k_stage_plan(int64_t n, const int64_t *__restrict__ frp, const int32_t *__restrict__ fci,
+             const int64_t *__restrict__ fdiag, const int64_t *__restrict__ pinfo, int cap,
+             int32_t *cnt, int32_t *most, const int64_t *__restrict__ off, uint32_t *src,
+             uint16_t *pos, uint16_t *first) {
+  extern __shared__ int32_t rcs[];
+  const int lane = threadIdx.x & 31;
+  int32_t *rc = rcs + (size_t)(threadIdx.x >> 5) * cap;
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  int mx = 0;
+  for (int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; row < n; row += nw) {
+    const int64_t b0 = frp[row];
+    const int m = (int)(frp[row + 1] - b0), dp = (int)(fdiag[row] - b0);
+    for (int q = lane; q < m; q += 32) rc[q] = fci[b0 + q];
+    __syncwarp();
+    if (WRITE) {
+      const int64_t o = off[row];
+      stage_row(fci, pinfo, b0, m, dp, rc, lane,
+                [&](int t, int64_t from, int ps) {
+                  src[o + t] = (uint32_t)from;
+                  pos[o + t] = (uint16_t)ps;
+                },
+                [&](int q, int f) { first[b0 + q] = (uint16_t)f; });
+    } else {
+      const int t = stage_row(fci, pinfo, b0, m, dp, rc, lane, [](int, int64_t, int) {},
+                              [](int, int) {});
+      if (lane == 0) cnt[row] = t;
+      if (t > mx) mx = t;
+    }
+    __syncwarp();
+  }
+  if (!WRITE && lane == 0 && mx > 0) atomicMax(most, mx);
+}
+
+struct StagedRow {
+  double *rv, *sv, *ppiv;
+  unsigned long long *px;
+  uint32_t *src, *phd;
+  int32_t *rc, *moff;
+  uint16_t *pos;
+};
+
+// Shared memory of one warp: a row of `cap` entries with `tcap` updates.
+__host__ __device__ constexpr size_t staged_bytes(int cap, int tcap) {
+  return (size_t)cap * (8 + 8 + 8 + 4 + 4 + 4) + 16 + (size_t)tcap * (8 + 4 + 2);
+}
+
+__global__ void __launch_bounds__(kStagedThreads, 1)
+k_numeric_staged(int64_t n, const int64_t *__restrict__ arp, const int32_t *__restrict__ a2f,
+                 const double *__restrict__ aval, const int64_t *__restrict__ frp,
+                 const int32_t *__restrict__ fci, const int64_t *__restrict__ fdiag,
+                 const int64_t *__restrict__ pinfo, const int64_t *__restrict__ soff,
+                 const uint32_t *__restrict__ ssrc, const uint16_t *__restrict__ spos,
+                 const uint16_t *__restrict__ sfirst, double *fv,
+                 const int32_t *__restrict__ order, unsigned long long *ticket, DevErr *err,
+                 int cap, int tcap, int64_t limit_ns, int64_t hold, DivPrep *rdiag,
+                 const double *v0, double *xf) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  StagedRow w;
+  {
+    unsigned char *p = smem + (size_t)wib * staged_bytes(cap, tcap);
+    w.rv = reinterpret_cast<double *>(p);
+    w.ppiv = w.rv + cap;
+    w.px = reinterpret_cast<unsigned long long *>(w.ppiv + cap);
+    w.sv = reinterpret_cast<double *>(w.px + cap);
+    w.src = reinterpret_cast<uint32_t *>(w.sv + tcap);
+    w.phd = w.src + tcap;
+    w.rc = reinterpret_cast<int32_t *>(w.phd + cap);
+    w.moff = w.rc + cap;  // cap + 4
+    w.pos = reinterpret_cast<uint16_t *>(w.moff + cap + 4);
+  }
+  for (;;) {
+    unsigned long long tk = 0;
+    if (lane == 0) tk = atomicAdd(ticket, 1ull);
+    const int64_t slot = (int64_t)__shfl_sync(FULL_MASK, tk, 0);
+    if (slot >= n) return;
+    const int64_t row = order ? (int64_t)order[slot] : slot;
+    if (earlier_failed(err, row)) continue;
+    const int64_t b0 = frp[row], o = soff[row];
+    const int m = (int)(frp[row + 1] - b0), total = (int)(soff[row + 1] - o);
+    const int dp = (int)(fdiag[row] - b0);
+    for (int q = lane; q < m; q += 32) w.rv[q] = 0.0;
+    auto look_pivot = [&](int q) {  // f_hh and its published reciprocal
+      w.ppiv[q] = ld_gpu(&fv[w.phd[q]]);
+      unsigned long long x = ~0ull;
+      if (rdiag)
+        asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(x) : "l"(&rdiag[w.rc[q]].x));
+      w.px[q] = x;
+    };
+    for (int q = lane; q < dp; q += 32) {
+      w.rc[q] = fci[b0 + q];
+      w.phd[q] = (uint32_t)(pinfo[b0 + q] >> kUlenBits);
+      w.moff[q] = sfirst[b0 + q];
+      look_pivot(q);
+    }
+    if (lane == 0) w.moff[dp] = total;
+    for (int t = lane; t < total; t += 32) {
+      const uint32_t s = ssrc[o + t];
+      w.src[t] = s;
+      w.pos[t] = spos[o + t];
+      w.sv[t] = ld_gpu(&fv[s]);  // a first look at everything
+    }
+    __syncwarp();
+    bool bad = false;
+    for (int64_t p = arp[row] + lane; p < arp[row + 1]; p += 32) {
+      const double a = aval[p];
+      if (!isfinite(a)) bad = true;
+      w.rv[a2f[p]] = a;
+    }
+    if (__any_sync(FULL_MASK, bad)) {
+      if (lane == 0) set_err(err, row, ILUK_ENONFINITE);
+      continue;
+    }
+    __syncwarp();
+    bool ok = true;
+    for (int q = 0; q < dp && ok; ++q) {
+      const int e0 = w.moff[q], e1 = w.moff[q + 1];
+      double piv = w.ppiv[q];
+      unsigned long long xr = w.px[q];
+      auto missing = [&]() {
+        bool p = pend_f(piv);
+        for (int t = e0 + lane; t < e1; t += 32) p = p || pend_f(w.sv[t]);
+        return p;
+      };
+      if (__any_sync(FULL_MASK, missing())) {
+        // this pivot's values, and up to 96 more updates of the pivots after it
+        // (their diagonals too), looked at together from registers
+        const int qe = q + kStageAhead < dp ? q + kStageAhead : dp, te = w.moff[qe];
+        const int qa = q + 1 + lane;  // the following pivot this lane watches
+        double val[kStageLook], pa = 0.0;
+        uint32_t src[kStageLook];
+#pragma unroll
+        for (int u = 0; u < kStageLook; ++u) {
+          const int t = e0 + lane + 32 * u;
+          val[u] = t < te ? w.sv[t] : 0.0;
+          src[u] = t < te ? w.src[t] : 0u;
+        }
+        if (qa < qe) pa = w.ppiv[qa];
+        const uint32_t pd = w.phd[q], pad = qa < qe ? w.phd[qa] : 0u;
+        const DivPrep *rx = rdiag ? &rdiag[w.rc[q]] : nullptr;
+        const uint64_t tw = globaltimer_ns();
+        for (unsigned it = 0;; ++it) {
+#pragma unroll
+          for (int u = 0; u < kStageLook; ++u)
+            if (pend_f(val[u])) val[u] = ld_gpu(&fv[src[u]]);
+          if (pend_f(pa)) pa = ld_gpu(&fv[pad]);
+          if (pend_f(piv)) piv = ld_gpu(&fv[pd]);
+          if (rx && xr == ~0ull)
+            asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(xr) : "l"(&rx->x));
+          bool p = pend_f(piv);
+#pragma unroll
+          for (int u = 0; u < kStageLook; ++u)
+            p = p || (e0 + lane + 32 * u < e1 && pend_f(val[u]));
+          for (int t = e0 + lane + 32 * kStageLook; t < e1; t += 32) {  // longer pivot rows
+            double x = w.sv[t];
+            if (pend_f(x)) w.sv[t] = x = ld_gpu(&fv[w.src[t]]);
+            p = p || pend_f(x);
+          }
+          if (!__any_sync(FULL_MASK, p)) break;
+          const bool stop = (it & 31u) == 31u && (earlier_failed(err, row) ||
+                                                  (int64_t)(globaltimer_ns() - tw) > limit_ns);
+          if (__any_sync(FULL_MASK, stop)) {  // the whole warp gives up together
+            ok = false;
+            break;
+          }
+          if (it >= 8) __nanosleep(it < 16 ? 16 : kPollSleepMax);
+        }
+#pragma unroll
+        for (int u = 0; u < kStageLook; ++u) {
+          const int t = e0 + lane + 32 * u;
+          if (t < te) w.sv[t] = val[u];
+        }
+        if (qa < qe) w.ppiv[qa] = pa;
+        xr = __shfl_sync(FULL_MASK, xr, 0);
+        __syncwarp();
+        if (!ok) break;
+      }
+      // the multiplier f_ih / f_hh, correctly rounded (see apply_pivots)
+      const double fih =
+          xr != ~0ull ? div_fin(w.rv[q], DivPrep{xr, piv}) : div_int(w.rv[q], piv);
+      for (int t = e0 + lane; t < e1; t += 32) {
+        const int ps = w.pos[t];
+        w.rv[ps] = sub_prod(w.rv[ps], fih, w.sv[t]);
+      }
+      __syncwarp();  // every lane has read rv[q] and applied this pivot
+      if (lane == 0) w.rv[q] = fih;
+    }
+    if (!ok) {
+      if (lane == 0 && !earlier_failed(err, row)) set_err(err, row, ILUK_ETIMEOUT);
+      continue;
+    }
+    __syncwarp();
+    if (lane == 0 && w.rv[dp] == 0.0) set_err(err, row, ILUK_EZEROPIVOT);
+    // the diagonal and U part first (what later rows wait for), then the rest
+    if (row != hold) {
+      for (int t = lane; t < m; t += 32) {
+        const int q = t + dp < m ? t + dp : t + dp - m;
+        fv[b0 + q] = w.rv[q];
+      }
+      if (rdiag && lane == 0) publish_recip(&rdiag[row], w.rv[dp]);
+      __syncwarp();
+      if (xf && !forward_entry(row, dp, w.rv, w.rc, v0, xf, err, limit_ns, lane)) {
+        if (lane == 0 && !earlier_failed(err, row)) set_err(err, row, ILUK_ETIMEOUT);
+      }
+    }
+    __syncwarp();
+  }
+}
+
+// ---------------------------------------------------------------------------
 // Symbolic and numeric phases in one launch (k >= 2).  The CTAs below g_sym
 // run the symbolic row walk; the others factor rows as soon as the walk has
 // finished them.  A numeric row waits for its own pattern (the symbolic row
@@ -801,6 +1097,77 @@ static int numeric_cap(const iluk_sym *S, size_t static_smem, bool wide, int *wa
   return -1;  // a row of F exceeds shared memory
 }
 
+// The update plan of a pattern whose level orders are built (see
+// k_numeric_staged), made on first use; false when the pattern does not suit
+// it (long rows, more updates than kStageMax a row, more plan than an eighth of
+// the free memory) or while `s` is being captured.  Synchronous.
+constexpr int kStageMaxRow = 128;  // entries of a row of F
+constexpr int kStageMax = 2048;    // updates of a row
+static std::mutex g_stage_mu;
+static bool ensure_stage_plan(const iluk_sym *Sc, cudaStream_t s) {
+  iluk_sym *S = const_cast<iluk_sym *>(Sc);  // the plan is a cache of the pattern
+  std::lock_guard<std::mutex> lk(g_stage_mu);
+  StagePlan &pl = S->stage;
+  if (pl.state != 0) return pl.state > 0;
+  if (S->n == 0 || S->max_row > kStageMaxRow || S->nnz >= (int64_t)UINT32_MAX) return false;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  cudaStreamIsCapturing(s, &cs);
+  if (cs != cudaStreamCaptureStatusNone) return false;
+  int32_t *cnt = nullptr, *most = nullptr;
+  int64_t *scan_tmp = nullptr;
+  auto leave = [&](int state) {
+    for (void *p : {(void *)cnt, (void *)most, (void *)scan_tmp})
+      if (p) cudaFreeAsync(p, s);
+    if (state < 0) {
+      for (void *p : {(void *)pl.off, (void *)pl.src, (void *)pl.pos, (void *)pl.first})
+        if (p) cudaFreeAsync(p, s);
+      pl = StagePlan();
+      cudaGetLastError();
+    }
+    pl.state = state;
+    return state > 0;
+  };
+  const int64_t n = S->n;
+  const int cap = (S->max_row + 31) & ~31;
+  const size_t smem = (size_t)cap * 8 * sizeof(int32_t);
+  int64_t grid = (n + 7) / 8;
+  if (grid > (int64_t)num_sms() * 32) grid = (int64_t)num_sms() * 32;
+  if (cudaMallocAsync((void **)&cnt, n * sizeof(int32_t), s) != cudaSuccess ||
+      cudaMallocAsync((void **)&most, sizeof(int32_t), s) != cudaSuccess ||
+      cudaMemsetAsync(most, 0, sizeof(int32_t), s) != cudaSuccess ||
+      cudaMallocAsync((void **)&scan_tmp, scan_tmp_elems(n) * sizeof(int64_t), s) != cudaSuccess ||
+      cudaMallocAsync((void **)&pl.off, (n + 1) * sizeof(int64_t), s) != cudaSuccess)
+    return leave(-1);
+  k_stage_plan<false><<<(unsigned)grid, 256, smem, s>>>(n, S->rowptr, S->colind, S->diag, S->pinfo,
+                                                        cap, cnt, most, nullptr, nullptr, nullptr,
+                                                        nullptr);
+  note_launch();
+  int32_t hm = 0;
+  int64_t total = 0;
+  size_t free_b = 0, total_b = 0;
+  if (launch_scan_lengths(n, cnt, pl.off, scan_tmp, s) != cudaSuccess ||
+      cudaMemcpyAsync(&hm, most, sizeof(hm), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+      cudaMemcpyAsync(&total, pl.off + n, sizeof(total), cudaMemcpyDeviceToHost, s) !=
+          cudaSuccess ||
+      cudaStreamSynchronize(s) != cudaSuccess || cudaMemGetInfo(&free_b, &total_b) != cudaSuccess)
+    return leave(-1);
+  if (hm > kStageMax || (size_t)total * 6 + (size_t)S->nnz * 2 > free_b / 8) return leave(-1);
+  if (cudaMallocAsync((void **)&pl.src, (total > 0 ? total : 1) * sizeof(uint32_t), s) !=
+          cudaSuccess ||
+      cudaMallocAsync((void **)&pl.pos, (total > 0 ? total : 1) * sizeof(uint16_t), s) !=
+          cudaSuccess ||
+      cudaMallocAsync((void **)&pl.first, S->nnz * sizeof(uint16_t), s) != cudaSuccess)
+    return leave(-1);
+  k_stage_plan<true><<<(unsigned)grid, 256, smem, s>>>(n, S->rowptr, S->colind, S->diag, S->pinfo,
+                                                       cap, nullptr, nullptr, pl.off, pl.src,
+                                                       pl.pos, pl.first);
+  note_launch();
+  pl.most = hm;
+  // complete before another stream's factorization may find it
+  if (cudaStreamSynchronize(s) != cudaSuccess) return leave(-1);
+  return leave(1);
+}
+
 static cudaError_t launch_numeric_impl(const iluk_sym *S, int64_t nbatch, const double *avals,
                                        double *fvals, DivPrep *rdiag, unsigned long long *ticket,
                                        DevErr *errs, const double *v0, double *xf,
@@ -809,6 +1176,8 @@ static cudaError_t launch_numeric_impl(const iluk_sym *S, int64_t nbatch, const 
   const int32_t *order = S->levels_built ? S->lord.corder : nullptr;
   ProfScope prof_scope(ILUK_PROF_NUMERIC, s);
   const bool wide = order != nullptr && S->n >= kWideLevelRows * (int64_t)S->lord.nlev;
+  const bool staged = nbatch == 1 && order != nullptr &&
+                      S->n >= kStageLevelRows * (int64_t)S->lord.nlev && ensure_stage_plan(S, s);
   // rows publish their entries as soon as final (see apply_pivots) where F's
   // rows are long, or where a level holds few entries of L (fewer than
   // kEarlyLevelEntries: the band matrices at k <= 1 gain 15-35 %), or before
@@ -829,8 +1198,34 @@ static cudaError_t launch_numeric_impl(const iluk_sym *S, int64_t nbatch, const 
     k_fill_pending_f<<<(unsigned)b, 256, 0, s>>>(nv, fvals);
     note_launch();
   }
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
+  cudaError_t e = cudaSuccess;
+  if (rdiag) {  // every row writes its own entry; ~0 marks the ones not written yet
+    e = cudaMemsetAsync(rdiag, 0xff, (size_t)S->n * sizeof(DivPrep), s);
+    if (e != cudaSuccess) return e;
+  }
+  if (staged) {
+    const int scap = (S->max_row + 31) & ~31, tcap = (S->stage.most + 31) & ~31;
+    const size_t per = staged_bytes(scap, tcap);
+    int sw = (int)(((size_t)max_smem_optin() - 1024) / per);
+    // about eight levels' rows in flight, more only poll (2D 256^2, 64 rows a
+    // level: 1.52 ms with 16 warps, 1.73 with 32; 27-point 90^3 4.1 and 3.1 ms)
+    const int64_t rows8 = 8 * S->n / S->lord.nlev;
+    const int sw_max = rows8 > 8 * (int64_t)num_sms() ? kStagedThreads / 32 : 16;
+    if (sw > sw_max) sw = sw_max;
+    e = cudaFuncSetAttribute(k_numeric_staged, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)(per * sw));
+    if (e != cudaSuccess) return e;
+    int64_t grid = num_sms();
+    const int64_t want = (S->n + sw - 1) / sw;
+    if (grid > want) grid = want;
+    k_numeric_staged<<<(unsigned)grid, sw * 32, per * sw, s>>>(
+        S->n, S->arowptr, S->a2f, avals, S->rowptr, S->colind, S->diag, S->pinfo, S->stage.off,
+        S->stage.src, S->stage.pos, S->stage.first, fvals, order, ticket, errs, scap, tcap,
+        wait_limit(), hold_row(), rdiag, v0, xf);
+    note_launch();
+    return cudaGetLastError();
+  }
+  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   int bps = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, warps * 32, smem);
@@ -839,10 +1234,6 @@ static cudaError_t launch_numeric_impl(const iluk_sym *S, int64_t nbatch, const 
   const int64_t want = (S->n * nbatch + warps - 1) / warps;
   if (grid > want) grid = want;
   if (grid < 1) grid = 1;
-  if (rdiag) {  // every row writes its own entry; ~0 marks the ones not written yet
-    e = cudaMemsetAsync(rdiag, 0xff, (size_t)S->n * sizeof(DivPrep), s);
-    if (e != cudaSuccess) return e;
-  }
   kern<<<(unsigned)grid, warps * 32, smem, s>>>(
       S->n, nbatch, S->arowptr, S->a2f, avals, S->nnzA, S->rowptr, S->colind, S->diag, S->pinfo,
       fvals, S->nnz, order, ticket, errs, cap, map_cap, wait_limit(), hold_row(), rdiag, v0,
