@@ -598,9 +598,9 @@ k_numeric(int64_t n, int64_t nbatch, const int64_t *__restrict__ arp,
 // entry sees its updates in the same order as above.
 // What bounds it: per level one hand-off through L2, then multiplier (div_fin)
 // and update of the trailing pivots one after the other (~550 cycles each).
-// Refactorization: 27-point 50^3 k = 1 4.15 -> 2.71 ms, 90^3 k = 0 5.92 -> 3.05, 30^3
-// k = 1 1.43 -> 1.00, 3D 64^3 k = 2 2.70 -> 2.06, 72^3 k = 0 1.27 -> 0.79, 2D 256^2 k = 2
-// 1.68 -> 1.52; making the plan for 64^3 0.35 ms.  On narrower DAGs (below
+// Refactorization: 27-point 50^3 k = 1 4.19 -> 2.82 ms, 90^3 k = 0 5.92 -> 3.05, 30^3
+// k = 1 1.43 -> 0.99, 3D 64^3 k = 2 2.70 -> 2.14, 72^3 k = 0 1.27 -> 0.79, 2D 256^2 k = 2
+// 1.68 -> 1.51; making the plan for 64^3 0.35 ms.  On narrower DAGs (below
 // kStageLevelRows) the early publishing above is worth more: random band k = 1,
 // 38 rows a level, 4.41 ms there and 5.61 here.  Tried and slower: the
 // multipliers of all pivots that do not update each other at once (27-point 50^3
@@ -1210,7 +1210,7 @@ static cudaError_t launch_numeric_impl(const iluk_sym *S, int64_t nbatch, const 
     // about eight levels' rows in flight, more only poll (2D 256^2, 64 rows a
     // level: 1.52 ms with 16 warps, 1.73 with 32; 27-point 90^3 4.1 and 3.1 ms)
     const int64_t rows8 = 8 * S->n / S->lord.nlev;
-    const int sw_max = rows8 > 8 * (int64_t)num_sms() ? kStagedThreads / 32 : 16;
+    const int sw_max = rows8 > 16 * (int64_t)num_sms() ? kStagedThreads / 32 : 16;
     if (sw > sw_max) sw = sw_max;
     e = cudaFuncSetAttribute(k_numeric_staged, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)(per * sw));
