@@ -37,6 +37,8 @@ struct BatchItemDev {
   int32_t nlev_u;
   const double *b;
   double *x;
+  int32_t max_row;  // entries of the longest row of F
+  int32_t lane;     // numeric phase with a row per lane
 };
 
 struct BatchResultDev {
@@ -401,8 +403,8 @@ __device__ bool cta_sweep_spin(const BatchItemDev &it, const double *fv,
   return s_fail == 0;
 }
 
-// Numeric factorization, level by level over the forward level sets; one
-// warp per row, the row in the warp's shared slice, pivots ascending (the IKJ
+// Numeric factorization, level by level over the forward level sets; a row per
+// lane on wide levels of short rows (numeric_rows_lane), else one warp per row, the row in the warp's shared slice, pivots ascending (the IKJ
 // order of Eq. lufactor2).  Under the level schedule every pivot row of a
 // row is final before the row starts, so the warp first stages all of them at
 // once: for each pivot h its diagonal f_hh and the reciprocal published when
@@ -641,6 +643,87 @@ __device__ __forceinline__ bool numeric_rows_half(const BatchItemDev &it, double
   return true;
 }
 
+// A row per lane, 32 rows of a level per warp: an FP64 instruction holds the
+// SM's FP64 unit for a whole warp however few lanes work, and a row of a dozen
+// entries leaves most lanes of a half-warp idle.  Each lane walks its row's
+// pivots in ascending order and merges the pivot row's columns with its own, so
+// every entry sees the updates of the forms below in their order.  The row
+// slices take the inner-product partials' memory, entry-major so that lanes
+// never share a bank, and as many warps work as it holds slices (6 at 13
+// entries a row).  What bounds it: the gathers of the pivot rows, 32 lines each;
+// eight entries ahead instead of four gave 1-2 %.  256 equal systems, 512
+// threads each, factorization and residual only, half-warps -> lanes (rows a
+// level): 3D 32^3 k = 1 (175) 11.6 -> 7.3 ms, k = 0 (349) 6.8 -> 2.6, 20^3 k = 1
+// (70) 3.06 -> 2.79, 2D 200^2 k = 1 (67) 9.6 -> 5.8.  Below kLaneLevelRows a
+// level fills too few lanes: 10^3 k = 0 (36) 0.22 -> 0.23, 2D 64^2 k = 1 (22)
+// 1.03 -> 1.45, 10^3 k = 1 (18) 0.48 -> 0.96.
+constexpr int kLaneAhead = 4;        // pivot-row entries loaded together
+constexpr int kLaneMaxRow = 16;      // longest row a lane takes
+constexpr int kLaneLevelRows = 48;   // rows a level from which lanes take rows
+// 32 rows of a level, one per lane.
+template <int NT>
+__device__ __forceinline__ void numeric_rows_lane(const BatchItemDev &it, double *fv,
+                                                  unsigned long long *rdx, double *rv,
+                                                  int32_t *rc, int64_t row, int *s_bad,
+                                                  long long *s_badrow) {
+  if (row < 0) return;
+  const int64_t b0 = it.frp[row];
+  const int m = (int)(it.frp[row + 1] - b0);
+  const int dp = (int)(it.fdiag[row] - b0);
+  for (int q = 0; q < m; ++q) {
+    rc[q * 32] = it.fci[b0 + q];
+    rv[q * 32] = 0.0;
+  }
+  bool bad = false;
+  for (int64_t p = it.farp[row], pe = it.farp[row + 1]; p < pe; ++p) {
+    const double a = it.aval[p];
+    if (!isfinite(a)) bad = true;
+    rv[it.a2f[p] * 32] = a;
+  }
+  if (bad) numeric_report(s_bad, s_badrow, ILUK_ENONFINITE, row);
+  int64_t hd = 0, he = 0;
+  DivPrep pr{0, 0.0};
+  if (dp > 0) {
+    const int h = rc[0];
+    hd = it.fdiag[h];
+    he = it.frp[h + 1];
+    pr = DivPrep{rdx[h], fv[hd]};
+  }
+  for (int q = 0; q < dp; ++q) {
+    const double fih = div_fin(rv[q * 32], pr);
+    rv[q * 32] = fih;
+    int64_t nhd = 0, nhe = 0;  // the next pivot, loaded meanwhile
+    if (q + 1 < dp) {
+      const int h = rc[(q + 1) * 32];
+      nhd = it.fdiag[h];
+      nhe = it.frp[h + 1];
+      pr = DivPrep{rdx[h], fv[nhd]};
+    }
+    int p = q + 1;
+    for (int64_t r0 = hd + 1; r0 < he; r0 += kLaneAhead) {
+      int32_t jv[kLaneAhead];
+      double uv[kLaneAhead];
+#pragma unroll
+      for (int g = 0; g < kLaneAhead; ++g) {
+        const bool in = r0 + g < he;
+        jv[g] = in ? it.fci[r0 + g] : 0x7fffffff;
+        uv[g] = in ? fv[r0 + g] : 0.0;
+      }
+#pragma unroll
+      for (int g = 0; g < kLaneAhead; ++g) {
+        while (p < m && rc[p * 32] < jv[g]) ++p;
+        if (p < m && rc[p * 32] == jv[g]) rv[p * 32] = sub_prod(rv[p * 32], fih, uv[g]);
+      }
+    }
+    hd = nhd;
+    he = nhe;
+  }
+  for (int q = 0; q < m; ++q) fv[b0 + q] = rv[q * 32];
+  const double d = rv[dp * 32];
+  rdx[row] = div_prep(d).x;
+  if (d == 0.0) numeric_report(s_bad, s_badrow, ILUK_EZEROPIVOT, row);
+}
+
 template <int NT>
 __device__ bool cta_numeric(const BatchItemDev &it, double *fv, unsigned long long *rdx,
                             double *svals, int32_t *scols, double *stage_base, int cap,
@@ -659,9 +742,21 @@ __device__ bool cta_numeric(const BatchItemDev &it, double *fv, unsigned long lo
     s_badrow = 0x7fffffffffffffffLL;
   }
   __syncthreads();
+  // warps that take lane rows: as many as the partials' memory holds row slices
+  const int lw_fit = 8 * kDotP / (it.max_row * 32 * 12);
+  const int lw = lw_fit < kBWarps ? lw_fit : kBWarps;
+  double *lrv = stage_base + (size_t)wid * it.max_row * 32 + lane;
+  int32_t *lrc = reinterpret_cast<int32_t *>(stage_base + (size_t)lw * it.max_row * 32) +
+                 (size_t)wid * it.max_row * 32 + lane;
   for (int l = 0; l < it.nlev_l; ++l) {
     const int64_t lb = it.lstart[l], le = it.lstart[l + 1];
-    if (kPairs) {
+    if (it.lane) {
+      if (wid < lw) {
+        for (int64_t s0 = lb + (int64_t)wid * 32; s0 < le; s0 += (int64_t)lw * 32)
+          numeric_rows_lane<NT>(it, fv, rdx, lrv, lrc,
+                                s0 + lane < le ? it.lord[s0 + lane] : -1, &s_bad, &s_badrow);
+      }
+    } else if (kPairs) {
       for (int64_t sp = lb + 2 * wid; sp < le; sp += 2 * kBWarps) {
         const int64_t rowA = it.lord[sp];
         const int64_t rowB = sp + 1 < le ? it.lord[sp + 1] : -1;
@@ -923,6 +1018,9 @@ void batch_pack_item(void *dst, const iluk_sym *S, const int64_t *arp, const int
   d.nlev_u = S->uord.nlev;
   d.b = b;
   d.x = x;
+  d.max_row = S->max_row > 0 ? S->max_row : 1;
+  d.lane = d.max_row <= kLaneMaxRow &&
+           S->n >= kLaneLevelRows * S->lord.nlev;
   *reinterpret_cast<BatchItemDev *>(dst) = d;
 }
 
