@@ -39,6 +39,8 @@ struct BatchItemDev {
   double *x;
   int32_t max_row;  // entries of the longest row of F
   int32_t lane;     // numeric phase with a row per lane
+  int32_t packed;   // spinning sweeps on the packed copy (SweepPack)
+  int64_t llen, ulen;  // slots of the forward and backward level orders
 };
 
 struct BatchResultDev {
@@ -52,6 +54,7 @@ struct BatchWork {
   // the diagonal the numeric phase publishes (div_prep, one 64-bit word a row)
   double *fval, *V, *w, *z, *u, *tmp;
   int64_t ldv;  // stride between basis vectors
+  unsigned char *pack;  // the packed sweeps of the item in work, or null
 };
 
 // --- in-CTA building blocks -------------------------------------------------
@@ -397,6 +400,173 @@ __device__ bool cta_sweep_spin(const BatchItemDev &it, const double *fv,
       st_cta_f64(&out[cur.row], y);
     }
     cur = nxt;
+  }
+  if (!ok && lane == 0) atomicExch(&s_fail, 1);
+  __syncthreads();
+  return s_fail == 0;
+}
+
+// The spinning sweep on a packed copy of F.  The form above gathers every
+// coefficient, column and divisor from a row of its own, 32 cache lines per load
+// of a warp, some 700 L1 wavefronts per 32 rows; that, not FP64, bounded it.
+// After the numeric phase each 32-slot chunk's rows are therefore written once
+// entry by entry, lanes side by side: the loads of a sweep take one or two
+// wavefronts and only the inputs are gathered.  A warp waits for one input of
+// its rows at a time and applies it before it looks at the next, so only the
+// missing input is polled and the arithmetic runs during the waits.  Chains
+// longer than kPackQ finish from F.  Same order per chain as the form above.
+// 512 threads each, before -> after: 256 systems 2D 64^2 k = 1 24.2 -> 18.0 ms,
+// 160 of 2D 100^2 k = 1 75.5 -> 57.1, 256 of 3D 32^3 k = 0 60.8 -> 50.6, k = 1
+// 45.1 -> 42.1 (there FP64 binds).  It wins on every level width measured, down
+// to 5 rows (2D 20^2 k = 2 2.24 -> 1.87 ms); the line at kPackLevelRows only
+// bounds the copy, whose levels are padded to 32 slots.
+constexpr int kPackLevelRows = 4;
+constexpr int kPackQ = kSpinPf;  // coefficients of a chain in the packed copy
+
+struct SweepPack {
+  double *cv;       // [chunk][q][lane]
+  ulonglong2 *dv;   // [slot] reciprocal word and divisor (backward)
+  int2 *info;       // [slot] row (-1: padding) and chain length
+  int32_t *ci;      // [chunk][q][lane]
+};
+
+__host__ __device__ inline size_t pack_bytes(int64_t len, bool forward) {
+  return (size_t)len * (kPackQ * 12 + 8 + (forward ? 0 : 16));
+}
+
+template <bool FORWARD>
+__device__ __forceinline__ SweepPack sweep_pack(const BatchItemDev &it, unsigned char *base) {
+  const int64_t len = FORWARD ? it.llen : it.ulen;
+  if (!FORWARD) base += pack_bytes(it.llen, true);
+  SweepPack k;
+  k.dv = reinterpret_cast<ulonglong2 *>(base);
+  k.cv = reinterpret_cast<double *>(base + (FORWARD ? 0 : 16 * len));
+  k.info = reinterpret_cast<int2 *>(k.cv + len * kPackQ);
+  k.ci = reinterpret_cast<int32_t *>(k.info + len);
+  return k;
+}
+
+template <int NT, bool FORWARD>
+__device__ void cta_pack(const BatchItemDev &it, const double *fv, const unsigned long long *rdx,
+                         unsigned char *base) {
+  const SweepPack k = sweep_pack<FORWARD>(it, base);
+  const int32_t *order = FORWARD ? it.lord : it.uord;
+  const int64_t len = FORWARD ? it.llen : it.ulen;
+  for (int64_t slot = threadIdx.x; slot < len; slot += NT) {
+    const int row = order[slot];
+    int cnt = 0;
+    int64_t first = 0;
+    if (row >= 0) {
+      const int64_t d = it.fdiag[row];
+      first = FORWARD ? it.frp[row] : it.frp[row + 1] - 1;
+      cnt = (int)(FORWARD ? d - first : first - d);
+      if (!FORWARD)
+        k.dv[slot] = make_ulonglong2(rdx[row], (unsigned long long)__double_as_longlong(fv[d]));
+    }
+    k.info[slot] = make_int2(row, cnt);
+    const int64_t at = (slot >> 5) * (32 * kPackQ) + (slot & 31);
+#pragma unroll
+    for (int q = 0; q < kPackQ; ++q) {
+      if (q < cnt) {
+        const int64_t pq = FORWARD ? first + q : first - q;
+        k.cv[at + 32 * q] = fv[pq];
+        k.ci[at + 32 * q] = it.fci[pq];
+      }
+    }
+  }
+}
+
+template <int NT, bool FORWARD>
+__device__ bool cta_sweep_packed(const BatchItemDev &it, const double *fv, unsigned char *base,
+                                 const double *in, double *out, int64_t limit_ns) {
+  const SweepPack k = sweep_pack<FORWARD>(it, base);
+  const int64_t len = FORWARD ? it.llen : it.ulen;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  __shared__ int s_fail;
+  if (threadIdx.x == 0) s_fail = 0;
+  for (int64_t i = threadIdx.x; i < it.n; i += NT)
+    out[i] = __longlong_as_double((long long)kSpinPending);
+  __syncthreads();
+  bool ok = true;
+  int2 ri = make_int2(-1, 0);
+  double rhs = 0.0;
+  if ((int64_t)wid * 32 < len) {
+    ri = k.info[(int64_t)wid * 32 + lane];
+    if (ri.x >= 0) rhs = in[ri.x];
+  }
+  for (int64_t s0 = (int64_t)wid * 32; s0 < len; s0 += NT) {
+    const int row = ri.x, cnt = ri.y;
+    double sacc = rhs;
+    const int64_t at = s0 * kPackQ + lane;
+    double cv[kPackQ], xv[kPackQ];
+    int32_t ci[kPackQ];
+#pragma unroll
+    for (int q = 0; q < kPackQ; ++q) {
+      cv[q] = 0.0;
+      ci[q] = 0;
+      if (q < cnt) {
+        ci[q] = k.ci[at + 32 * q];
+        cv[q] = k.cv[at + 32 * q];
+      }
+    }
+    ulonglong2 dv = make_ulonglong2(0, 0);
+    if (!FORWARD && row >= 0) dv = k.dv[s0 + lane];
+    ri = make_int2(-1, 0);  // the next chunk's rows
+    if (s0 + NT < len) ri = k.info[s0 + NT + lane];
+#pragma unroll
+    for (int q = 0; q < kPackQ; ++q) xv[q] = q < cnt ? ld_cta_f64(&out[ci[q]]) : 0.0;
+    rhs = ri.x >= 0 ? in[ri.x] : 0.0;
+    const int maxlen = __reduce_max_sync(FULL_MASK, cnt);
+    uint64_t t0 = 0;
+#pragma unroll
+    for (int q = 0; q < kPackQ; ++q) {
+      if (q < maxlen && ok) {
+        for (unsigned t = 0; __any_sync(FULL_MASK, spin_pending(xv[q])); ++t) {
+          if (spin_pending(xv[q])) xv[q] = ld_cta_f64(&out[ci[q]]);
+          if ((t & 31u) == 31u) {
+            const uint64_t now = globaltimer_ns();
+            if (t0 == 0) t0 = now;
+            const bool stop = *((volatile int *)&s_fail) || (int64_t)(now - t0) > limit_ns;
+            if (__any_sync(FULL_MASK, stop)) {  // the whole warp gives up together
+              ok = false;
+              break;
+            }
+          }
+        }
+        if (q < cnt) sacc = __dsub_rn(sacc, __dmul_rn(cv[q], xv[q]));
+      }
+    }
+    for (int q = kPackQ; q < maxlen && ok; ++q) {
+      const bool act = q < cnt;
+      int64_t pq = 0;
+      double x = 0.0;
+      int32_t c = 0;
+      if (act) {
+        pq = FORWARD ? it.frp[row] + q : it.frp[row + 1] - 1 - q;
+        c = it.fci[pq];
+        x = ld_cta_f64(&out[c]);
+      }
+      for (unsigned t = 0; __any_sync(FULL_MASK, spin_pending(x)); ++t) {
+        if (spin_pending(x)) x = ld_cta_f64(&out[c]);
+        if ((t & 31u) == 31u) {
+          const uint64_t now = globaltimer_ns();
+          if (t0 == 0) t0 = now;
+          const bool stop = *((volatile int *)&s_fail) || (int64_t)(now - t0) > limit_ns;
+          if (__any_sync(FULL_MASK, stop)) {
+            ok = false;
+            break;
+          }
+        }
+      }
+      if (act) sacc = __dsub_rn(sacc, __dmul_rn(fv[pq], x));
+    }
+    if (!ok) break;
+    if (row >= 0) {
+      double y = FORWARD ? sacc
+                         : div_fin(sacc, DivPrep{dv.x, __longlong_as_double((long long)dv.y)});
+      if (spin_pending(y)) y = __longlong_as_double(0x7FF8000000000000ll);  // never the marker
+      st_cta_f64(&out[row], y);
+    }
   }
   if (!ok && lane == 0) atomicExch(&s_fail, 1);
   __syncthreads();
@@ -784,7 +954,11 @@ __device__ bool cta_numeric(const BatchItemDev &it, double *fv, unsigned long lo
 
 template <int NT, bool SPIN>
 __device__ bool cta_apply(const BatchItemDev &it, const double *fv, const unsigned long long *rdx,
-                          const double *p, double *tmp, double *y, int64_t limit_ns) {
+                          unsigned char *pack, const double *p, double *tmp, double *y,
+                          int64_t limit_ns) {
+  if (SPIN && pack != nullptr)
+    return cta_sweep_packed<NT, true>(it, fv, pack, p, tmp, limit_ns) &&
+           cta_sweep_packed<NT, false>(it, fv, pack, tmp, y, limit_ns);
   if (SPIN)
     return cta_sweep_spin<NT, true>(it, fv, rdx, p, tmp, limit_ns) &&
            cta_sweep_spin<NT, false>(it, fv, rdx, tmp, y, limit_ns);
@@ -845,6 +1019,12 @@ k_batch_solve(const BatchItemDev *items, int64_t nitems, BatchResultDev *results
     }
     if (!cta_numeric<NT>(it, wk.fval, rdx, svals, scols, sh, cap, res)) continue;
 
+    unsigned char *pack = SPIN && it.packed ? wk.pack : nullptr;
+    if (pack != nullptr) {  // read after the barriers of the next steps
+      cta_pack<NT, true>(it, wk.fval, rdx, pack);
+      cta_pack<NT, false>(it, wk.fval, rdx, pack);
+    }
+
     // GMRES(m): the same steps, in the same order, as gmres_solve.
     const double bnorm = cta_dot<NT>(n, const_cast<double *>(it.b), nullptr, 0.0, false, nullptr,
                                      sh, true);
@@ -867,7 +1047,7 @@ k_batch_solve(const BatchItemDev *items, int64_t nitems, BatchResultDev *results
       for (int j = 0; j < m; ++j) {
         double *vj = wk.V + (size_t)j * wk.ldv;
         double *zj = wk.z + (size_t)j * wk.ldv;
-        if (!cta_apply<NT, SPIN>(it, wk.fval, rdx, vj, wk.tmp, zj, limit_ns)) {
+        if (!cta_apply<NT, SPIN>(it, wk.fval, rdx, pack, vj, wk.tmp, zj, limit_ns)) {
           if (threadIdx.x == 0) s_stop = 3;  // a bounded wait ran out
           __syncthreads();
           break;
@@ -995,6 +1175,12 @@ size_t batch_item_bytes() { return sizeof(BatchItemDev); }
 size_t batch_result_bytes() { return sizeof(BatchResultDev); }
 size_t batch_work_bytes() { return sizeof(BatchWork); }
 
+// Bytes of the packed copy of S (0: its sweeps read F).
+size_t batch_pack_bytes(const iluk_sym *S) {
+  if (S->n < kPackLevelRows * S->lord.nlev || S->n < kPackLevelRows * S->uord.nlev) return 0;
+  return pack_bytes(S->lord.len, true) + pack_bytes(S->uord.len, false);
+}
+
 // Host-side packing of descriptors (layouts are private to this file).
 void batch_pack_item(void *dst, const iluk_sym *S, const int64_t *arp, const int32_t *aci,
                      const double *aval, const double *b, double *x) {
@@ -1021,12 +1207,15 @@ void batch_pack_item(void *dst, const iluk_sym *S, const int64_t *arp, const int
   d.max_row = S->max_row > 0 ? S->max_row : 1;
   d.lane = d.max_row <= kLaneMaxRow &&
            S->n >= kLaneLevelRows * S->lord.nlev;
+  d.llen = S->lord.len;
+  d.ulen = S->uord.len;
+  d.packed = batch_pack_bytes(S) > 0;
   *reinterpret_cast<BatchItemDev *>(dst) = d;
 }
 
 void batch_pack_work(void *dst, double *fval, double *V, double *w, double *z, double *u,
-                     double *tmp, int64_t ldv) {
-  BatchWork d{fval, V, w, z, u, tmp, ldv};
+                     double *tmp, int64_t ldv, unsigned char *pack) {
+  BatchWork d{fval, V, w, z, u, tmp, ldv, pack};
   *reinterpret_cast<BatchWork *>(dst) = d;
 }
 

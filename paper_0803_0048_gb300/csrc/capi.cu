@@ -6,6 +6,7 @@
 // Hessenberg system) is compiled with FMA contraction off, one IEEE rounding
 // per operation, like the kernels.
 #include <algorithm>
+#include <array>
 #include <atomic>
 #include <cmath>
 #include <cstdio>
@@ -1437,6 +1438,7 @@ int iluk_batch_create(const iluk_batch_item *items, int64_t nitems, int restart,
   B->maxit = maxit;
   int64_t maxn = 1, maxf = 1;
   int maxrow = 1;
+  size_t maxpack = 0;
   std::vector<unsigned char> hitems(batch_item_bytes() * (nitems ? nitems : 1));
   for (int64_t i = 0; i < nitems; ++i) {
     const iluk_batch_item &it = items[i];
@@ -1469,6 +1471,7 @@ int iluk_batch_create(const iluk_batch_item *items, int64_t nitems, int restart,
     if (it.S->n > maxn) maxn = it.S->n;
     if (it.S->nnz > maxf) maxf = it.S->nnz;
     if (it.S->max_row > maxrow) maxrow = it.S->max_row;
+    maxpack = std::max(maxpack, batch_pack_bytes(it.S));
   }
   B->cap = (maxrow + 31) & ~31;
   if (batch_smem_bytes(1024, B->cap, restart) + 8 * 1024 > (size_t)max_smem_optin()) {
@@ -1490,6 +1493,8 @@ int iluk_batch_create(const iluk_batch_item *items, int64_t nitems, int restart,
     return ILUK_ENOMEM;
   }
   std::vector<unsigned char> hwork(batch_work_bytes() * B->nwork);
+  std::vector<unsigned char *> packs(B->nwork, nullptr);
+  std::vector<std::array<double *, 6>> slots;
   for (int64_t w = 0; w < B->nwork; ++w) {
     double *fval, *V, *vw, *z, *u, *tmp;
     if (dalloc(&fval, maxf, s) != cudaSuccess || (B->bufs.push_back(fval), false) ||
@@ -1502,7 +1507,23 @@ int iluk_batch_create(const iluk_batch_item *items, int64_t nitems, int restart,
       return ILUK_ENOMEM;
     }
     B->bufs.push_back(tmp);
-    batch_pack_work(hwork.data() + w * batch_work_bytes(), fval, V, vw, z, u, tmp, ldv);
+    slots.push_back({fval, V, vw, z, u, tmp});
+  }
+  // the packed sweeps take what memory is left; a slot without reads F instead
+  for (int64_t w = 0; w < B->nwork; ++w) {
+    unsigned char *pack = nullptr;
+    if (maxpack > 0 && (w == 0 || packs[w - 1])) {
+      if (dalloc(&pack, maxpack, s) == cudaSuccess) {
+        B->bufs.push_back(reinterpret_cast<double *>(pack));
+      } else {
+        pack = nullptr;
+        cudaGetLastError();
+      }
+    }
+    packs[w] = pack;
+    const std::array<double *, 6> &q = slots[w];
+    batch_pack_work(hwork.data() + w * batch_work_bytes(), q[0], q[1], q[2], q[3], q[4], q[5], ldv,
+                    pack);
   }
   CK(cudaMemcpyAsync(B->items, hitems.data(), hitems.size(), cudaMemcpyHostToDevice, s));
   CK(cudaMemcpyAsync(B->work, hwork.data(), hwork.size(), cudaMemcpyHostToDevice, s));

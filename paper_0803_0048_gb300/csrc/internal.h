@@ -322,8 +322,9 @@ size_t batch_smem_bytes(int nt, int cap, int m);
 int batch_max_restart();
 void batch_pack_item(void *dst, const iluk_sym *S, const int64_t *arp, const int32_t *aci,
                      const double *aval, const double *b, double *x);
+size_t batch_pack_bytes(const iluk_sym *S);
 void batch_pack_work(void *dst, double *fval, double *V, double *w, double *z, double *u,
-                     double *tmp, int64_t ldv);
+                     double *tmp, int64_t ldv, unsigned char *pack);
 void batch_unpack_result(const void *src, int32_t *status, int32_t *iters, int32_t *cycles,
                          int64_t *row, double *relres);
 cudaError_t launch_batch_solve(int nt, bool spin, const void *items, int64_t nitems,
