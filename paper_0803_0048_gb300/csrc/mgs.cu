@@ -8,10 +8,14 @@
 // elements p + 4096 r (a row of 32 for each r): they keep their part of w, and of
 // the v_i as it passes, in shared memory for the whole step, so w is read
 // once and each v_i once.  In a CTA the warps of three SM sub-partitions form
-// the updates and products, four rows at a time (one on small systems), while warp 0, alone on its
-// sub-partition's FP64 pipe, adds the products in order (one chain per lane): a
-// product's place holds a signalling NaN, which no product is, until it is
-// there, and again once it is taken.  The tree runs over CTAs instead of
+// the updates and products, a row at a time, while warp 0 adds the products in
+// order (one chain per lane): a product's place holds a signalling NaN, which no
+// product is, until it is there, and again once it is taken.  Against six busy
+// warps a chain of additions still gets one in per 76 cycles, so that warp's own
+// loads, votes and stores must not stand in its way: it takes Q products at a
+// time and fetches the next Q, into registers of their own, and frees the places
+// between the additions, whose latency hides both (before, four at a time ahead of
+// their additions, a row took 118 cycles).  The tree runs over CTAs instead of
 // through one CTA's memory: its strides 64 and 32 (in CTAs) inside a cluster of
 // four, the partials pushed to the cluster's first CTA, its strides 16 .. 1
 // over the 32 clusters' vectors, which travel through L2 and are summed by every
@@ -20,11 +24,13 @@
 // step's tag in both 64-bit words, so they are their own flags and nothing is
 // cleared in between.  (Clusters of eight would not all be resident: 15 fit.)
 // What bounds it: per inner product the four FP64 operations an element on the
-// 128 SMs' pipes, which is also the chain of n / 4096 additions (~76 cycles each),
-// and ~2.5 us of hand-offs and tree, instead of a launch, a counter and one
-// CTA's tree.  Per inner product, launches included: n = 4,096 10.5 -> 3.3 us,
-// 65,536 11.7 -> 4.4, 262,144 14.4 -> 7.2, 729,000 20.5 -> 14.1 us (a third of the
-// warps or twice as many compute warps measured the same).
+// 128 SMs' pipes, which is also the chain of n / 4096 additions (76 cycles each,
+// 90 measured), and ~2.5 us of hand-offs and tree, instead of a launch, a counter
+// and one CTA's tree.  Per inner product, launches included, one launch a step ->
+// four products ahead of their additions -> this: n = 4,096 10.5 -> 2.9 -> 2.95 us,
+// 65,536 11.7 -> 4.2 -> 3.8, 262,144 14.4 -> 7.2 -> 6.2, 729,000 20.5 -> 14.1 -> 11.6
+// (a third of the warps or twice as many compute warps measured the same, and so
+// did two or four rows at a time).
 // All CTAs are resident (cooperative launch); every wait is bounded.
 #include "internal.h"
 
@@ -99,7 +105,7 @@ struct MgsWait {
   }
 };
 
-template <int R>
+template <int Q>
 __global__ void __cluster_dims__(kMgsCluster, 1, 1) __launch_bounds__(kMgsThreads, 1)
 k_mgs(int64_t n, int rows, const double *__restrict__ w, const double *__restrict__ V,
       int64_t ldv, int j, double *hc, double *vout, uint4 *xchg, unsigned tag0, int *fail,
@@ -115,8 +121,7 @@ k_mgs(int64_t n, int rows, const double *__restrict__ w, const double *__restric
     if (threadIdx.x == 0) *fail = 1;
     return;
   }
-  const int nch = (rows + R - 1) / R;
-  const size_t part = (size_t)nch * R * 32;
+  const size_t part = (size_t)rows * 32;
   const int cl = blockIdx.x / kMgsCluster;
   const int64_t p = (int64_t)(cl + kMgsClusters * (int)rank) * 32 + lane;
   double *sw = sm + lane, *sv = sw + part, *sp = sw + 3 * part;  // sv: even, then odd
@@ -158,8 +163,8 @@ k_mgs(int64_t n, int rows, const double *__restrict__ w, const double *__restric
   };
 
   if (cw >= 0) {
-    // this warp's chunks of R rows: cw, cw + kMgsComputeWarps, ...
-    // (rows and elements past the end hold +0.0)
+    // this warp's rows: cw, cw + kMgsComputeWarps, ... (elements past the end
+    // hold +0.0)
     auto fetch = [&](const double *src, double *dst, int r) {
       const int64_t i = p + (int64_t)r * kDotP;
       const unsigned a = (unsigned)__cvta_generic_to_shared(dst + (size_t)r * 32);
@@ -168,15 +173,14 @@ k_mgs(int64_t n, int rows, const double *__restrict__ w, const double *__restric
       else
         dst[(size_t)r * 32] = 0.0;
     };
-    for (int c = cw; c < nch; c += kMgsComputeWarps)
-      for (int r = c * R; r < (c + 1) * R; ++r) {
-        fetch(w, sw, r);
-        fetch(V, sv, r);
-        if (j >= 1) fetch(V + ldv, sv + part, r);
-      }
+    for (int r = cw; r < rows; r += kMgsComputeWarps) {
+      fetch(w, sw, r);
+      fetch(V, sv, r);
+      if (j >= 1) fetch(V + ldv, sv + part, r);
+    }
     bool ok = true;
     const bool sums = rank == 0 && warp <= 3;
-    if (cw < nch || sums) {
+    if (cw < rows || sums) {
       double h = 0.0;
       for (int s = 0; s < ninner; ++s) {
         if (s > 0) ok = wait([&] { return smem_try(&sh.h, tag0 + (unsigned)(s - 1), h); });
@@ -184,37 +188,18 @@ k_mgs(int64_t n, int rows, const double *__restrict__ w, const double *__restric
         asm volatile("cp.async.wait_all;" ::: "memory");
         double *vi = sv + (s & 1 ? 0 : part);                  // v_{s-1}
         const double *vn = s <= j ? sv + (s & 1 ? part : 0) : sw;  // v_s; at last w itself
-        for (int c = cw; c < nch; c += kMgsComputeWarps) {
-          const size_t o = (size_t)c * R * 32;
-          double x[R], y[R];
-#pragma unroll
-          for (int u = 0; u < R; ++u) {
-            x[u] = sw[o + u * 32];
-            y[u] = vi[o + u * 32];
-          }
+        for (int r = cw; r < rows; r += kMgsComputeWarps) {
+          const size_t o = (size_t)r * 32;
+          double x = sw[o];
           if (s > 0) {
-#pragma unroll
-            for (int u = 0; u < R; ++u) y[u] = __dmul_rn(h, y[u]);
-#pragma unroll
-            for (int u = 0; u < R; ++u) {
-              x[u] = __dsub_rn(x[u], y[u]);
-              sw[o + u * 32] = x[u];
-            }
+            x = __dsub_rn(x, __dmul_rn(h, vi[o]));
+            sw[o] = x;
           }
-#pragma unroll
-          for (int u = 0; u < R; ++u) y[u] = vn[o + u * 32];
-#pragma unroll
-          for (int u = 0; u < R; ++u) {
-            y[u] = __dmul_rn(x[u], y[u]);
-            asm volatile("st.volatile.shared.f64 [%0], %1;" ::"r"(
-                             (unsigned)__cvta_generic_to_shared(sp + o + u * 32)),
-                         "d"(y[u]));
-          }
+          asm volatile("st.volatile.shared.f64 [%0], %1;" ::"r"(
+                           (unsigned)__cvta_generic_to_shared(sp + o)),
+                       "d"(__dmul_rn(x, vn[o])));
           // v_{s-1} is done with: v_{s+1} takes its place
-          if (s > 0 && s + 1 <= j)
-#pragma unroll
-            for (int u = 0; u < R; ++u)
-              fetch(V + (int64_t)(s + 1) * ldv, vi, c * R + u);
+          if (s > 0 && s + 1 <= j) fetch(V + (int64_t)(s + 1) * ldv, vi, r);
         }
         if (sums) {
           double x;
@@ -231,63 +216,74 @@ k_mgs(int64_t n, int rows, const double *__restrict__ w, const double *__restric
       if (ok) ok = wait([&] { return smem_try(&sh.h, tag0 + (unsigned)(ninner - 1), h); });
       if (ok && h != 0.0) {  // h = 0: a breakdown, v_{j+1} is not needed
         const DivPrep pd = div_prep(h);
-        for (int c = cw; c < nch; c += kMgsComputeWarps)
-          for (int r = c * R; r < (c + 1) * R; ++r) {
-            const int64_t i = p + (int64_t)r * kDotP;
-            if (i < n) vout[i] = div_fin(sw[(size_t)r * 32], pd);
-          }
+        for (int r = cw; r < rows; r += kMgsComputeWarps) {
+          const int64_t i = p + (int64_t)r * kDotP;
+          if (i < n) vout[i] = div_fin(sw[(size_t)r * 32], pd);
+        }
       }
     }
   } else if (warp == 0) {
     const int lane_rows = p < n ? (int)((n - p + kDotP - 1) / kDotP) : 0;
     const unsigned pa = (unsigned)__cvta_generic_to_shared(sp);
-    auto look = [&](int c, double (&y)[R]) {
-#pragma unroll
-      for (int u = 0; u < R; ++u)
-        asm volatile("ld.volatile.shared.f64 %0, [%1];"
-                     : "=d"(y[u])
-                     : "r"(pa + (unsigned)(c * R + u) * 256u));
+    double sum = 0.0, ya[Q], yb[Q];
+    auto look = [&](double &y, int r) {
+      asm volatile("ld.volatile.shared.f64 %0, [%1];" : "=d"(y) : "r"(pa + (unsigned)r * 256u));
     };
-    auto there = [&](const double (&y)[R]) {
+    auto release = [&](int r) {
+      asm volatile("st.volatile.shared.u64 [%0], %1;" ::"r"(pa + (unsigned)r * 256u),
+                   "l"(kNoProduct));
+    };
+    auto there = [&](const double (&y)[Q], int q) {
       bool all = true;
 #pragma unroll
-      for (int u = 0; u < R; ++u)
-        all = all && (unsigned long long)__double_as_longlong(y[u]) != kNoProduct;
+      for (int u = 0; u < Q; ++u)
+        all = all && (u >= q || (unsigned long long)__double_as_longlong(y[u]) != kNoProduct);
       return all;
+    };
+    auto await = [&](double (&y)[Q], int r, int q) {  // the products of rows r .. r + q - 1
+      return wait([&] {
+#pragma unroll
+        for (int u = 0; u < Q; ++u)
+          if (u < q) look(y[u], r + u);
+        return there(y, q);
+      });
+    };
+    // adds the Q products y of rows r .. and fetches the q after them into z
+    auto group = [&](const double (&y)[Q], double (&z)[Q], int r, int q) {
+#pragma unroll
+      for (int u = 0; u < Q; ++u) {
+        asm volatile("add.rn.f64 %0, %0, %1;" : "+d"(sum) : "d"(y[u]));
+        if (u < q) look(z[u], r + Q + u);
+        release(r + u);
+      }
+      return __all_sync(FULL_MASK, there(z, q)) || await(z, r + Q, q);
+    };
+    // the last q products: a lane may have no element in the last row
+    auto finish = [&](const double (&y)[Q], int r, int q) {
+#pragma unroll
+      for (int u = 0; u < Q; ++u)
+        if (u < q) {
+          if (r + u < lane_rows) sum = __dadd_rn(sum, y[u]);
+          release(r + u);
+        }
     };
     for (int s = 0; s < ninner; ++s) {
       const unsigned tag = tag0 + (unsigned)s;
-      double sum = 0.0, y[R], z[R];
-      bool ok = true;
-      look(0, y);
-      for (int c = 0; c < nch; ++c) {
-        if (!__all_sync(FULL_MASK, there(y)))
-          ok = wait([&] {
-            look(c, y);
-            return there(y);
-          });
-        if (!ok) break;
-        // the next products' loads, and these places free again, before the
-        // additions, whose latency covers them
-        if (c + 1 < nch) look(c + 1, z);
-#pragma unroll
-        for (int u = 0; u < R; ++u)
-          asm volatile("st.volatile.shared.u64 [%0], %1;" ::"r"(
-                           pa + (unsigned)(c * R + u) * 256u),
-                       "l"(kNoProduct));
-        if (c + 1 < nch) {  // then all rows are there
-#pragma unroll
-          for (int u = 0; u < R; ++u) sum = __dadd_rn(sum, y[u]);
-        } else {
-          const int left = lane_rows - c * R;  // this lane's rows from the chunk on
-#pragma unroll
-          for (int u = 0; u < R; ++u)
-            if (u < left) sum = __dadd_rn(sum, y[u]);
-        }
-#pragma unroll
-        for (int u = 0; u < R; ++u) y[u] = z[u];
+      sum = 0.0;
+      auto left = [&](int r) { return rows - r < Q ? rows - r : Q; };
+      bool ok = await(ya, 0, left(0));
+      int r = 0;
+      for (; ok && r + 2 * Q < rows; r += 2 * Q) {
+        ok = group(ya, yb, r, Q) &&
+             group(yb, ya, r + Q, left(r + 2 * Q));
       }
       if (!ok) break;
+      if (r + Q < rows) {
+        if (!group(ya, yb, r, left(r + Q))) break;
+        finish(yb, r + Q, left(r + Q));
+      } else {
+        finish(ya, r, left(r));
+      }
       cluster_put(&sh.slot[rank][lane], 0u, sum, tag);
       if (rank == 0) {
         double a[kMgsCluster];
@@ -333,14 +329,16 @@ k_mgs(int64_t n, int rows, const double *__restrict__ w, const double *__restric
   asm volatile("barrier.cluster.arrive.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
 }
 
-// Rows a compute warp takes at a time: four, whose operations fill each other's
-// latency, or one while that leaves compute warps without rows.
-static int mgs_rows(int64_t rows) { return rows >= 4 * kMgsComputeWarps ? 4 : 1; }
+// Products the adding warp takes at a time: larger groups hide more of its loads
+// and votes, but it starts only when a whole one is there.  Per inner product
+// with groups of 1, 4, 8: 1 row 2.95, 3.05, 3.12 us; 4 rows 3.17, 3.18, 3.23; 16 rows
+// 4.07, 3.77, 3.97; 64 rows 7.73, 6.24, 6.23; 178 rows 16.4, 12.1, 11.6 us.
+static int mgs_group(int rows) { return rows >= 64 ? 8 : rows >= 4 ? 4 : 1; }
 
 // Shared memory for n elements, 0 when a CTA cannot hold its part.
 static size_t mgs_smem(int64_t n, int *rows) {
-  const int64_t r = (n + kDotP - 1) / kDotP, R = mgs_rows(r);
-  const size_t need = (size_t)((r + R - 1) / R) * R * 32 * 4 * sizeof(double);
+  const int64_t r = (n + kDotP - 1) / kDotP;
+  const size_t need = (size_t)r * 32 * 4 * sizeof(double);
   if (r < 1 || need + sizeof(MgsShared) + 1024 > (size_t)max_smem_optin()) return 0;
   *rows = (int)r;
   return need;
@@ -358,7 +356,8 @@ cudaError_t launch_mgs(int64_t n, const double *w, const double *V, int64_t ldv,
   const size_t smem = mgs_smem(n, &rows);
   if (smem == 0 || !ms->xchg) return cudaErrorInvalidConfiguration;
   ProfScope prof_scope(ILUK_PROF_DOT, s);
-  const auto kern = mgs_rows(rows) == 4 ? k_mgs<4> : k_mgs<1>;
+  const int group = mgs_group(rows);
+  const auto kern = group == 8 ? k_mgs<8> : group == 4 ? k_mgs<4> : k_mgs<1>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem);
   if (e != cudaSuccess) return e;
