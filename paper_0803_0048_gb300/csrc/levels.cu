@@ -285,6 +285,9 @@ int build_levels_pair(int64_t n, const int64_t *rp, const int32_t *ci, const int
   }
   int st = order_from_depth(n, depth, nlev[0], fwd, s);
   if (st == ILUK_OK) st = order_from_depth(n, depth + n, nlev[1], bwd, s);
+  // the orders are read on other streams than the one they were built on (beside
+  // a numeric phase; another caller's), which nothing else makes wait
+  if (st == ILUK_OK && cudaStreamSynchronize(s) != cudaSuccess) st = ILUK_ECUDA;
   cleanup();
   return st;
 }
