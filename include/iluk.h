@@ -114,7 +114,8 @@ enum { ILUK_PREC_NONE = 0, ILUK_PREC_ILU = 1, ILUK_PREC_IILU = 2 };
  * lockstep warps over all SMs (FLAGS), on one SM (SINGLE_CTA) or on a small
  * thread-block cluster (CLUSTER; both for sweeps whose rows hold at most 8
  * entries, longer rows run as WARP_GRID); one warp per row over all SMs
- * (WARP_GRID) or on one cluster (WARP_CLUSTER).  AUTO times them and keeps the fastest;
+ * (WARP_GRID) or on one cluster (WARP_CLUSTER).  AUTO times those that suit the
+ * shape of F's DAG and keeps the fastest (iluk_solve picks from the shape alone);
  * the pick is remembered by the symbolic handle, and later factorizations of
  * the same pattern use it without timing again.
  * A schedule byte holds the kind in bits 0-3 and, for the warp-per-row
@@ -167,8 +168,9 @@ int64_t iluk_launch_count(void);
  * those events and fills ms[kind] (total milliseconds) and count[kind]
  * (launches) for kind < nkinds (host arrays).  Enabling clears the records.
  * OVERLAPPED collects the work a call runs on a second stream beside its main
- * kernel (the level orders built during the first numeric phase of a
- * pattern): its time is hidden, not added, so it is kept apart. */
+ * kernel (the level orders of a deep, narrow DAG, built beside the first
+ * numeric phase of a pattern): its time is hidden, not added, so it is kept
+ * apart. */
 enum {
   ILUK_PROF_VALIDATE = 0, ILUK_PROF_SYMBOLIC = 1, ILUK_PROF_COMPACT = 2, ILUK_PROF_DEPTH = 3,
   ILUK_PROF_NUMERIC = 4, ILUK_PROF_SWEEP = 5 /* forward sweeps */, ILUK_PROF_TRANSPOSE = 6, ILUK_PROF_IILU_BUILD = 7,
@@ -201,9 +203,9 @@ int iluk_symbolic(const iluk_pattern *A, int k, iluk_sym **S, iluk_info *info, v
 int iluk_sym_query(const iluk_sym *S, iluk_sym_view *view);
 /* Longest dependency chains of the forward and backward sweeps over F's
  * pattern (the number of rows on the critical path of each sweep).  They come
- * with the sweeps' level orders, which the first iluk_numeric on S builds on a
- * second stream while it factorizes; if none has run yet, this call builds
- * them (synchronous on `stream`).  Cached in S afterwards. */
+ * with the sweeps' level orders, which the first iluk_numeric on S builds before
+ * its rows, or beside them on a deep, narrow DAG; if none has run yet, this call
+ * builds them (synchronous on `stream`).  Cached in S afterwards. */
 int iluk_sym_depth(iluk_sym *S, int32_t *depth_lower, int32_t *depth_upper, void *stream);
 /* Copy S's arrays into caller-owned device buffers (any pointer may be NULL
  * to skip that array).  Asynchronous. */
@@ -225,20 +227,20 @@ int iluk_numeric(const iluk_sym *S, const double *A_val, iluk_fac **F, iluk_info
 /* Re-run the numeric phase into an existing handle with new values. */
 int iluk_refactor(iluk_fac *F, const double *A_val, iluk_info *info, void *stream);
 /*
- * a2 + a3 together: iluk_symbolic(A, k) then iluk_numeric, with the numeric
- * phase running beside the symbolic one (k >= 2: one launch in which each row
- * is factored as soon as its pattern is final, its values kept in an arena
- * laid out like the symbolic one until both phases end).  *S and *F receive
- * handles equal, bit for bit, to those of the two calls, except that the
- * level orders of the sweeps are not built: the sweeps walk rows in index
+ * a2 + a3 together: iluk_symbolic(A, k) then iluk_numeric.  *S and *F receive
+ * handles equal, bit for bit, to those of the two calls, except that the level
+ * orders of the sweeps are built only on wide DAGs, such as 3D grids (n at
+ * least 128 times the forward depth).  On others the sweeps walk rows in index
  * order (ascending forward, descending backward; any order that puts every
  * dependency first gives the same bits) until a later iluk_numeric or
- * iluk_refactor on S, or iluk_sym_depth, builds them (on wide DAGs, such as 3D
- * grids, level orders give much faster sweeps: call iluk_sym_depth first, or
- * the two calls).  For k <= 1 the two phases run one after the other (rows
- * need no other rows' patterns), also without level orders.  Falls back to the
- * two calls for rows of F longer than 512 entries and whenever the combined
- * launch reports an error (the two calls then report it).
+ * iluk_refactor on S, or iluk_sym_depth, builds them.
+ * The phases run one after the other where rows need not wait for one another's
+ * patterns (k <= 1, and k >= 2 on patterns of limited reach).  Else (k >= 2) the
+ * numeric phase runs beside the symbolic one, in one launch in which each row is
+ * factored as soon as its pattern is final, its values kept in an arena laid out
+ * like the symbolic one until both phases end; that launch falls back to the two
+ * calls for rows of F longer than 512 entries and whenever it reports an error
+ * (the two calls then report it).
  * Synchronous; errors as iluk_symbolic and iluk_numeric.
  */
 int iluk_factor(const iluk_pattern *A, const double *A_val, int k, iluk_sym **S, iluk_fac **F,
@@ -269,8 +271,8 @@ int iluk_apply_sched(iluk_fac *F, const double *p, double *y, int transpose, int
  * forward | backward << 8; it applies to the sweeps of F and of its
  * transpose.  ILUK_SCHED_AUTO (the default) lets the first application
  * outside a stream capture time every schedule (and, for the warp-per-row
- * kinds, several CTA widths) on each sweep and keep the fastest
- * (iluk_get_schedule then returns the packed pair); the transposed sweeps are
+ * kinds, several CTA widths) that suits the shape of the DAG on each sweep and
+ * keep the fastest (iluk_get_schedule then returns the packed pair); the transposed sweeps are
  * timed on their first use and keep their own pair.  Both picks are
  * remembered by the symbolic handle: later factorizations of the same
  * pattern use them without timing again.  An unknown kind or width is
@@ -435,14 +437,15 @@ int iluk_transpose(const iluk_pattern *A, const double *A_val, int64_t *t_rowptr
  * iterations, cycles, relres; x0 = 0, basis ILUK_BASIS_AUTO), device buffers
  * as those calls take them.  What the one call adds is overlap: the first
  * GMRES vector v_1 = b / ||b|| does not depend on the factors, so it is
- * formed first and the one-launch factorization (k >= 2) solves L x = v_1
- * beside its numeric phase, each row's entry of x computed by the warp that
- * has just factored the row (the forward substitution of Eq. forwardsubA, in the
- * same order and roundings as the forward sweep); the first application of
- * the preconditioner then runs only its backward sweep.  When the one-launch
- * path is not taken (k <= 1, a fallback to the two separate phases) the first
- * application runs both sweeps, as gmres_solve does.  sched is the sweep
- * schedule (as iluk_set_schedule; ILUK_SCHED_AUTO times them once F exists).
+ * formed first and the numeric phase solves L x = v_1 as it goes, each row's
+ * entry of x computed by the warp that has just factored the row (the forward
+ * substitution of Eq. forwardsubA, in the same order and roundings as the
+ * forward sweep); the first application of the preconditioner then runs only
+ * its backward sweep.  After a fallback to the two separate calls the first
+ * application runs both sweeps, as gmres_solve does.  Level orders are built
+ * where the solve's sweeps gain from them.  sched is the sweep schedule (as
+ * iluk_set_schedule; ILUK_SCHED_AUTO picks one from the shape of F's DAG,
+ * without timing: the factors keep it, the pattern does not).
  * The factorization is returned through S_out and F_out when both are
  * non-NULL (the caller destroys them), else freed.  A failure of the
  * factorization is reported as iluk_factor reports it (x then holds 0 or is
@@ -461,7 +464,7 @@ int iluk_solve(const iluk_pattern *A, const double *A_val, int k, const double *
  * the inputs to the device on `stream`, runs iluk_solve(k, restart, rtol,
  * maxit, sched) on them (iluk_factor(k) and gmres_solve preconditioned by the
  * ILU(k) sweeps, the first forward sweep inside the factorization; with
- * ILUK_SCHED_AUTO the schedules are timed inside the call), copies x back
+ * ILUK_SCHED_AUTO the schedule follows from the DAG's shape), copies x back
  * and frees its device memory.
  * Synchronous; statuses and info as the calls it makes (x is written even
  * when GMRES returns ILUK_ENOCONV).

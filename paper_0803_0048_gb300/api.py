@@ -197,9 +197,9 @@ def numeric(S: Symbolic, vals: torch.Tensor) -> Factors:
 
 
 def factor(rowptr: torch.Tensor, colind: torch.Tensor, vals: torch.Tensor, k: int):
-    """a2 + a3 with the numeric phase running beside the symbolic one (k >= 2);
-    the same (Symbolic, Factors) as ``symbolic`` then ``numeric``, bit for bit.
-    The sweeps walk index orders until level orders are built."""
+    """a2 + a3 in one call; the same (Symbolic, Factors) as ``symbolic`` then
+    ``numeric``, bit for bit.  Level orders are built on wide DAGs only; on
+    others the sweeps walk index orders until they are."""
     A = CsrPattern(rowptr, colind)
     _vecs((vals, A.nnz, "values of A"))
     hs, hf = C.c_void_p(), C.c_void_p()
@@ -221,10 +221,10 @@ def solve(rowptr: torch.Tensor, colind: torch.Tensor, vals: torch.Tensor, b: tor
     Factors) with ``return_factors`` (precond "ilu" only).
 
     With "ilu" this is one C call (iluk_solve): GMRES forms v_1 = b / ||b||
-    first, the one-launch factorization (k >= 2) solves L x = v_1 beside its
-    numeric phase, and the first preconditioner application runs only its
-    backward sweep; the results are those of ``factor`` then ``gmres`` bit
-    for bit.  ``sched`` is the sweep schedule (0: autotune once F exists)."""
+    first, the numeric phase solves L x = v_1 as it goes, and the first
+    preconditioner application runs only its backward sweep; the results are
+    those of ``factor`` then ``gmres`` bit for bit.  ``sched`` is the sweep
+    schedule (0: picked from the shape of F's DAG)."""
     if precond not in ("ilu", "iilu", "none"):
         raise ValueError("precond must be 'ilu', 'iilu' or 'none'")
     if return_factors and precond != "ilu":
@@ -406,7 +406,8 @@ def solve_host(rowptr, colind, vals, b, k, restart=30, rtol=1e-8, maxit=10000, s
                x=None, check=True):
     """a1-a6 from host memory in one C call (iluk_solve_host): CPU tensors in
     (pinned memory copies fastest), x out on the host.  ``sched`` is a sweep
-    schedule (Factors.schedule() of an earlier solve, or 0 to autotune).
+    schedule (Factors.schedule() of an earlier solve, or 0: picked from the
+    shape of F's DAG).
     Returns (x, info)."""
     n = rowptr.numel() - 1
     nnz = colind.numel()

@@ -4,10 +4,10 @@
 // Each CTA of a persistent grid takes the next instance (an atomic ticket) and
 // runs its whole pipeline alone: ILU(k) numeric factorization, then
 // right-preconditioned GMRES(m) with the ILU sweeps, exactly the algorithm of
-// the single-instance path.  Inside a CTA there is no waiting on flags: the
-// factorization and both sweeps walk the instance's level sets (built by the
-// symbolic phase) with a __syncthreads between levels, and the warps walk the
-// rows of a level with converged FP64 instructions.  Inner products follow the
+// the single-instance path.  The factorization walks the instance's level sets
+// with a __syncthreads between levels; the sweeps walk them with barriers too or
+// (spinning) poll the values their rows need, on a copy of the factors packed
+// for that where the levels are wide enough.  Inner products follow the
 // same 4096-partial fixed tree as the single-instance path, so every instance
 // is bit-identical to solving it on its own.  Instances may have different
 // patterns and sizes (uneven grids); those sharing one symbolic handle share

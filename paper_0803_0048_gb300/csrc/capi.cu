@@ -489,7 +489,7 @@ static int symbolic_impl(const iluk_pattern *A, int k, iluk_sym **out, iluk_info
   CKS(finish());
   cleanup();
   // The level orders of the two sweeps depend only on the pattern; they are
-  // built by the first numeric phase, on a second stream while the
+  // built by the first numeric phase, before its rows or, on a deep DAG, while the
   // factorization runs (see ensure_levels).
 #undef CKS
   *out = S;
@@ -501,13 +501,16 @@ int iluk_symbolic(const iluk_pattern *A, int k, iluk_sym **out, iluk_info *info,
 }
 
 // Build the sweeps' level orders of S once (synchronous on `s`), unless a DAG
-// is deeper than `cap` levels (kLevelsTooDeep: no orders).
+// is deeper than `cap` levels (cap_b: the backward one; kLevelsTooDeep: no orders) or, with
+// `growth`, as deep as its row index suggests (kLevelsLinear: none).
 static std::mutex g_levels_mu;
-static int ensure_levels(const iluk_sym *Sc, cudaStream_t s, int64_t cap = INT32_MAX) {
+static int ensure_levels(const iluk_sym *Sc, cudaStream_t s, int64_t cap = INT32_MAX,
+                         int64_t cap_b = -1, bool growth = false) {
   iluk_sym *S = const_cast<iluk_sym *>(Sc);  // the level orders are a cache of the pattern
   std::lock_guard<std::mutex> lk(g_levels_mu);
   if (S->levels_built) return ILUK_OK;
-  const int st = build_levels_pair(S->n, S->rowptr, S->colind, S->diag, &S->lord, &S->uord, (int)cap, s);
+  const int st = build_levels_pair(S->n, S->rowptr, S->colind, S->diag, &S->lord, &S->uord,
+                                   (int)cap, (int)(cap_b < 0 ? cap : cap_b), growth, s);
   if (st != ILUK_OK) return st;
   S->depth_lower = S->lord.nlev;
   S->depth_upper = S->uord.nlev;
@@ -574,22 +577,33 @@ void iluk_fac_destroy(iluk_fac *F) {
 }
 
 // v0 (may be null): also L x = v0 into F->tmp, which must be pending.
+// The most levels of orders that are built before the rows are factored.
+static int64_t first_levels(const iluk_sym *S) {
+  constexpr int64_t kFirstLevels = 2048, kFirstRows = 64;
+  return std::max(kFirstLevels, S->n / kFirstRows);
+}
+
 static int numeric_into(iluk_fac *F, const double *A_val, iluk_info *info, cudaStream_t s,
-                        bool build_levels = true, const double *v0 = nullptr) {
+                        bool build_levels = true, const double *v0 = nullptr,
+                        int64_t beside = 0, int64_t beside_b = 0) {
   const iluk_sym *S = F->S;
   // The first factorization of this pattern builds the sweeps' level orders,
-  // first, so that its rows are taken in level order too (3D 64^3, k = 2: 0.8 +
-  // 2.7 ms; in index order beside the build the rows took 17.4 ms); a DAG
+  // first, so that its rows are taken in level order too (3D 64^3, k = 2: 1.2 +
+  // 2.5 ms; in index order beside the build the rows took 17.4 ms); a DAG
   // deeper than kFirstLevels and narrower than kFirstRows rows a level is not
   // worth waiting for: its orders are built on a second stream while its rows
   // go in index order, which costs them little (random band, k = 2: 15,777
   // levels, 10 rows each).
-  constexpr int64_t kFirstLevels = 2048, kFirstRows = 64;
+  // So are those of a DAG whose depth grows with the row index (levels.cu):
+  // random band n = 160,000, symbolic and numeric phase, orders first -> beside
+  // the rows: k = 0 2.40 -> 1.71 ms, k = 1 7.08 -> 5.31.  `beside`: the caller's bound on the levels of orders
+  // built beside the rows (beside_b: of the backward DAG), 0: none.
   int lst = ILUK_OK;
   if (build_levels && !S->levels_built) {
-    const int64_t cap = std::max(kFirstLevels, S->n / kFirstRows);
-    lst = ensure_levels(S, s, cap);
-    if (lst != ILUK_OK && lst != kLevelsTooDeep) return fail(info, lst);
+    lst = ensure_levels(S, s, first_levels(S), -1, true);
+    if (lst != ILUK_OK && lst != kLevelsTooDeep && lst != kLevelsLinear) return fail(info, lst);
+    if (!S->levels_built) beside = beside_b = INT32_MAX;
+    lst = ILUK_OK;
   }
   // the numeric phase's row ticket lives in the handle's scratch
   CK(cudaMemsetAsync(F->sync, 0, sweep_sync_ints(S->n) * sizeof(int), s));
@@ -597,17 +611,18 @@ static int numeric_into(iluk_fac *F, const double *A_val, iluk_info *info, cudaS
   // the numeric phase also fills the reciprocals of the diagonal
   CK(launch_numeric(S, A_val, F->val, F->rdiag, reinterpret_cast<unsigned long long *>(F->sync),
                     F->err, v0, v0 ? F->tmp : nullptr, s));
-  if (lst == kLevelsTooDeep) {
+  if (beside > 0) {
     cudaStream_t side = nullptr;
     if (cudaStreamCreateWithFlags(&side, cudaStreamNonBlocking) == cudaSuccess) {
       prof_override = ILUK_PROF_OVERLAPPED;
-      lst = ensure_levels(S, side);
+      lst = ensure_levels(S, side, beside, beside_b);
       prof_override = -1;
       cudaStreamDestroy(side);
     } else {
       cudaGetLastError();
-      lst = ensure_levels(S, s);
+      lst = ensure_levels(S, s, beside, beside_b);
     }
+    if (lst == kLevelsTooDeep) lst = ILUK_OK;
   }
   int64_t row;
   int st = read_err(F->err, s, &row, nullptr);
@@ -693,9 +708,11 @@ static int factor_impl(const iluk_pattern *A, const double *A_val, int k, iluk_s
     *F_out = F2;
     return ILUK_OK;
   };
-  // The two phases one after the other, each over the whole GPU.  Level orders
-  // come between them where the DAG is wide (kWideSweepRows) or a solve's
-  // sweeps gain from them (kSolveSweepRows); else the sweeps walk index orders.
+  // The two phases one after the other, each over the whole GPU.  The sweeps get
+  // level orders where the DAG is wide (kWideSweepRows) or a solve's sweeps gain
+  // from them (kSolveSweepRows), else index orders.  The rows are factored in
+  // level order unless the DAG is deep or its depth grows with the row index
+  // (see numeric_into), then with the orders made beside them.
   auto serial = [&]() -> int {
     cudaStream_t s2 = (cudaStream_t)stream;
     iluk_sym *S2 = nullptr;
@@ -707,9 +724,18 @@ static int factor_impl(const iluk_pattern *A, const double *A_val, int k, iluk_s
     if (solving)
       levels = std::max(S2->n / kSolveSweepRows,
                         S2->max_row <= kRingMaxRow ? kRingLevels : kSolveLevels);
-    st2 = levels > 0 ? ensure_levels(S2, s2, levels) : kLevelsTooDeep;
+    const int64_t levels_b = solving ? levels : INT32_MAX;  // of the backward DAG
+    if (S2->n > 0) {
+      // below kFirstOrderRows rows the orders cost more than the rows gain (2D
+      // 64^2 k = 2 0.99 ms with them, 0.75 without; 3D 20^3 k = 2 1.09, 0.89;
+      // 27-point 30^3 k = 1 2.37, 2.80; 2D 256^2 k = 1 2.42, 6.57)
+      constexpr int64_t kFirstOrderRows = 16384;
+      const int64_t cap =
+          S2->n < kFirstOrderRows ? levels : std::max(levels, first_levels(S2));
+      st2 = ensure_levels(S2, s2, cap, std::max(cap, levels_b), true);
+    }
+    const bool linear = st2 == kLevelsLinear;
     cudaError_t e2 = cudaSuccess;
-    if (st2 == kLevelsTooDeep) e2 = build_index_orders(S2->n, &S2->xlord, &S2->xuord, s2);
     if (e2 == cudaSuccess) e2 = dalloc(&F2->val, S2->nnz, s2);
     if (e2 == cudaSuccess) e2 = dalloc(&F2->sync, sweep_sync_ints(S2->n), s2);
     if (e2 == cudaSuccess) e2 = dalloc(&F2->tmp, S2->n, s2);
@@ -718,11 +744,22 @@ static int factor_impl(const iluk_pattern *A, const double *A_val, int k, iluk_s
     if (e2 == cudaSuccess) e2 = launch_fill_pending(S2->n, F2->tmp, s2);
     if (e2 != cudaSuccess) {
       st2 = fail(info, e2 == cudaErrorMemoryAllocation ? ILUK_ENOMEM : ILUK_ECUDA);
-    } else if (st2 == ILUK_OK || st2 == kLevelsTooDeep) {
-      st2 = numeric_into(F2, A_val, info, s2, false, v0);
+    } else if (st2 == ILUK_OK || st2 == kLevelsTooDeep || linear) {
+      st2 = numeric_into(F2, A_val, info, s2, false, v0, linear ? levels : 0, levels_b);
     } else {
       fail(info, st2);
     }
+    if (st2 == ILUK_OK && S2->levels_built &&
+        (S2->depth_lower > levels || S2->depth_upper > levels_b)) {
+      // orders that only the rows were to have
+      level_order_free(S2->lord, s2);
+      level_order_free(S2->uord, s2);
+      S2->depth_lower = S2->depth_upper = -1;
+      S2->levels_built = false;
+    }
+    if (st2 == ILUK_OK && !S2->levels_built &&
+        build_index_orders(S2->n, &S2->xlord, &S2->xuord, s2) != cudaSuccess)
+      st2 = fail(info, ILUK_ENOMEM);
     if (st2 != ILUK_OK) {
       iluk_fac_destroy(F2);
       iluk_sym_destroy(S2);
@@ -969,8 +1006,8 @@ static int ensure_transpose(iluk_fac *F, cudaStream_t s) {
   dfree(cursor, s);
   dfree(scan_tmp, s);
   if (!F->tlord.order && S->n) {
-    int st = build_levels_pair(S->n, F->trowptr, F->tcolind, F->tdiag, &F->tlord, &F->tuord, INT32_MAX,
-                               s);
+    int st = build_levels_pair(S->n, F->trowptr, F->tcolind, F->tdiag, &F->tlord, &F->tuord,
+                               INT32_MAX, INT32_MAX, false, s);
     if (st != ILUK_OK) return st;
   }
   return ILUK_OK;
@@ -1040,8 +1077,8 @@ static int shape_schedule(const iluk_sym *S) {
   return ILUK_SCHED_WIDTH(ILUK_SCHED_WARP_GRID, 512);
 }
 
-// Autotuner: time every sweep schedule (the warp-per-row ones at several CTA
-// widths) on this factorization, forward and backward sweeps separately, and
+// Autotuner: time the sweep schedules that suit the shape of F's DAG (the
+// warp-per-row ones at several CTA widths) on this factorization, forward and backward sweeps separately, and
 // keep the fastest of each (packed as forward | backward << 8); the sweeps of
 // the transpose (U^T then L^T, a different DAG) get their own pick, made the
 // first time they run (the transpose must exist).  The sweeps' speed depends

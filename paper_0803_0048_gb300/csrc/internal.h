@@ -229,9 +229,10 @@ cudaError_t build_fill_pattern(int64_t n, int64_t nnz, const int64_t *arp, const
                                int64_t max_row, cudaStream_t s);
 
 // Levels (levels.cu): synchronous; allocates both orders on success.
-constexpr int kLevelsTooDeep = -1;
+constexpr int kLevelsTooDeep = -1, kLevelsLinear = -2;
 int build_levels_pair(int64_t n, const int64_t *rp, const int32_t *ci, const int64_t *dg,
-                      LevelOrder *fwd, LevelOrder *bwd, int cap, cudaStream_t s);
+                      LevelOrder *fwd, LevelOrder *bwd, int cap, int cap_b, bool growth,
+                      cudaStream_t s);
 
 // Numeric (numeric.cu)
 // The factor values double as ready flags (numeric.cu); fval is overwritten.

@@ -7,11 +7,14 @@
 // starting on a warp boundary (short levels are padded with -1), so the 32
 // rows of a warp never depend on one another: a warp's lanes only ever wait
 // for rows held by other warps.
+#include <algorithm>
+
 #include "internal.h"
 
 namespace iluk {
 
 constexpr int kDepthThreads = 512;
+constexpr int64_t kGrowthRows = 4096;  // least rows of a DAG whose growth is looked at
 constexpr int kDepthBatch = 4;  // inputs a lane looks at together
 
 // One row per lane: a warp claims the next 32 rows in sweep order through a
@@ -24,14 +27,31 @@ constexpr int kDepthBatch = 4;  // inputs a lane looks at together
 // or not all CTAs are resident.
 // What bounds it: one L2 round trip (~900 cycles) a level.  With a warp per
 // row the rows in flight (one per warp) covered only a part of a wide DAG's
-// wavefront: 3D 64^3, k = 2 (694 levels) 5.8 ms for both directions.
-// A row deeper than `cap` ends the launch (fail = 2): the caller wants no
-// orders for a DAG that deep.
+// wavefront: 3D 64^3, k = 2 (694 levels) 5.8 -> 1.2 ms for both directions.
+// A row deeper than `cap` ends the launch, both directions of it (fail = 2): the
+// caller wants no orders for a DAG that deep.
+// With g, the warp that completes the first g->rows rows looks at how their
+// depth grew (fail = 3 ends the launch): in proportion to the row index, index
+// order nearly is level order, rows in index order find as many others ready and
+// the orders can wait (random bands); where it saturates (grids: the first line
+// and plane hold most of it) rows in index order starve.  The depths of the first
+// 1/32 of the rows against those of the first 1/64: bands 1.67 (n = 20,000 and
+// 160,000, k = 0) to 2.8 (k = 2), grids 1.01 to 1.61 (27-point 30^3, k = 1), of 21
+// patterns.
+struct DepthGrowth {
+  int rows, half;        // the first rows looked at, and half of them
+  int most, most_half;   // their depths
+  int done;              // rows completed
+};
+__device__ __forceinline__ bool grows_linearly(int most, int half) {
+  return 20 * (int64_t)most >= 33 * (int64_t)half;
+}
 template <bool FORWARD>
 __device__ void depth_rows(int64_t n, const int64_t *__restrict__ rp,
                            const int32_t *__restrict__ ci, const int64_t *__restrict__ dg,
                            int32_t *depth, int32_t *maxdepth, DevErr *err, int64_t limit_ns,
-                           unsigned long long *ticket, int *fail, int cap) {
+                           unsigned long long *ticket, int *fail, int *other, int cap,
+                           DepthGrowth *g) {
   const int lane = threadIdx.x & 31;
   int dmax_local = 0;
   for (;;) {
@@ -84,7 +104,10 @@ __device__ void depth_rows(int64_t n, const int64_t *__restrict__ rp,
           asm volatile("st.relaxed.gpu.global.b32 [%0], %1;" ::"l"(&depth[row]), "r"(dm)
                        : "memory");
           if (dm > dmax_local) dmax_local = dm;
-          if (dm > cap) atomicExch(fail, 2);
+          if (dm > cap) {
+            atomicExch(fail, 2);
+            atomicCAS(other, 0, 2);
+          }
           done = moved = true;
         }
       }
@@ -120,6 +143,24 @@ __device__ void depth_rows(int64_t n, const int64_t *__restrict__ rp,
       }
     }
     if (gone) break;
+    if (g != nullptr && t - lane < g->rows) {
+      const int own = mine && t < g->rows ? dm : 0;
+      const int m = __reduce_max_sync(FULL_MASK, own);
+      const int mh = __reduce_max_sync(FULL_MASK, t < g->half ? own : 0);
+      const int cnt = __popc(__ballot_sync(FULL_MASK, t < g->rows));
+      if (lane == 0) {
+        atomicMax(&g->most, m);
+        if (mh) atomicMax(&g->most_half, mh);
+        __threadfence();
+        if (atomicAdd(&g->done, cnt) + cnt == g->rows) {
+          __threadfence();
+          if (grows_linearly(atomicAdd(&g->most, 0), atomicAdd(&g->most_half, 0))) {
+            atomicExch(fail, 3);
+            atomicExch(other, 3);
+          }
+        }
+      }
+    }
   }
   dmax_local = __reduce_max_sync(FULL_MASK, dmax_local);
   if (lane == 0 && dmax_local) atomicMax(maxdepth, dmax_local);
@@ -130,12 +171,14 @@ __device__ void depth_rows(int64_t n, const int64_t *__restrict__ rp,
 __global__ void __launch_bounds__(kDepthThreads)
 k_depth_pair(int64_t n, const int64_t *__restrict__ rp, const int32_t *__restrict__ ci,
              const int64_t *__restrict__ dg, int32_t *depth_f, int32_t *depth_b, int32_t *mx,
-             DevErr *err, unsigned long long *ctl, int64_t limit_ns, int cap) {
+             DevErr *err, unsigned long long *ctl, int64_t limit_ns, int cap, int cap_b,
+             DepthGrowth *g) {
   int *fail = reinterpret_cast<int *>(ctl + 2);
   if ((blockIdx.x & 1) == 0)
-    depth_rows<true>(n, rp, ci, dg, depth_f, mx, err, limit_ns, ctl, fail, cap);
+    depth_rows<true>(n, rp, ci, dg, depth_f, mx, err, limit_ns, ctl, fail, fail + 1, cap, g);
   else
-    depth_rows<false>(n, rp, ci, dg, depth_b, mx + 1, err + 1, limit_ns, ctl + 1, fail + 1, cap);
+    depth_rows<false>(n, rp, ci, dg, depth_b, mx + 1, err + 1, limit_ns, ctl + 1, fail + 1, fail,
+                      cap_b, nullptr);
 }
 
 __global__ void k_level_count(int64_t n, const int32_t *__restrict__ depth, int32_t *cnt) {
@@ -226,10 +269,12 @@ static int order_from_depth(int64_t n, const int32_t *depth, int32_t nlev, Level
 
 // Synchronous: the depths of both sweep DAGs (one launch), then the two padded
 // level orders.  On success fwd->order / bwd->order (and their level starts)
-// are new device allocations.  kLevelsTooDeep (and no orders) when a DAG is
-// deeper than cap.
+// are new device allocations.  kLevelsTooDeep (and no orders) when the forward
+// DAG is deeper than cap or the backward one than cap_b; kLevelsLinear (and none)
+// when `growth` asks and the forward depth grows with the row index.
 int build_levels_pair(int64_t n, const int64_t *rp, const int32_t *ci, const int64_t *dg,
-                      LevelOrder *fwd, LevelOrder *bwd, int cap, cudaStream_t s) {
+                      LevelOrder *fwd, LevelOrder *bwd, int cap, int cap_b, bool growth,
+                      cudaStream_t s) {
   ProfScope prof_scope(ILUK_PROF_DEPTH, s);
   *fwd = LevelOrder();
   *bwd = LevelOrder();
@@ -237,12 +282,22 @@ int build_levels_pair(int64_t n, const int64_t *rp, const int32_t *ci, const int
   int32_t *depth = nullptr, *mx = nullptr;
   DevErr *err = nullptr;
   unsigned long long *ctl = nullptr;  // two tickets, two failure flags
+  DepthGrowth *g = nullptr, hg = {};
+  hg.rows = (int)std::min<int64_t>(n / 32, INT32_MAX);
+  hg.half = hg.rows / 2;
+  growth = growth && n >= kGrowthRows;
   auto cleanup = [&]() {
     if (depth) cudaFreeAsync(depth, s);
     if (mx) cudaFreeAsync(mx, s);
     if (err) cudaFreeAsync(err, s);
     if (ctl) cudaFreeAsync(ctl, s);
+    if (g) cudaFreeAsync(g, s);
   };
+  if (growth && (cudaMallocAsync((void **)&g, sizeof(hg), s) != cudaSuccess ||
+                 cudaMemcpyAsync(g, &hg, sizeof(hg), cudaMemcpyHostToDevice, s) != cudaSuccess)) {
+    cleanup();
+    return ILUK_ECUDA;
+  }
   if (cudaMallocAsync((void **)&depth, 2 * n * sizeof(int32_t), s) != cudaSuccess ||
       cudaMallocAsync((void **)&mx, 2 * sizeof(int32_t), s) != cudaSuccess ||
       cudaMallocAsync((void **)&err, 2 * sizeof(DevErr), s) != cudaSuccess ||
@@ -263,13 +318,14 @@ int build_levels_pair(int64_t n, const int64_t *rp, const int32_t *ci, const int
   if (grid > want) grid = want;
   if (grid < 2) grid = 2;
   k_depth_pair<<<(unsigned)grid, kDepthThreads, 0, s>>>(n, rp, ci, dg, depth, depth + n, mx, err,
-                                                        ctl, wait_limit(), cap);
+                                                        ctl, wait_limit(), cap, cap_b, g);
   note_launch();
   DevErr herr[2];
-  int32_t nlev[2] = {0, 0};
+  int32_t nlev[2] = {0, 0}, fail[2] = {0, 0};
   if (cudaGetLastError() != cudaSuccess ||
       cudaMemcpyAsync(herr, err, sizeof(herr), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
       cudaMemcpyAsync(nlev, mx, sizeof(nlev), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+      cudaMemcpyAsync(fail, ctl + 2, sizeof(fail), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess) {
     cleanup();
     return ILUK_ECUDA;
@@ -279,7 +335,11 @@ int build_levels_pair(int64_t n, const int64_t *rp, const int32_t *ci, const int
       cleanup();
       return (int)(herr[d].key & 0xff);
     }
-  if (nlev[0] > cap || nlev[1] > cap) {
+  if (fail[0] == 3 || fail[1] == 3) {
+    cleanup();
+    return kLevelsLinear;
+  }
+  if (nlev[0] > cap || nlev[1] > cap_b) {
     cleanup();
     return kLevelsTooDeep;
   }

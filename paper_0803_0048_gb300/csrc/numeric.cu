@@ -17,6 +17,9 @@
 // every set advances through the rows together and the sets' independent
 // rows fill the GPU while each set's dependency chain is walked.
 //
+// On wide level orders of short rows k_numeric_staged takes the rows, from a list
+// of every row's updates made once per pattern (see there).
+//
 // k_factor_fused runs this phase beside the symbolic one in one launch, each
 // row starting as soon as its pattern is final (see the section below).
 #include <mutex>

@@ -9,15 +9,18 @@
 // factor's fixed-point reciprocal of f_ii and gives IEEE's quotient
 // (div_fin, common.cuh).
 //
-// Five schedules of the same row task, all bit-identical; the factor handle
-// times them (the warp-per-row ones at several CTA widths) on its first
-// application and keeps the fastest for each direction:
+// Six schedules of the same row task, all bit-identical; the factor handle
+// times those that suit the shape of its DAG (the warp-per-row ones at several
+// CTA widths) on its first application and keeps the fastest for each direction
+// (a one-call solve picks from the shape alone):
 //  * WARP_CLUSTER: one warp per row in one 16-CTA thread-block cluster, x in
 //    the cluster's distributed shared memory on the producer's SM; the warp
 //    subtracts the longest ready prefix of its chain as values arrive, and
 //    when only the last entry is missing, the lane that owns it finishes the
 //    row alone (poll, multiply, subtract, divide, store).
 //    Suits deep, narrow DAGs, where the hand-off latency sets the time.
+//  * WARP_CLUSTER_HELP: the same with a second cluster that subtracts the
+//    leading entries of long rows ahead of their warps.
 //  * WARP_GRID: the same over all SMs with x in global memory (L2 hand-offs);
 //    suits wide DAGs, which need many SMs in flight.
 //  * FLAGS: 32 rows of one level per warp in lockstep over all SMs (L2
