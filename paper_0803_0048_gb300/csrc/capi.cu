@@ -596,8 +596,9 @@ static int numeric_into(iluk_fac *F, const double *A_val, iluk_info *info, cudaS
   // levels, 10 rows each).
   // So are those of a DAG whose depth grows with the row index (levels.cu):
   // random band n = 160,000, symbolic and numeric phase, orders first -> beside
-  // the rows: k = 0 2.40 -> 1.71 ms, k = 1 7.08 -> 5.31.  `beside`: the caller's bound on the levels of orders
-  // built beside the rows (beside_b: of the backward DAG), 0: none.
+  // the rows: k = 0 2.40 -> 1.71 ms, k = 1 7.08 -> 5.31.
+  // `beside`: the caller's bound on the levels of orders built beside the rows
+  // (beside_b: of the backward DAG), 0: none.
   int lst = ILUK_OK;
   if (build_levels && !S->levels_built) {
     lst = ensure_levels(S, s, first_levels(S), -1, true);
