@@ -20,7 +20,7 @@ struct OwnerCode {
 // first use: chunk c is slots 32 c .. 32 c + 31 of the padded order, its plan
 // rows are coff[c] .. coff[c + 1] - 1 (the longest chain of the chunk), and
 // slot[32 r + lane] says where the input of that chain entry sits in the
-// order (or ~row when it lies too far back for the ring).
+// order (or a negative code of the row when it lies too far back for the ring).
 struct LanePlan {
   int64_t nch = 0;
   int maxw = 0;                    // longest chain

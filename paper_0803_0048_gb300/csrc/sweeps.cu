@@ -324,10 +324,21 @@ struct LaneMeta {
 
 template <int W>
 struct LaneWin {
-  int sl[W];  // slot of the input; ~row: far, read from global memory; kNoSlot: none
+  int sl[W];  // slot of the input; far_code(row): read from global memory; kNoSlot: none
   double f[W];
 };
 constexpr int kNoSlot = INT_MAX;  // reads the spare entry
+
+// A far input (row 0 .. INT_MAX - 1) in a plan: negative, and its tag, code + 1
+// like a slot's, has the top bit set.  No slot's tag has it, nor has the tag 0
+// of the entries that no slot has reached, so a far input is never taken for
+// one that the ring holds.  (~row is no such code: row 0's tag would be 0.)
+__host__ __device__ constexpr int far_code(int row) { return -2 - row; }
+__host__ __device__ constexpr int far_row(int code) { return -2 - code; }
+static_assert(far_code(0) < 0 && (unsigned)far_code(0) + 1u > (unsigned)INT_MAX &&
+                  far_code(INT_MAX - 1) < 0 &&
+                  (unsigned)far_code(INT_MAX - 1) + 1u > (unsigned)INT_MAX,
+              "far inputs: negative codes, tags of no slot");
 
 __device__ __forceinline__ void lane_meta(LaneMeta &m, const int32_t *__restrict__ order,
                                           const LanePlan &pl, int64_t c, int lane) {
@@ -413,7 +424,7 @@ __device__ __forceinline__ bool lane_take(const LaneWin<W> &wn, double &s, unsig
         if (wn.sl[u] == kNoSlot || (r[u].y == want[u] && r[u].w == want[u])) continue;
         const bool is_far = wn.sl[u] < 0;
         if (!is_far && r[u].y <= want[u] && r[u].w <= want[u]) continue;  // not there yet
-        const double g = ld_val(&out[is_far ? ~wn.sl[u] : order[wn.sl[u]]]);
+        const double g = ld_val(&out[is_far ? far_row(wn.sl[u]) : order[wn.sl[u]]]);
         if (pending(g)) {
           again = true;
           continue;
@@ -546,7 +557,7 @@ __global__ void k_lane_slots(LanePlan pl, const int32_t *__restrict__ slot_of,
       if (e >= skip) {
         const int32_t col = ci[FORWARD ? f + (e - skip) : f - (e - skip)];
         const int32_t sl = slot_of[col];
-        v = slot - sl < kRingNear ? sl : ~col;
+        v = slot - sl < kRingNear ? sl : far_code(col);
       }
       pslot[(off + e) * 32 + lane] = v;
     }
