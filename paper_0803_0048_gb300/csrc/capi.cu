@@ -1044,12 +1044,14 @@ static const SweepAux *sweep_aux(iluk_fac *F, int sched, cudaStream_t s) {
   return &F->aux;
 }
 
-// The schedule of a one-call solve, from the shape of F's DAG alone: timing
+// The schedule of a one-call solve, from the shape of F's DAGs alone: timing
 // the kinds takes several applications each, more than such a solve makes
 // (random band, n = 160,000, k = 2: 710 ms of timing in a 790 ms call; 2D 64^2:
-// 8 of 18 ms).  `e`: entries of L a level, `r`: rows a level.  Where the lines
-// lie (one application, the kinds timed over 37 grids and bands of 576 to
-// 373,248 rows, k = 0..2; the pick is within ~10 % of the best on all):
+// 8 of 18 ms).  Each direction has its own DAG and its own pick: `e` entries (of L
+// or of U, and no fewer than two a row, which a row costs anyway) a level, `r`
+// rows a level.  Where the lines lie (one application, the
+// kinds timed over 37 grids and bands of 576 to 373,248 rows, k = 0..2; the
+// pick is within ~10 % of the best on all):
 //  * rows of at most 8 entries a side (kRingMaxRow), orders built: one SM up
 //    to 320 entries a level (2D 256^2, e = 287: 0.85 ms, four SMs 0.87; 2D
 //    300^2, e = 337: 1.10 / 1.01), four SMs up to 1,000 (3D 30^3 k = 1, e = 957:
@@ -1058,29 +1060,39 @@ static const SweepAux *sweep_aux(iluk_fac *F, int sched, cudaStream_t s) {
 //    20^3 k = 2, e = 394: 0.30 ms, grid 0.36; 27-point 20^3 k = 1, e = 868: 0.46
 //    / 0.44), with helpers where rows hold 60 entries or more;
 //  * else the warp-per-row grid.
+// With the forward DAG's shape for both directions one-sided patterns lose (one
+// application: upper bidiagonal, n = 6,000, 3.15 ms, with its own 2.11; 2D 256^2
+// upwind 0.53 and 0.28).
 // Without level orders the depth is unknown, but above n / 64 (see factor_impl):
 // narrow.
-static int shape_schedule(const iluk_sym *S) {
-  if (S->n == 0) return ILUK_SCHED_WARP_GRID;
-  const double rows = (double)S->nnz / (double)S->n;
-  const int wc = rows >= 60.0 ? ILUK_SCHED_WARP_CLUSTER_HELP : ILUK_SCHED_WARP_CLUSTER;
-  auto pair = [](int f, int b) { return f | (b << 8); };
-  if (!S->levels_built)
-    return pair(ILUK_SCHED_WIDTH(wc, 512), ILUK_SCHED_WIDTH(wc, 384));
-  const double depth = std::max(S->depth_lower, 1);
-  const double e = ((double)S->nnz - (double)S->n) / 2.0 / depth, r = (double)S->n / depth;
+static int shape_direction(const iluk_sym *S, const LevelOrder &lo) {
+  const double n = (double)S->n, depth = std::max(lo.nlev, 1);
+  const double e = std::max((double)lo.entries, 2.0 * n) / depth, r = n / depth;
   if (S->max_row <= kRingMaxRow && e <= 1000.0)
     return e <= 320.0 ? ILUK_SCHED_SINGLE_CTA : ILUK_SCHED_CLUSTER;
   if (e <= 850.0) {
+    const int wc = 2.0 * (double)lo.entries + n >= 60.0 * n ? ILUK_SCHED_WARP_CLUSTER_HELP
+                                                            : ILUK_SCHED_WARP_CLUSTER;
     const int w = r >= 20.0 ? 512 : 384;
     return ILUK_SCHED_WIDTH(wc, w);
   }
   return ILUK_SCHED_WIDTH(ILUK_SCHED_WARP_GRID, 512);
 }
 
-// Autotuner: time the sweep schedules that suit the shape of F's DAG (the
-// warp-per-row ones at several CTA widths) on this factorization, forward and backward sweeps separately, and
-// keep the fastest of each (packed as forward | backward << 8); the sweeps of
+static int shape_schedule(const iluk_sym *S) {
+  if (S->n == 0) return ILUK_SCHED_WARP_GRID;
+  auto pair = [](int f, int b) { return f == b ? f : f | (b << 8); };
+  if (!S->levels_built) {
+    const int wc = (double)S->nnz >= 60.0 * (double)S->n ? ILUK_SCHED_WARP_CLUSTER_HELP
+                                                         : ILUK_SCHED_WARP_CLUSTER;
+    return pair(ILUK_SCHED_WIDTH(wc, 512), ILUK_SCHED_WIDTH(wc, 384));
+  }
+  return pair(shape_direction(S, S->lord), shape_direction(S, S->uord));
+}
+
+// Autotuner: time the sweep schedules that suit the shape of F's DAGs (the
+// warp-per-row ones at several CTA widths) on this factorization, forward and
+// backward sweeps separately, and keep the fastest of each (packed as forward | backward << 8); the sweeps of
 // the transpose (U^T then L^T, a different DAG) get their own pick, made the
 // first time they run (the transpose must exist).  The sweeps' speed depends
 // on the pattern, not on the values, so each pick is kept with the symbolic
@@ -1120,22 +1132,38 @@ static int pick_schedule(iluk_fac *F, cudaStream_t s, bool transpose = false) {
   cudaEventCreate(&e2);
   // The warp-per-row kinds at several CTA widths: fewer warps keep fewer rows
   // in flight (less polling), more warps start each row earlier.  Where the
-  // orders tell a wide DAG (over 2,500 entries of L a level), the kinds that
-  // keep to a few SMs are left out: there they take 2 to 20 times the grid's
-  // time, most of all in these trials.
-  const bool wide = S->levels_built && S->nnz / 2 > 2500 * (int64_t)S->depth_lower;
-  std::vector<int> candidates = {ILUK_SCHED_FLAGS, ILUK_SCHED_WARP_GRID,
-                                 ILUK_SCHED_WIDTH(ILUK_SCHED_WARP_GRID, 512),
-                                 ILUK_SCHED_WIDTH(ILUK_SCHED_WARP_GRID, 256)};
-  if (!wide)
-    for (int c : {(int)ILUK_SCHED_SINGLE_CTA, (int)ILUK_SCHED_CLUSTER,
-                  ILUK_SCHED_WIDTH(ILUK_SCHED_WARP_CLUSTER, 768),
-                  ILUK_SCHED_WIDTH(ILUK_SCHED_WARP_CLUSTER, 512),
-                  ILUK_SCHED_WIDTH(ILUK_SCHED_WARP_CLUSTER, 384),
-                  ILUK_SCHED_WIDTH(ILUK_SCHED_WARP_CLUSTER_HELP, 512),
-                  ILUK_SCHED_WIDTH(ILUK_SCHED_WARP_CLUSTER_HELP, 384)})
-      candidates.push_back(c);
-  for (int sched : candidates) {
+  // orders tell a wide DAG (over 2,500 entries a level, half the diagonal among
+  // them), the kinds that keep to a few SMs are left out: there they take 2 to 20
+  // times the grid's time, most of all in these trials.  Each direction by its
+  // own DAG (by the forward one alone an upper bidiagonal matrix of 6,000 rows
+  // took 3.16 ms an application instead of 2.06, 2D 256^2 with upper neighbours
+  // only 0.45 instead of 0.28).
+  auto is_wide = [&](const LevelOrder &lo) {
+    return lo.order != nullptr && lo.entries + S->n / 2 > 2500 * (int64_t)lo.nlev;
+  };
+  const bool wide_f = is_wide(transpose ? F->tlord : S->lord);
+  const bool wide_b = is_wide(transpose ? F->tuord : S->uord);
+  struct {
+    int sched;
+    bool few_sms;
+  } const candidates[] = {{ILUK_SCHED_FLAGS, false},
+                          {ILUK_SCHED_WARP_GRID, false},
+                          {ILUK_SCHED_WIDTH(ILUK_SCHED_WARP_GRID, 512), false},
+                          {ILUK_SCHED_WIDTH(ILUK_SCHED_WARP_GRID, 256), false},
+                          {ILUK_SCHED_SINGLE_CTA, true},
+                          {ILUK_SCHED_CLUSTER, true},
+                          {ILUK_SCHED_WIDTH(ILUK_SCHED_WARP_CLUSTER, 768), true},
+                          {ILUK_SCHED_WIDTH(ILUK_SCHED_WARP_CLUSTER, 512), true},
+                          {ILUK_SCHED_WIDTH(ILUK_SCHED_WARP_CLUSTER, 384), true},
+                          {ILUK_SCHED_WIDTH(ILUK_SCHED_WARP_CLUSTER_HELP, 512), true},
+                          {ILUK_SCHED_WIDTH(ILUK_SCHED_WARP_CLUSTER_HELP, 384), true}};
+  for (const auto &cand : candidates) {
+    const bool try_f = !(cand.few_sms && wide_f), try_b = !(cand.few_sms && wide_b);
+    if (!try_f && !try_b) continue;
+    // a direction that leaves this kind out still runs: the other one needs its vectors
+    const int sf = try_f ? cand.sched : (int)ILUK_SCHED_WARP_GRID;
+    const int sb = try_b ? cand.sched : (int)ILUK_SCHED_WARP_GRID;
+    const int sched = sf | (sb << 8);
     float mf = 1e30f, mb = 1e30f;
     for (int rep = 0; rep < 3; ++rep) {
       // the forward sweep alone, then the backward sweep alone, on the same
@@ -1169,13 +1197,13 @@ static int pick_schedule(iluk_fac *F, cudaStream_t s, bool transpose = false) {
         if (b < mb) mb = b;
       }
     }
-    if (mf < best_f) {
+    if (try_f && mf < best_f) {
       best_f = mf;
-      pick_f = sched;
+      pick_f = sf;
     }
-    if (mb < best_b) {
+    if (try_b && mb < best_b) {
       best_b = mb;
-      pick_b = sched;
+      pick_b = sb;
     }
   }
   cudaEventDestroy(e0);

@@ -35,6 +35,7 @@ struct LevelOrder {
   int64_t *lstart = nullptr;  // int64[nlev+1]: first slot of each level
   int64_t len = 0;
   int32_t nlev = 0;
+  int64_t entries = 0;        // off-diagonal entries the sweep reads (of L, or of U)
   int32_t *corder = nullptr;  // the same rows without padding (clen = rows)
   int64_t clen = 0;
   OwnerCode owner[8];         // cache, see OwnerCode

@@ -49,11 +49,12 @@ __device__ __forceinline__ bool grows_linearly(int most, int half) {
 template <bool FORWARD>
 __device__ void depth_rows(int64_t n, const int64_t *__restrict__ rp,
                            const int32_t *__restrict__ ci, const int64_t *__restrict__ dg,
-                           int32_t *depth, int32_t *maxdepth, DevErr *err, int64_t limit_ns,
-                           unsigned long long *ticket, int *fail, int *other, int cap,
-                           DepthGrowth *g) {
+                           int32_t *depth, int32_t *maxdepth, unsigned long long *entries,
+                           DevErr *err, int64_t limit_ns, unsigned long long *ticket, int *fail,
+                           int *other, int cap, DepthGrowth *g) {
   const int lane = threadIdx.x & 31;
   int dmax_local = 0;
+  int64_t entries_local = 0;
   for (;;) {
     unsigned long long tk = 0;
     if (lane == 0) tk = atomicAdd(ticket, 32ull);
@@ -69,6 +70,7 @@ __device__ void depth_rows(int64_t n, const int64_t *__restrict__ rp,
       const int64_t d = dg[row];
       first = FORWARD ? rp[row] : rp[row + 1] - 1;
       len = (int)(FORWARD ? d - first : first - d);
+      entries_local += len;
     }
     int q = 0, dm = 0;
     bool done = !mine;
@@ -163,22 +165,27 @@ __device__ void depth_rows(int64_t n, const int64_t *__restrict__ rp,
     }
   }
   dmax_local = __reduce_max_sync(FULL_MASK, dmax_local);
+#pragma unroll
+  for (int o = 16; o >= 1; o >>= 1)
+    entries_local += __shfl_xor_sync(FULL_MASK, entries_local, o);
   if (lane == 0 && dmax_local) atomicMax(maxdepth, dmax_local);
+  if (lane == 0 && entries_local) atomicAdd(entries, (unsigned long long)entries_local);
 }
 
 // Even CTAs compute the forward depths, odd CTAs the backward depths (the two
-// DAGs are independent).  ctl: two tickets, then two failure flags.
+// DAGs are independent).  ctl: two tickets, the two DAGs' entries, two failure flags.
 __global__ void __launch_bounds__(kDepthThreads)
 k_depth_pair(int64_t n, const int64_t *__restrict__ rp, const int32_t *__restrict__ ci,
              const int64_t *__restrict__ dg, int32_t *depth_f, int32_t *depth_b, int32_t *mx,
              DevErr *err, unsigned long long *ctl, int64_t limit_ns, int cap, int cap_b,
              DepthGrowth *g) {
-  int *fail = reinterpret_cast<int *>(ctl + 2);
+  int *fail = reinterpret_cast<int *>(ctl + 4);
   if ((blockIdx.x & 1) == 0)
-    depth_rows<true>(n, rp, ci, dg, depth_f, mx, err, limit_ns, ctl, fail, fail + 1, cap, g);
+    depth_rows<true>(n, rp, ci, dg, depth_f, mx, ctl + 2, err, limit_ns, ctl, fail, fail + 1, cap,
+                     g);
   else
-    depth_rows<false>(n, rp, ci, dg, depth_b, mx + 1, err + 1, limit_ns, ctl + 1, fail + 1, fail,
-                      cap_b, nullptr);
+    depth_rows<false>(n, rp, ci, dg, depth_b, mx + 1, ctl + 3, err + 1, limit_ns, ctl + 1,
+                      fail + 1, fail, cap_b, nullptr);
 }
 
 __global__ void k_level_count(int64_t n, const int32_t *__restrict__ depth, int32_t *cnt) {
@@ -281,7 +288,7 @@ int build_levels_pair(int64_t n, const int64_t *rp, const int32_t *ci, const int
   if (n == 0) return ILUK_OK;
   int32_t *depth = nullptr, *mx = nullptr;
   DevErr *err = nullptr;
-  unsigned long long *ctl = nullptr;  // two tickets, two failure flags
+  unsigned long long *ctl = nullptr;  // two tickets, two entry counts, two failure flags
   DepthGrowth *g = nullptr, hg = {};
   hg.rows = (int)std::min<int64_t>(n / 32, INT32_MAX);
   hg.half = hg.rows / 2;
@@ -301,10 +308,10 @@ int build_levels_pair(int64_t n, const int64_t *rp, const int32_t *ci, const int
   if (cudaMallocAsync((void **)&depth, 2 * n * sizeof(int32_t), s) != cudaSuccess ||
       cudaMallocAsync((void **)&mx, 2 * sizeof(int32_t), s) != cudaSuccess ||
       cudaMallocAsync((void **)&err, 2 * sizeof(DevErr), s) != cudaSuccess ||
-      cudaMallocAsync((void **)&ctl, 3 * sizeof(unsigned long long), s) != cudaSuccess ||
+      cudaMallocAsync((void **)&ctl, 5 * sizeof(unsigned long long), s) != cudaSuccess ||
       cudaMemsetAsync(depth, 0, 2 * n * sizeof(int32_t), s) != cudaSuccess ||
       cudaMemsetAsync(mx, 0, 2 * sizeof(int32_t), s) != cudaSuccess ||
-      cudaMemsetAsync(ctl, 0, 3 * sizeof(unsigned long long), s) != cudaSuccess ||
+      cudaMemsetAsync(ctl, 0, 5 * sizeof(unsigned long long), s) != cudaSuccess ||
       launch_fill_err(err, s) != cudaSuccess || launch_fill_err(err + 1, s) != cudaSuccess) {
     cleanup();
     return ILUK_ECUDA;
@@ -321,11 +328,17 @@ int build_levels_pair(int64_t n, const int64_t *rp, const int32_t *ci, const int
                                                         ctl, wait_limit(), cap, cap_b, g);
   note_launch();
   DevErr herr[2];
-  int32_t nlev[2] = {0, 0}, fail[2] = {0, 0};
+  int32_t nlev[2] = {0, 0};
+  struct {
+    unsigned long long ticket[2], entries[2];
+    int32_t fail[2];
+  } hctl = {};
+  static_assert(sizeof(hctl) == 5 * sizeof(unsigned long long), "as the kernel lays ctl out");
+  const int32_t *fail = hctl.fail;
   if (cudaGetLastError() != cudaSuccess ||
       cudaMemcpyAsync(herr, err, sizeof(herr), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
       cudaMemcpyAsync(nlev, mx, sizeof(nlev), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-      cudaMemcpyAsync(fail, ctl + 2, sizeof(fail), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+      cudaMemcpyAsync(&hctl, ctl, sizeof(hctl), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess) {
     cleanup();
     return ILUK_ECUDA;
@@ -345,6 +358,8 @@ int build_levels_pair(int64_t n, const int64_t *rp, const int32_t *ci, const int
   }
   int st = order_from_depth(n, depth, nlev[0], fwd, s);
   if (st == ILUK_OK) st = order_from_depth(n, depth + n, nlev[1], bwd, s);
+  fwd->entries = (int64_t)hctl.entries[0];
+  bwd->entries = (int64_t)hctl.entries[1];
   // the orders are read on other streams than the one they were built on (beside
   // a numeric phase; another caller's), which nothing else makes wait
   if (st == ILUK_OK && cudaStreamSynchronize(s) != cudaSuccess) st = ILUK_ECUDA;
