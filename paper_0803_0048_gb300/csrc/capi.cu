@@ -1052,7 +1052,7 @@ static const SweepAux *sweep_aux(iluk_fac *F, int sched, cudaStream_t s) {
 // rows a level.  Where the lines lie (one application, the
 // kinds timed over 37 grids and bands of 576 to 373,248 rows, k = 0..2; the
 // pick is within ~10 % of the best on all):
-//  * rows of at most 8 entries a side (kRingMaxRow), orders built: one SM up
+//  * rows of at most 8 entries on the side (kRingSide), orders built: one SM up
 //    to 320 entries a level (2D 256^2, e = 287: 0.85 ms, four SMs 0.87; 2D
 //    300^2, e = 337: 1.10 / 1.01), four SMs up to 1,000 (3D 30^3 k = 1, e = 957:
 //    0.28 ms, warp-per-row grid 0.34; k = 0, e = 1,043: 0.196 / 0.192);
@@ -1068,7 +1068,7 @@ static const SweepAux *sweep_aux(iluk_fac *F, int sched, cudaStream_t s) {
 static int shape_direction(const iluk_sym *S, const LevelOrder &lo) {
   const double n = (double)S->n, depth = std::max(lo.nlev, 1);
   const double e = std::max((double)lo.entries, 2.0 * n) / depth, r = n / depth;
-  if (S->max_row <= kRingMaxRow && e <= 1000.0)
+  if (lo.longest <= kRingSide && e <= 1000.0)
     return e <= 320.0 ? ILUK_SCHED_SINGLE_CTA : ILUK_SCHED_CLUSTER;
   if (e <= 850.0) {
     const int wc = 2.0 * (double)lo.entries + n >= 60.0 * n ? ILUK_SCHED_WARP_CLUSTER_HELP

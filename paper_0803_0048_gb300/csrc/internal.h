@@ -36,6 +36,7 @@ struct LevelOrder {
   int64_t len = 0;
   int32_t nlev = 0;
   int64_t entries = 0;        // off-diagonal entries the sweep reads (of L, or of U)
+  int32_t longest = 0;        // the most of them in a row
   int32_t *corder = nullptr;  // the same rows without padding (clen = rows)
   int64_t clen = 0;
   OwnerCode owner[8];         // cache, see OwnerCode
@@ -144,7 +145,10 @@ constexpr int64_t kWideSweepRows = 128;
 constexpr int64_t kSolveSweepRows = 64;
 constexpr int64_t kSolveLevels = 600;
 constexpr int64_t kRingLevels = 8192;
-constexpr int kRingMaxRow = 2 * 8 + 1;
+// The most entries a row may have, on the side that is swept, to be taken by a
+// ring sweep, and the longest row of F of which that can be said for both sides.
+constexpr int kRingSide = 8;
+constexpr int kRingMaxRow = 2 * kRingSide + 1;
 
 int64_t wait_limit();
 void note_launch();              // counts kernel launches (iluk_launch_count)

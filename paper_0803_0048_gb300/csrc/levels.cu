@@ -49,11 +49,12 @@ __device__ __forceinline__ bool grows_linearly(int most, int half) {
 template <bool FORWARD>
 __device__ void depth_rows(int64_t n, const int64_t *__restrict__ rp,
                            const int32_t *__restrict__ ci, const int64_t *__restrict__ dg,
-                           int32_t *depth, int32_t *maxdepth, unsigned long long *entries,
-                           DevErr *err, int64_t limit_ns, unsigned long long *ticket, int *fail,
-                           int *other, int cap, DepthGrowth *g) {
+                           int32_t *depth, int32_t *maxdepth, int32_t *longest,
+                           unsigned long long *entries, DevErr *err, int64_t limit_ns,
+                           unsigned long long *ticket, int *fail, int *other, int cap,
+                           DepthGrowth *g) {
   const int lane = threadIdx.x & 31;
-  int dmax_local = 0;
+  int dmax_local = 0, longest_local = 0;
   int64_t entries_local = 0;
   for (;;) {
     unsigned long long tk = 0;
@@ -71,6 +72,7 @@ __device__ void depth_rows(int64_t n, const int64_t *__restrict__ rp,
       first = FORWARD ? rp[row] : rp[row + 1] - 1;
       len = (int)(FORWARD ? d - first : first - d);
       entries_local += len;
+      if (len > longest_local) longest_local = len;
     }
     int q = 0, dm = 0;
     bool done = !mine;
@@ -168,12 +170,15 @@ __device__ void depth_rows(int64_t n, const int64_t *__restrict__ rp,
 #pragma unroll
   for (int o = 16; o >= 1; o >>= 1)
     entries_local += __shfl_xor_sync(FULL_MASK, entries_local, o);
+  longest_local = __reduce_max_sync(FULL_MASK, longest_local);
   if (lane == 0 && dmax_local) atomicMax(maxdepth, dmax_local);
+  if (lane == 0 && longest_local) atomicMax(longest, longest_local);
   if (lane == 0 && entries_local) atomicAdd(entries, (unsigned long long)entries_local);
 }
 
 // Even CTAs compute the forward depths, odd CTAs the backward depths (the two
-// DAGs are independent).  ctl: two tickets, the two DAGs' entries, two failure flags.
+// DAGs are independent).  mx: the two depths, the two longest rows; ctl: two
+// tickets, the two DAGs' entries, two failure flags.
 __global__ void __launch_bounds__(kDepthThreads)
 k_depth_pair(int64_t n, const int64_t *__restrict__ rp, const int32_t *__restrict__ ci,
              const int64_t *__restrict__ dg, int32_t *depth_f, int32_t *depth_b, int32_t *mx,
@@ -181,10 +186,10 @@ k_depth_pair(int64_t n, const int64_t *__restrict__ rp, const int32_t *__restric
              DepthGrowth *g) {
   int *fail = reinterpret_cast<int *>(ctl + 4);
   if ((blockIdx.x & 1) == 0)
-    depth_rows<true>(n, rp, ci, dg, depth_f, mx, ctl + 2, err, limit_ns, ctl, fail, fail + 1, cap,
-                     g);
+    depth_rows<true>(n, rp, ci, dg, depth_f, mx, mx + 2, ctl + 2, err, limit_ns, ctl, fail,
+                     fail + 1, cap, g);
   else
-    depth_rows<false>(n, rp, ci, dg, depth_b, mx + 1, ctl + 3, err + 1, limit_ns, ctl + 1,
+    depth_rows<false>(n, rp, ci, dg, depth_b, mx + 1, mx + 3, ctl + 3, err + 1, limit_ns, ctl + 1,
                       fail + 1, fail, cap_b, nullptr);
 }
 
@@ -306,11 +311,11 @@ int build_levels_pair(int64_t n, const int64_t *rp, const int32_t *ci, const int
     return ILUK_ECUDA;
   }
   if (cudaMallocAsync((void **)&depth, 2 * n * sizeof(int32_t), s) != cudaSuccess ||
-      cudaMallocAsync((void **)&mx, 2 * sizeof(int32_t), s) != cudaSuccess ||
+      cudaMallocAsync((void **)&mx, 4 * sizeof(int32_t), s) != cudaSuccess ||
       cudaMallocAsync((void **)&err, 2 * sizeof(DevErr), s) != cudaSuccess ||
       cudaMallocAsync((void **)&ctl, 5 * sizeof(unsigned long long), s) != cudaSuccess ||
       cudaMemsetAsync(depth, 0, 2 * n * sizeof(int32_t), s) != cudaSuccess ||
-      cudaMemsetAsync(mx, 0, 2 * sizeof(int32_t), s) != cudaSuccess ||
+      cudaMemsetAsync(mx, 0, 4 * sizeof(int32_t), s) != cudaSuccess ||
       cudaMemsetAsync(ctl, 0, 5 * sizeof(unsigned long long), s) != cudaSuccess ||
       launch_fill_err(err, s) != cudaSuccess || launch_fill_err(err + 1, s) != cudaSuccess) {
     cleanup();
@@ -328,7 +333,7 @@ int build_levels_pair(int64_t n, const int64_t *rp, const int32_t *ci, const int
                                                         ctl, wait_limit(), cap, cap_b, g);
   note_launch();
   DevErr herr[2];
-  int32_t nlev[2] = {0, 0};
+  int32_t nlev[4] = {0, 0, 0, 0};  // and the longest rows
   struct {
     unsigned long long ticket[2], entries[2];
     int32_t fail[2];
@@ -360,6 +365,8 @@ int build_levels_pair(int64_t n, const int64_t *rp, const int32_t *ci, const int
   if (st == ILUK_OK) st = order_from_depth(n, depth + n, nlev[1], bwd, s);
   fwd->entries = (int64_t)hctl.entries[0];
   bwd->entries = (int64_t)hctl.entries[1];
+  fwd->longest = nlev[2];
+  bwd->longest = nlev[3];
   // the orders are read on other streams than the one they were built on (beside
   // a numeric phase; another caller's), which nothing else makes wait
   if (st == ILUK_OK && cudaStreamSynchronize(s) != cudaSuccess) st = ILUK_ECUDA;

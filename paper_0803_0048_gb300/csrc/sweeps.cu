@@ -221,7 +221,7 @@ constexpr int kRing = 8192;
 constexpr int kRingNear = kRing - 2048;
 constexpr int kLaneMaxThreads = 256;
 constexpr int kLaneW = 4;        // most entries of a window
-constexpr int kLaneMaxRow = 8;   // and of a row
+constexpr int kLaneMaxRow = kRingSide;  // and of a row
 // the ring, a spare entry of no tag, and spare entries of every thread
 constexpr size_t kRingBytes = (size_t)(kRing + 1 + kLaneMaxThreads * kLaneW) * 16;
 

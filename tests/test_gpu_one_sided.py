@@ -84,3 +84,26 @@ def test_autotuner_per_direction(sign):
     assert deep in FEW_SMS and flat in ALL_SMS
     assert_bits_equal(F.apply(pd, transpose=True), oracle.apply_t(A.n, trp, tci, tv, p),
                       "transposed")
+
+
+@pytest.mark.parametrize("lower,upper", [(8, 2), (9, 2), (14, 2), (15, 1), (2, 9), (2, 14)])
+def test_one_call_pick_by_the_side_it_sweeps(lower, upper):
+    """Rows of up to 8 entries on a side are swept on the ring, longer ones by
+    a cluster on DAGs this narrow, whatever the other side holds (rows of up to
+    17 entries in all, for which the solve builds the level orders)."""
+    n = 6000
+    A = from_rows(n, lambda i: [i - 7 * j for j in range(1, lower + 1)] +
+                  [i + 11 * j for j in range(1, upper + 1)], 3)
+    rp, ci, av = to_dev(A)
+    b, bd = vec(82, n)
+    x, info, (S, F) = P.solve(rp, ci, av, bd, 0, return_factors=True)
+    f, b_ = kinds(F.schedule())
+    ring = (L.SCHED_SINGLE_CTA, L.SCHED_CLUSTER)
+    assert (f in ring) == (lower <= 8) and (b_ in ring) == (upper <= 8)
+    assert f in FEW_SMS and b_ in FEW_SMS
+    ref = oracle.factor(A, 0)
+    st, xo, it, *_ = oracle.gmres(n, A.rowptr, A.colind, A.val, b, oracle.PREC_ILU,
+                                  (ref["rowptr"], ref["colind"], ref["val"]), 30, 1e-8,
+                                  dotmode=oracle.DOT_TREE)
+    assert st == oracle.OK and info.iters == it
+    assert_bits_equal(x, xo, f"{lower} lower, {upper} upper")
