@@ -1048,14 +1048,18 @@ static const SweepAux *sweep_aux(iluk_fac *F, int sched, cudaStream_t s) {
 // the kinds takes several applications each, more than such a solve makes
 // (random band, n = 160,000, k = 2: 710 ms of timing in a 790 ms call; 2D 64^2:
 // 8 of 18 ms).  Each direction has its own DAG and its own pick: `e` entries (of L
-// or of U, and no fewer than two a row, which a row costs anyway) a level, `r`
-// rows a level.  Where the lines lie (one application, the
-// kinds timed over 37 grids and bands of 576 to 373,248 rows, k = 0..2; the
-// pick is within ~10 % of the best on all):
+// or of U) a level, `r` rows a level.  Where the lines lie (one application, the
+// kinds timed over 37 grids and bands of 576 to 373,248 rows, k = 0..2, and 35
+// grids around the lines; the pick is within ~10 % of the best on all):
 //  * rows of at most 8 entries on the side (kRingSide), orders built: one SM up
-//    to 320 entries a level (2D 256^2, e = 287: 0.85 ms, four SMs 0.87; 2D
-//    300^2, e = 337: 1.10 / 1.01), four SMs up to 1,000 (3D 30^3 k = 1, e = 957:
-//    0.28 ms, warp-per-row grid 0.34; k = 0, e = 1,043: 0.196 / 0.192);
+//    to e + 2 r = 390, four SMs up to 1,300, then the grid (a row costs about two
+//    entries: by entries alone one SM kept 2D 300^2 k = 0, e = 299, r = 150, 0.81 ms,
+//    four SMs 0.58).  One SM / four: 2D k = 0, 160^2 (e + 2 r = 319) 0.274 / 0.281 ms, 200^2
+//    (399) 0.395 / 0.359; k = 1, 160^2 (267) 0.375 / 0.409, 200^2 (333) 0.517 /
+//    0.512; k = 2, 256^2 (383) 0.831 / 0.870, 300^2 (449) 1.090 / 1.020; 3D k = 0,
+//    14^3 (329) 0.054 / 0.058, 18^3 (542) 0.085 / 0.074; k = 1, 16^3 (335) 0.116 /
+//    0.118, 18^3 (426) 0.140 / 0.134.  Four SMs / grid: 3D 30^3 k = 1 (1,188) 0.277 /
+//    0.316, k = 0 (1,504) 0.193 / 0.175;
 //  * longer rows: a warp per row on a cluster up to 850 entries a level (3D
 //    20^3 k = 2, e = 394: 0.30 ms, grid 0.36; 27-point 20^3 k = 1, e = 868: 0.46
 //    / 0.44), with helpers where rows hold 60 entries or more;
@@ -1067,16 +1071,19 @@ static const SweepAux *sweep_aux(iluk_fac *F, int sched, cudaStream_t s) {
 // narrow.
 static int shape_direction(const iluk_sym *S, const LevelOrder &lo) {
   const double n = (double)S->n, depth = std::max(lo.nlev, 1);
-  const double e = std::max((double)lo.entries, 2.0 * n) / depth, r = n / depth;
-  if (lo.longest <= kRingSide && e <= 1000.0)
-    return e <= 320.0 ? ILUK_SCHED_SINGLE_CTA : ILUK_SCHED_CLUSTER;
-  if (e <= 850.0) {
+  const double e = (double)lo.entries / depth, r = n / depth;
+  const int grid = ILUK_SCHED_WIDTH(ILUK_SCHED_WARP_GRID, 512);
+  if (lo.longest <= kRingSide) {
+    const double w = e + 2.0 * r;
+    return w <= 390.0 ? ILUK_SCHED_SINGLE_CTA : w <= 1300.0 ? ILUK_SCHED_CLUSTER : grid;
+  }
+  if (std::max(e, 2.0 * r) <= 850.0) {
     const int wc = 2.0 * (double)lo.entries + n >= 60.0 * n ? ILUK_SCHED_WARP_CLUSTER_HELP
                                                             : ILUK_SCHED_WARP_CLUSTER;
     const int w = r >= 20.0 ? 512 : 384;
     return ILUK_SCHED_WIDTH(wc, w);
   }
-  return ILUK_SCHED_WIDTH(ILUK_SCHED_WARP_GRID, 512);
+  return grid;
 }
 
 static int shape_schedule(const iluk_sym *S) {

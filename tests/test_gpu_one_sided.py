@@ -107,3 +107,16 @@ def test_one_call_pick_by_the_side_it_sweeps(lower, upper):
                                   dotmode=oracle.DOT_TREE)
     assert st == oracle.OK and info.iters == it
     assert_bits_equal(x, xo, f"{lower} lower, {upper} upper")
+
+
+@pytest.mark.parametrize("N,k,kind", [(128, 0, L.SCHED_SINGLE_CTA), (256, 0, L.SCHED_CLUSTER),
+                                      (300, 1, L.SCHED_CLUSTER), (200, 2, L.SCHED_SINGLE_CTA)])
+def test_one_call_pick_counts_rows_too(N, k, kind):
+    """Levels of many short rows go to four SMs before levels of few longer
+    ones with as many entries do (256^2 k = 0: 255 entries a level on 128 rows;
+    200^2 k = 2: 199 on 50)."""
+    A = W.conv_diff(N, 2, (20.0, 20.0))
+    rp, ci, av = to_dev(A)
+    b, bd = vec(83, A.n)
+    x, info, (S, F) = P.solve(rp, ci, av, bd, k, maxit=2, check=False, return_factors=True)
+    assert kinds(F.schedule()) == (kind, kind)
