@@ -531,7 +531,8 @@ int iluk_batch_results(iluk_batch *B, iluk_info *infos, void *stream);
  * 512 and 1024 threads per item (as many items at once as fit on each SM:
  * up to four, two, one), each with level-barrier sweeps (every level of the
  * in-CTA sweeps ends at a barrier; left out where every item's levels are wide
- * enough for the packed spinning sweeps) and with spinning sweeps (each warp
+ * enough for the packed spinning sweeps, whose copies of the factors that solve
+ * makes, in at most an eighth of the free memory) and with spinning sweeps (each warp
  * polls the values its rows need, no barriers), and keeps the fastest; the results
  * do not depend on the choice.  Threads per item chosen (0 until the first
  * solve) and whether the sweeps spin (1) or use level barriers (0). */

@@ -1476,6 +1476,11 @@ struct iluk_batch {
   int restart = 30, maxit = 10000, cap = 32, width = 0;
   bool spin = false;  // in-CTA sweeps polling values instead of level barriers
   bool packed = false;  // every item's spinning sweeps run on a packed copy
+  // the packed copies are made by the first solve that may spin (make_packs)
+  bool packs_made = false, allpack = false;
+  size_t maxpack = 0;
+  int64_t ldv = 0;
+  std::vector<std::array<double *, 6>> slots;  // the buffers of each work slot
   double rtol = 1e-8;
   int64_t nwork = 0;  // work slots (CTAs of the widest grid)
   std::vector<int64_t> order;  // ticket t runs item order[t]: largest items first
@@ -1497,6 +1502,22 @@ void iluk_batch_destroy(iluk_batch *B) {
   delete B;
 }
 
+}  // extern "C"
+
+// The work slots' descriptors, the first of them with a packed copy each.
+static cudaError_t upload_work(const iluk_batch *B, const std::vector<unsigned char *> &packs,
+                               cudaStream_t s) {
+  std::vector<unsigned char> hwork(batch_work_bytes() * B->nwork);
+  for (size_t w = 0; w < B->slots.size(); ++w) {
+    const std::array<double *, 6> &q = B->slots[w];
+    batch_pack_work(hwork.data() + w * batch_work_bytes(), q[0], q[1], q[2], q[3], q[4], q[5],
+                    B->ldv, w < packs.size() ? packs[w] : nullptr);
+  }
+  return cudaMemcpyAsync(B->work, hwork.data(), hwork.size(), cudaMemcpyHostToDevice, s);
+}
+
+extern "C" {
+
 int iluk_batch_create(const iluk_batch_item *items, int64_t nitems, int restart, double rtol,
                       int maxit, iluk_batch **out, void *stream) {
   iluk_info *info = nullptr;
@@ -1512,8 +1533,7 @@ int iluk_batch_create(const iluk_batch_item *items, int64_t nitems, int restart,
   B->maxit = maxit;
   int64_t maxn = 1, maxf = 1;
   int maxrow = 1;
-  size_t maxpack = 0;
-  bool allpack = nitems > 0;
+  B->allpack = nitems > 0;
   std::vector<unsigned char> hitems(batch_item_bytes() * (nitems ? nitems : 1));
   for (int64_t i = 0; i < nitems; ++i) {
     const iluk_batch_item &it = items[i];
@@ -1547,8 +1567,8 @@ int iluk_batch_create(const iluk_batch_item *items, int64_t nitems, int restart,
     if (it.S->nnz > maxf) maxf = it.S->nnz;
     if (it.S->max_row > maxrow) maxrow = it.S->max_row;
     const size_t pack = batch_pack_bytes(it.S);
-    maxpack = std::max(maxpack, pack);
-    allpack = allpack && pack > 0;
+    B->maxpack = std::max(B->maxpack, pack);
+    B->allpack = B->allpack && pack > 0;
   }
   B->cap = (maxrow + 31) & ~31;
   if (batch_smem_bytes(1024, B->cap, restart) + 8 * 1024 > (size_t)max_smem_optin()) {
@@ -1569,9 +1589,7 @@ int iluk_batch_create(const iluk_batch_item *items, int64_t nitems, int restart,
     cleanup();
     return ILUK_ENOMEM;
   }
-  std::vector<unsigned char> hwork(batch_work_bytes() * B->nwork);
-  std::vector<unsigned char *> packs(B->nwork, nullptr);
-  std::vector<std::array<double *, 6>> slots;
+  B->ldv = ldv;
   for (int64_t w = 0; w < B->nwork; ++w) {
     double *fval, *V, *vw, *z, *u, *tmp;
     if (dalloc(&fval, maxf, s) != cudaSuccess || (B->bufs.push_back(fval), false) ||
@@ -1584,30 +1602,42 @@ int iluk_batch_create(const iluk_batch_item *items, int64_t nitems, int restart,
       return ILUK_ENOMEM;
     }
     B->bufs.push_back(tmp);
-    slots.push_back({fval, V, vw, z, u, tmp});
+    B->slots.push_back({fval, V, vw, z, u, tmp});
   }
-  // the packed sweeps take what memory is left; a slot without reads F instead
-  for (int64_t w = 0; w < B->nwork; ++w) {
-    unsigned char *pack = nullptr;
-    if (maxpack > 0 && (w == 0 || packs[w - 1])) {
-      if (dalloc(&pack, maxpack, s) == cudaSuccess) {
-        B->bufs.push_back(reinterpret_cast<double *>(pack));
-      } else {
-        pack = nullptr;
-        cudaGetLastError();
-      }
-    }
-    packs[w] = pack;
-    const std::array<double *, 6> &q = slots[w];
-    batch_pack_work(hwork.data() + w * batch_work_bytes(), q[0], q[1], q[2], q[3], q[4], q[5], ldv,
-                    pack);
-  }
-  B->packed = allpack && packs.back() != nullptr;
   CK(cudaMemcpyAsync(B->items, hitems.data(), hitems.size(), cudaMemcpyHostToDevice, s));
-  CK(cudaMemcpyAsync(B->work, hwork.data(), hwork.size(), cudaMemcpyHostToDevice, s));
+  CK(upload_work(B, {}, s));
   CK(cudaStreamSynchronize(s));
   *out = B;
   return ILUK_OK;
+}
+
+// Packed copies for the spinning sweeps, one a work slot, of the largest item
+// that takes one: made outside a capture by the first solve that may spin.  They
+// take at most an eighth of the free memory, so that what the process does beside
+// the batch finds room (levels of four rows, padded to 32 slots of 176 bytes, make
+// a copy of 1.4 KB a row, more than both GMRES bases at restart 30); a slot without
+// one reads F instead.
+static void make_packs(iluk_batch *B, cudaStream_t s) {
+  if (B->packs_made || B->maxpack == 0) return;
+  size_t free_b = 0, total_b = 0;
+  if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
+    cudaGetLastError();
+    return;
+  }
+  B->packs_made = true;
+  const int64_t fit = std::min<int64_t>(B->nwork, (int64_t)(free_b / 8 / B->maxpack));
+  std::vector<unsigned char *> packs;
+  for (int64_t w = 0; w < fit; ++w) {
+    unsigned char *pack = nullptr;
+    if (dalloc(&pack, B->maxpack, s) != cudaSuccess) {
+      cudaGetLastError();
+      break;
+    }
+    B->bufs.push_back(reinterpret_cast<double *>(pack));
+    packs.push_back(pack);
+  }
+  if (upload_work(B, packs, s) != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) return;
+  B->packed = B->allpack && (int64_t)packs.size() == B->nwork;
 }
 
 static cudaError_t batch_launch(iluk_batch *B, int width, bool spin, cudaStream_t s) {
@@ -1620,10 +1650,15 @@ int iluk_batch_solve(iluk_batch *B, void *stream) {
   if (!B) return ILUK_EINVAL;
   if (B->nitems == 0) return ILUK_OK;
   cudaStream_t s = (cudaStream_t)stream;
-  if (B->width == 0) {
+  bool capturing = false;
+  if (B->width == 0 || (B->spin && !B->packs_made)) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     cudaStreamIsCapturing(s, &cs);
-    if (cs != cudaStreamCaptureStatusNone) {
+    capturing = cs != cudaStreamCaptureStatusNone;
+    if (!capturing) make_packs(B, s);
+  }
+  if (B->width == 0) {
+    if (capturing) {
       B->width = 1024;
     } else {
       // Autotuner: run the whole batch at each width, with level-barrier
