@@ -601,7 +601,7 @@ k_numeric(int64_t n, int64_t nbatch, const int64_t *__restrict__ arp,
 // entry sees its updates in the same order as above.
 // What bounds it: per level one hand-off through L2, then multiplier (div_fin)
 // and update of the trailing pivots one after the other (~550 cycles each).
-// Refactorization: 27-point 50^3 k = 1 4.19 -> 2.82 ms, 90^3 k = 0 5.92 -> 3.05, 30^3
+// Refactorization: 27-point 50^3 k = 1 4.19 -> 2.78 ms, 90^3 k = 0 5.92 -> 3.05, 30^3
 // k = 1 1.43 -> 0.99, 3D 64^3 k = 2 2.70 -> 2.14, 72^3 k = 0 1.27 -> 0.79, 2D 256^2 k = 2
 // 1.68 -> 1.51; making the plan for 64^3 0.35 ms.  On narrower DAGs (below
 // kStageLevelRows) the early publishing above is worth more: random band k = 1,
@@ -613,6 +613,10 @@ k_numeric(int64_t n, int64_t nbatch, const int64_t *__restrict__ arp,
 constexpr int64_t kStageLevelRows = 48;
 constexpr int kStageAhead = 6;
 constexpr int kStageLook = 4;  // updates a lane watches while it waits
+constexpr int kStageMaxRow = 128;  // entries of a row of F
+constexpr int kStageMax = 2048;    // updates of a row
+static_assert(32 * kStageLook >= kStageMaxRow - 1,
+              "a warp watches all updates of one pivot (to its right in the row) at once");
 
 // One row's updates: calls add(t, q, from, pos) for the t-th (in order), found
 // by pivot q (row-relative) at F's position `from`, for position pos; then
@@ -825,11 +829,6 @@ k_numeric_staged(int64_t n, const int64_t *__restrict__ arp, const int32_t *__re
 #pragma unroll
           for (int u = 0; u < kStageLook; ++u)
             p = p || (e0 + lane + 32 * u < e1 && pend_f(val[u]));
-          for (int t = e0 + lane + 32 * kStageLook; t < e1; t += 32) {  // longer pivot rows
-            double x = w.sv[t];
-            if (pend_f(x)) w.sv[t] = x = ld_gpu(&fv[w.src[t]]);
-            p = p || pend_f(x);
-          }
           if (!__any_sync(FULL_MASK, p)) break;
           const bool stop = (it & 31u) == 31u && (earlier_failed(err, row) ||
                                                   (int64_t)(globaltimer_ns() - tw) > limit_ns);
@@ -1104,8 +1103,6 @@ static int numeric_cap(const iluk_sym *S, size_t static_smem, bool wide, int *wa
 // k_numeric_staged), made on first use; false when the pattern does not suit
 // it (long rows, more updates than kStageMax a row, more plan than an eighth of
 // the free memory) or while `s` is being captured.  Synchronous.
-constexpr int kStageMaxRow = 128;  // entries of a row of F
-constexpr int kStageMax = 2048;    // updates of a row
 static std::mutex g_stage_mu;
 static bool ensure_stage_plan(const iluk_sym *Sc, cudaStream_t s) {
   iluk_sym *S = const_cast<iluk_sym *>(Sc);  // the plan is a cache of the pattern
