@@ -273,17 +273,15 @@ cudaError_t build_fill_pattern(int64_t n, int64_t nnz, const int64_t *arp, const
     int warps = kFillThreads / 32;
     while (warps > 1 && (size_t)words * 8 * warps > (size_t)max_smem_optin() / 2) warps >>= 1;
     const size_t smem = (size_t)words * 8 * warps;
-    e = cudaFuncSetAttribute(k_fill_rows<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_fill_rows<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)smem);
+    e = allow_smem(k_fill_rows<false>);
+    if (e == cudaSuccess) e = allow_smem(k_fill_rows<true>);
     if (e != cudaSuccess) break;
     int64_t grid = (n + warps - 1) / warps;
     if (grid > (int64_t)num_sms() * 32) grid = (int64_t)num_sms() * 32;
     k_fill_rows<false><<<(unsigned)grid, warps * 32, smem, s>>>(n, crp, cci, lev, ustart, p, words,
                                                                row_len, nullptr, nullptr, nullptr);
     note_launch();
+    e = cudaGetLastError();
     alloc(&nrp, n + 1);
     if (e == cudaSuccess) e = launch_scan_lengths(n, row_len, nrp, scan_tmp, s);
     int64_t nn = 0;
@@ -301,6 +299,9 @@ cudaError_t build_fill_pattern(int64_t n, int64_t nnz, const int64_t *arp, const
     k_fill_rows<true><<<(unsigned)grid, warps * 32, smem, s>>>(n, crp, cci, lev, ustart, p, words,
                                                               nullptr, nrp, nci, nlev);
     note_launch();
+    // a launch that was refused has written no pattern for the next pass to read
+    e = cudaGetLastError();
+    if (e != cudaSuccess) break;
     drop(rp);
     drop(ci);
     drop(lev);

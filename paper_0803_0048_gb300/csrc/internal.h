@@ -181,6 +181,17 @@ inline bool symbolic_indep(int k) { return k <= 1 && symbolic_variant() != 2; } 
 int num_sms();
 int max_smem_optin();
 
+// Lets `kern`, which has `fixed` bytes of static shared memory, be launched with as
+// much dynamic shared memory as the device gives, whatever this launch needs.  The
+// limit belongs to the function, not to the launch: set to each launch's own
+// size, a thread with a smaller one lowers it under another's feet, and that
+// launch is refused.
+template <class K>
+cudaError_t allow_smem(K kern, size_t fixed = 0) {
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              max_smem_optin() - (int)fixed);
+}
+
 // Validation / utilities (validate.cu)
 cudaError_t launch_validate(int64_t n, int64_t nnz, const int64_t *rp, const int32_t *ci,
                             DevErr *err, cudaStream_t s);
