@@ -1122,6 +1122,10 @@ k_batch_solve(const BatchItemDev *items, int64_t nitems, BatchResultDev *results
   }
 }
 
+// Left beside the dynamic shared memory (iluk_batch_create): the kernel's few static
+// words.
+constexpr size_t kBStatic = 1024;
+
 size_t batch_smem_bytes(int nt, int cap, int m) {
   return (size_t)kDotP * 8 + ((size_t)(m + 1) * m + 4 * (size_t)m + 1) * 8 +
          (size_t)(nt / 32) * cap * 12;
@@ -1135,8 +1139,7 @@ static cudaError_t launch_bs(const void *items, int64_t nitems, void *results, v
                              int maxit, int cap, bool spin, cudaStream_t s) {
   const size_t smem = batch_smem_bytes(NT, cap, m);
   auto kern = spin ? k_batch_solve<NT, true> : k_batch_solve<NT, false>;
-  cudaError_t e =
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(kern, kBStatic);
   if (e != cudaSuccess) return e;
   // as many CTAs as fit on the GPU at once, within the work slots
   int bps = 0;

@@ -358,8 +358,7 @@ cudaError_t launch_mgs(int64_t n, const double *w, const double *V, int64_t ldv,
   ProfScope prof_scope(ILUK_PROF_DOT, s);
   const int group = mgs_group(rows);
   const auto kern = group == 8 ? k_mgs<8> : group == 4 ? k_mgs<4> : k_mgs<1>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
+  cudaError_t e = allow_smem(kern, sizeof(MgsShared));
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(kMgsCluster * kMgsClusters));

@@ -1212,8 +1212,7 @@ static cudaError_t launch_numeric_impl(const iluk_sym *S, int64_t nbatch, const 
     const int64_t rows8 = 8 * S->n / S->lord.nlev;
     const int sw_max = rows8 > 16 * (int64_t)num_sms() ? kStagedThreads / 32 : 16;
     if (sw > sw_max) sw = sw_max;
-    e = cudaFuncSetAttribute(k_numeric_staged, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(per * sw));
+    e = allow_smem(k_numeric_staged);
     if (e != cudaSuccess) return e;
     int64_t grid = num_sms();
     const int64_t want = (S->n + sw - 1) / sw;
@@ -1225,7 +1224,7 @@ static cudaError_t launch_numeric_impl(const iluk_sym *S, int64_t nbatch, const 
     note_launch();
     return cudaGetLastError();
   }
-  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  e = allow_smem(kern, early ? kStaticSmem : 0);
   if (e != cudaSuccess) return e;
   int bps = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, warps * 32, smem);
@@ -1265,8 +1264,7 @@ cudaError_t launch_factor_fused(int64_t n, int64_t nnz_a, const int64_t *arp,
   }
   const size_t smem = sym_smem > num_smem ? sym_smem : num_smem;
   if (smem + kStaticSmem > (size_t)max_smem_optin()) return cudaErrorInvalidConfiguration;
-  cudaError_t e = cudaFuncSetAttribute(k_factor_fused, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
+  cudaError_t e = allow_smem(k_factor_fused, kStaticSmem);
   if (e != cudaSuccess) return e;
   int bps = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_factor_fused, kNumThreads, smem);

@@ -1235,8 +1235,7 @@ static int cluster_width(int64_t n, K kern, size_t fixed = 0, int widest = 16) {
       // schedulable widths do not depend on n beyond the shared memory size
       if (dev < 64 && cached[dev][0] == C && (size_t)cached[dev][1] >= smem) return C;
     }
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-            cudaSuccess ||
+    if (allow_smem(kern) != cudaSuccess ||
         cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
             cudaSuccess) {
       cudaGetLastError();
@@ -1277,7 +1276,7 @@ static int ring_cluster() {
 template <typename K, typename... Args>
 static cudaError_t launch_on_cluster(K kern, int C, int threads, size_t smem, cudaStream_t s,
                                      Args... args) {
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(kern);
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e != cudaSuccess) return e;
@@ -1303,7 +1302,7 @@ static cudaError_t launch_on_cluster(K kern, int C, int threads, size_t smem, cu
 // helper CTAs wait on the sweep's.
 template <typename K, typename... Args>
 static cudaError_t launch_help(K kern, int threads, size_t smem, cudaStream_t s, Args... args) {
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(kern);
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e != cudaSuccess) return e;

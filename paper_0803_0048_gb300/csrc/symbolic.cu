@@ -101,13 +101,11 @@ static cudaError_t symbolic_shape(int k, int cap, int mapw, int *warps_out, size
   int bps = 0;
   cudaError_t e;
   if (symbolic_indep(k)) {
-    e = cudaFuncSetAttribute(k_symbolic_rows<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
+    e = allow_smem(k_symbolic_rows<true>);
     if (e == cudaSuccess)
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_symbolic_rows<true>, warps * 32, smem);
   } else {
-    e = cudaFuncSetAttribute(k_symbolic_rows<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
+    e = allow_smem(k_symbolic_rows<false>);
     if (e == cudaSuccess)
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_symbolic_rows<false>, warps * 32,
                                                     smem);

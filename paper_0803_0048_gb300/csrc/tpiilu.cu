@@ -352,7 +352,7 @@ cudaError_t launch_iiluk_build(const iluk_sym *S, const double *fval, const DivP
     k_fill_pending_g<<<(unsigned)b, 256, 0, s>>>(S->nnz, g);
     note_launch();
   }
-  e = cudaFuncSetAttribute(k_iiluk_build, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  e = allow_smem(k_iiluk_build);
   if (e != cudaSuccess) return e;
   int bps = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_iiluk_build, warps * 32, smem);
