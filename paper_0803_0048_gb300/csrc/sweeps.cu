@@ -475,6 +475,27 @@ k_sweep_lane(const int32_t *__restrict__ order, LanePlan pl, const double *__res
   const unsigned own = rc.base + (unsigned)(kRing + 1 + threadIdx.x * kLaneW) * 16u;
   const int64_t step = (int64_t)rc.C * (blockDim.x >> 5);
   int64_t c = (int64_t)rc.rank + (int64_t)rc.C * (threadIdx.x >> 5);
+  auto hand_over = [&](int64_t slot, double s) {
+    if (rc.C == 1) {
+      ring_put_local(rc.base, slot, s);
+    } else {
+      for (unsigned k = 1; k <= rc.C; ++k)
+        ring_put(rc.base, (rc.rank + k) & (rc.C - 1), slot, s);
+    }
+  };
+  // Level 1 comes first and reads no x.  Without a divisor its rows pass their right-
+  // hand side through, and the marker becomes the quiet NaN that the other
+  // schedules store.
+  for (; c < pl.nch && pl.coff[c + 1] == pl.coff[c]; c += step) {
+    const int64_t slot = c * 32 + lane;
+    const int32_t row = order[slot];
+    double s = row >= 0 ? in[row] : 0.0;
+    if (DIVIDE && row >= 0) s = div_fin(s, rd[row]);
+    if (pending(s)) s = __longlong_as_double((long long)kQuietNaN);
+    if (clear && row >= 0) clear[row] = __longlong_as_double((long long)kPending);
+    hand_over(slot, s);
+    if (row >= 0) st_val(&out[row], s);
+  }
   LaneChunk<W> cur, nxt;
   lane_meta(cur.m, order, pl, c, lane);
   lane_meta(nxt.m, order, pl, c + step, lane);
@@ -497,13 +518,7 @@ k_sweep_lane(const int32_t *__restrict__ order, LanePlan pl, const double *__res
     }
     // (a padding lane has no divisor)
     if (DIVIDE && row >= 0) s = div_fin(s, rr);
-    const int64_t slot = c * 32 + lane;
-    if (rc.C == 1) {
-      ring_put_local(rc.base, slot, s);
-    } else {
-      for (unsigned k = 1; k <= rc.C; ++k)
-        ring_put(rc.base, (rc.rank + k) & (rc.C - 1), slot, s);
-    }
+    hand_over(c * 32 + lane, s);
     // (s comes from a subtraction or a division, never the signalling marker)
     if (row >= 0) st_val(&out[row], s);
     cur = nxt;
