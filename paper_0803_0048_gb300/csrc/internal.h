@@ -24,6 +24,7 @@ struct OwnerCode {
 struct LanePlan {
   int64_t nch = 0;
   int maxw = 0;                    // longest chain
+  bool refused = false;            // no plan: it would take too much memory
   const int64_t *coff = nullptr;   // int64[nch + 1]
   const int64_t *first = nullptr;  // per slot: position in F of the chain's first entry
   const int32_t *len = nullptr;    // per slot: chain length

@@ -1116,7 +1116,11 @@ static unsigned row_blocks(int64_t n) {
 }
 
 // What the ring kernels need beside a level order, built once per order and
-// kept with it.  Nothing is built while `s` is being captured.
+// kept with it, in at most an eighth of the free memory (rows in levels of one take
+// 512 bytes each, most of them padding); an order that was refused for that stays
+// with the other kinds.  (Asking costs 12 us, 0.4 % of a one-call solve on 2D 64^2:
+// up to 64 MB it is not done.)  Nothing is built while `s` is being captured.
+constexpr size_t kPlanUnasked = 64u << 20;
 static std::mutex g_plan_mu;
 
 static bool capturing(cudaStream_t s) {
@@ -1131,7 +1135,20 @@ static bool ensure_lane_plan(const LevelOrder &lo_c, int64_t n, const int64_t *r
   LevelOrder &lo = const_cast<LevelOrder &>(lo_c);  // a cache of the order
   std::lock_guard<std::mutex> lk(g_plan_mu);
   if (lo.plan.slot) return true;
-  if (!lo.order || lo.plan.maxw > kLaneMaxRow || capturing(s)) return false;
+  if (!lo.order || lo.plan.maxw > kLaneMaxRow || lo.plan.refused || capturing(s)) return false;
+  if (lo.longest > kLaneMaxRow) {  // not for these sweeps: remembered by maxw
+    lo.plan.maxw = lo.longest;
+    return false;
+  }
+  const size_t need = (size_t)lo.len * (12 + 4 * (size_t)lo.longest);
+  if (need > kPlanUnasked) {
+    size_t free_b = 0, total_b = 0;
+    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess || need > free_b / 8) {
+      cudaGetLastError();
+      lo.plan.refused = true;
+      return false;
+    }
+  }
   LanePlan pl;
   pl.nch = lo.len / 32;
   int32_t *slot_of = nullptr, *w = nullptr, *len = nullptr, *pslot = nullptr;
@@ -1166,11 +1183,6 @@ static bool ensure_lane_plan(const LevelOrder &lo_c, int64_t n, const int64_t *r
       cudaStreamSynchronize(s) != cudaSuccess)
     return free_all(false);
   pl.maxw = maxw;
-  if (maxw > kLaneMaxRow) {  // not for these sweeps: remembered by maxw
-    lo.plan = LanePlan();
-    lo.plan.maxw = maxw;
-    return free_all(false);
-  }
   if (cudaMallocAsync((void **)&pslot, (size_t)(rows > 0 ? rows : 1) * 32 * 4, s) != cudaSuccess)
     return free_all(false);
   pl.len = len;
