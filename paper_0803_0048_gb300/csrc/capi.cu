@@ -369,7 +369,7 @@ static int symbolic_impl(const iluk_pattern *A, int k, iluk_sym **out, iluk_info
   // below takes the patterns whose window they do not, and the compared
   // variants of k <= 1.
   if (n > 0 && (k >= 2 || symbolic_variant() == 0)) {
-    const int64_t cols = fill_window(n, A->rowptr, A->colind, s);
+    const int64_t cols = fill_window(n, nnz, A->rowptr, A->colind, k, s);
     if (cols > 0) {
       FillPattern fp;
       const int64_t row_max = max_smem_optin() / 5 / 32 * 32;
@@ -782,7 +782,7 @@ static int factor_impl(const iluk_pattern *A, const double *A_val, int k, iluk_s
   }
   cudaStream_t s = (cudaStream_t)stream;
   const int64_t n = A->n, nnz = A->nnz;
-  if (fill_window(n, A->rowptr, A->colind, s) > 0) return serial();
+  if (fill_window(n, nnz, A->rowptr, A->colind, k, s) > 0) return serial();
 
   SymArena ar{};
   DevErr *err = nullptr;

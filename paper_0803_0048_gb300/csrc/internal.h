@@ -240,7 +240,8 @@ struct FillPattern {
   uint8_t *level = nullptr;
   int64_t *diag = nullptr;
 };
-int64_t fill_window(int64_t n, const int64_t *arp, const int32_t *aci, cudaStream_t s);
+int64_t fill_window(int64_t n, int64_t nnz, const int64_t *arp, const int32_t *aci, int k,
+                    cudaStream_t s);
 cudaError_t build_fill_pattern(int64_t n, int64_t nnz, const int64_t *arp, const int32_t *aci,
                                int k, int64_t cols, FillPattern *fp, int32_t *maxrow, DevErr *err,
                                int64_t max_row, cudaStream_t s);

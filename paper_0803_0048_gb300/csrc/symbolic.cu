@@ -19,8 +19,8 @@
 // entries directly, one round trip after they land.  Rows are compacted into CSR
 // afterwards (Sec. 3.4).
 //
-// This walk takes the patterns of k >= 2 that reach too far for fill.cu, which
-// needs no waits, and those whose general walk is asked for.
+// This walk takes the patterns of k >= 2 that fill.cu, which needs no waits, does not
+// (fill_window: those that reach too far, or across the matrix at a high k), and those whose general walk is asked for.
 //
 // With k <= 1 rows are independent (Sec. 3.3: only level-0 entries can cause
 // fill), so the warp reads the pivot rows straight from A and never waits;
