@@ -502,7 +502,7 @@ int iluk_symbolic(const iluk_pattern *A, int k, iluk_sym **out, iluk_info *info,
 
 // Build the sweeps' level orders of S once (synchronous on `s`), unless a DAG
 // is deeper than `cap` levels (cap_b: the backward one; kLevelsTooDeep: no orders) or, with
-// `growth`, as deep as its row index suggests (kLevelsLinear: none).
+// `growth`, index order serves its rows as well (kLevelsLinear: none).
 static std::mutex g_levels_mu;
 static int ensure_levels(const iluk_sym *Sc, cudaStream_t s, int64_t cap = INT32_MAX,
                          int64_t cap_b = -1, bool growth = false) {
@@ -576,27 +576,24 @@ void iluk_fac_destroy(iluk_fac *F) {
   delete F;
 }
 
-// v0 (may be null): also L x = v0 into F->tmp, which must be pending.
 // The most levels of orders that are built before the rows are factored.
 static int64_t first_levels(const iluk_sym *S) {
   constexpr int64_t kFirstLevels = 2048, kFirstRows = 64;
   return std::max(kFirstLevels, S->n / kFirstRows);
 }
 
+// v0 (may be null): also L x = v0 into F->tmp, which must be pending.
 static int numeric_into(iluk_fac *F, const double *A_val, iluk_info *info, cudaStream_t s,
                         bool build_levels = true, const double *v0 = nullptr,
                         int64_t beside = 0, int64_t beside_b = 0) {
   const iluk_sym *S = F->S;
   // The first factorization of this pattern builds the sweeps' level orders,
   // first, so that its rows are taken in level order too (3D 64^3, k = 2: 1.2 +
-  // 2.5 ms; in index order beside the build the rows took 17.4 ms); a DAG
-  // deeper than kFirstLevels and narrower than kFirstRows rows a level is not
-  // worth waiting for: its orders are built on a second stream while its rows
-  // go in index order, which costs them little (random band, k = 2: 15,777
-  // levels, 10 rows each).
-  // So are those of a DAG whose depth grows with the row index (levels.cu):
-  // random band n = 160,000, symbolic and numeric phase, orders first -> beside
-  // the rows: k = 0 2.40 -> 1.71 ms, k = 1 7.08 -> 5.31.
+  // 2.5 ms; in index order beside the build the rows took 17.4 ms).  The orders are
+  // built on a second stream beside the rows, which go in index order, where that
+  // is faster: DAGs deeper than kFirstLevels and narrower than kFirstRows rows a
+  // level (random band, k = 2: 15,777 levels, 10 rows each), those of few rows, and
+  // those that index order serves nearly as well (levels.cu).
   // `beside`: the caller's bound on the levels of orders built beside the rows
   // (beside_b: of the backward DAG), 0: none.
   int lst = ILUK_OK;
@@ -712,8 +709,8 @@ static int factor_impl(const iluk_pattern *A, const double *A_val, int k, iluk_s
   // The two phases one after the other, each over the whole GPU.  The sweeps get
   // level orders where the DAG is wide (kWideSweepRows) or a solve's sweeps gain
   // from them (kSolveSweepRows), else index orders.  The rows are factored in
-  // level order unless the DAG is deep or its depth grows with the row index
-  // (see numeric_into), then with the orders made beside them.
+  // level order unless the DAG is deep or index order serves them (see
+  // numeric_into), then with the orders made beside them.
   auto serial = [&]() -> int {
     cudaStream_t s2 = (cudaStream_t)stream;
     iluk_sym *S2 = nullptr;
@@ -727,12 +724,7 @@ static int factor_impl(const iluk_pattern *A, const double *A_val, int k, iluk_s
                         S2->max_row <= kRingMaxRow ? kRingLevels : kSolveLevels);
     const int64_t levels_b = solving ? levels : INT32_MAX;  // of the backward DAG
     if (S2->n > 0) {
-      // below kFirstOrderRows rows the orders cost more than the rows gain (2D
-      // 64^2 k = 2 0.99 ms with them, 0.75 without; 3D 20^3 k = 2 1.09, 0.89;
-      // 27-point 30^3 k = 1 2.37, 2.80; 2D 256^2 k = 1 2.42, 6.57)
-      constexpr int64_t kFirstOrderRows = 16384;
-      const int64_t cap =
-          S2->n < kFirstOrderRows ? levels : std::max(levels, first_levels(S2));
+      const int64_t cap = std::max(levels, first_levels(S2));
       st2 = ensure_levels(S2, s2, cap, std::max(cap, levels_b), true);
     }
     const bool linear = st2 == kLevelsLinear;

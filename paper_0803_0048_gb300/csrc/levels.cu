@@ -14,7 +14,8 @@
 namespace iluk {
 
 constexpr int kDepthThreads = 512;
-constexpr int64_t kGrowthRows = 4096;  // least rows of a DAG whose growth is looked at
+constexpr int kWindowRows = 2048;          // about the rows in flight of a numeric phase
+constexpr int64_t kLevelOrderRows = 20000;  // least rows of a DAG for which orders come first
 constexpr int kDepthBatch = 4;  // inputs a lane looks at together
 
 // One row per lane: a warp claims the next 32 rows in sweep order through a
@@ -30,29 +31,68 @@ constexpr int kDepthBatch = 4;  // inputs a lane looks at together
 // wavefront: 3D 64^3, k = 2 (694 levels) 5.8 -> 1.2 ms for both directions.
 // A row deeper than `cap` ends the launch, both directions of it (fail = 2): the
 // caller wants no orders for a DAG that deep.
-// With g, the warp that completes the first g->rows rows looks at how their
-// depth grew (fail = 3 ends the launch): in proportion to the row index, index
-// order nearly is level order, rows in index order find as many others ready and
-// the orders can wait (random bands); where it saturates (grids: the first line
-// and plane hold most of it) rows in index order starve.  The depths of the first
-// 1/32 of the rows against those of the first 1/64: bands 1.67 (n = 20,000 and
-// 160,000, k = 0) to 2.8 (k = 2), grids 1.01 to 1.61 (27-point 30^3, k = 1), of 21
-// patterns.
+// With g, the warps that complete the first rows decide whether rows in index order
+// are worth more than waiting for the orders (fail = 3 ends the launch).  They look
+//  * at 1/64 of the rows, if that is 1,024 or more, whether their depth is over 2.05
+//    times that of the first half of them: faster than along any line of a grid;
+//  * at 1/32, whether it is 1.65 times that of the first 1/64: it grows with the row
+//    index (random bands at k >= 1, 1.85 to 3.2), index order nearly is level order;
+//  * at the same or at 4,096 rows, by what each way costs.  In index order the rows in
+//    flight are about kWindowRows successive ones, so the rows take n / kWindowRows
+//    times a window's depth, here the first one's; with the orders first they take
+//    the DAG's depth, reckoned from what the last quarter of those rows added, in
+//    steps that cost as much, after a depth kernel of that depth and ~0.3 ms.
+// Symbolic and numeric phase, orders first / beside the rows (steps in index order,
+// levels): 2D 256^2 k = 0 (8,448, 511) 1.87 / 6.0 ms, 128 x 512 k = 0 (4,608, 639) 2.28 /
+// 3.36, 64 x 1,024 k = 0 (3,072, 1,087) 3.52 / 2.55, 30 x 3,000 k = 0 (4,312, 3,029) 11.9 /
+// 7.3; 3D 30^3 k = 0 (818, 88) 0.94 / 1.07; 27-point 30^3 k = 0 (1,300, 204) 1.29 / 1.53,
+// k = 1 (1,850, 378) 2.35 / 2.39; random bands, whose windows add up to their depth, n =
+// 160,000 k = 0 2.46 / 1.58, k = 1 7.2 / 5.1, n = 40,000 with 4 a row k = 0 0.94 / 0.65.
+// The wrong side costs these differences and no more.
 struct DepthGrowth {
-  int rows, half;        // the first rows looked at, and half of them
-  int most, most_half;   // their depths
-  int done;              // rows completed
+  int most[6];  // depths of the first rows looked at (GrowthRows)
+  int done[3];  // rows completed of the three looks'
 };
-__device__ __forceinline__ bool grows_linearly(int most, int half) {
-  return 20 * (int64_t)most >= 33 * (int64_t)half;
+struct GrowthRows {
+  // the first 1/128, 1/64 and 1/32 of all rows, a window, 3/4 of and all of the last
+  // look's; whole warps
+  int part128, part64, part32, window, before, all;
+};
+__device__ __forceinline__ bool index_order_serves(int64_t n, int window, int before, int all,
+                                                   const GrowthRows &gr) {
+  const int64_t in_index_order = n * window / gr.window;
+  const int64_t levels = all + (n - gr.all) * (all - before) / (gr.all - gr.before);
+  return in_index_order <= 3 * levels + 200;
 }
+// Rows t0r .. t0r + 31, of depth m at most, are done: whether the launch should end.
+// Not inlined: the rows' loop above all is on the critical path.
+__device__ __noinline__ bool growth_look(int64_t n, int64_t t0r, int m, DepthGrowth *g,
+                                         GrowthRows gr) {
+  if (t0r < gr.part128) atomicMax(&g->most[0], m);
+  if (t0r < gr.part64) atomicMax(&g->most[1], m);
+  if (t0r < gr.part32) atomicMax(&g->most[2], m);
+  if (t0r < gr.window) atomicMax(&g->most[3], m);
+  if (t0r < gr.before) atomicMax(&g->most[4], m);
+  atomicMax(&g->most[5], m);
+  __threadfence();
+  const bool look0 = t0r < gr.part64 && atomicAdd(&g->done[0], 32) + 32 == gr.part64;
+  const bool look1 = t0r < gr.part32 && atomicAdd(&g->done[1], 32) + 32 == gr.part32;
+  const bool look2 = atomicAdd(&g->done[2], 32) + 32 == gr.all;
+  if (!look0 && !look1 && !look2) return false;
+  __threadfence();
+  const volatile int *most = g->most;
+  return (look0 && gr.part64 >= 1024 && 20 * (int64_t)most[1] > 41 * (int64_t)most[0]) ||
+         (look1 && 20 * (int64_t)most[2] >= 33 * (int64_t)most[1]) ||
+         (look2 && index_order_serves(n, most[3], most[4], most[5], gr));
+}
+
 template <bool FORWARD>
 __device__ void depth_rows(int64_t n, const int64_t *__restrict__ rp,
                            const int32_t *__restrict__ ci, const int64_t *__restrict__ dg,
                            int32_t *depth, int32_t *maxdepth, int32_t *longest,
                            unsigned long long *entries, DevErr *err, int64_t limit_ns,
                            unsigned long long *ticket, int *fail, int *other, int cap,
-                           DepthGrowth *g) {
+                           DepthGrowth *g, const GrowthRows &gr) {
   const int lane = threadIdx.x & 31;
   int dmax_local = 0, longest_local = 0;
   int64_t entries_local = 0;
@@ -147,22 +187,12 @@ __device__ void depth_rows(int64_t n, const int64_t *__restrict__ rp,
       }
     }
     if (gone) break;
-    if (g != nullptr && t - lane < g->rows) {
-      const int own = mine && t < g->rows ? dm : 0;
-      const int m = __reduce_max_sync(FULL_MASK, own);
-      const int mh = __reduce_max_sync(FULL_MASK, t < g->half ? own : 0);
-      const int cnt = __popc(__ballot_sync(FULL_MASK, t < g->rows));
-      if (lane == 0) {
-        atomicMax(&g->most, m);
-        if (mh) atomicMax(&g->most_half, mh);
-        __threadfence();
-        if (atomicAdd(&g->done, cnt) + cnt == g->rows) {
-          __threadfence();
-          if (grows_linearly(atomicAdd(&g->most, 0), atomicAdd(&g->most_half, 0))) {
-            atomicExch(fail, 3);
-            atomicExch(other, 3);
-          }
-        }
+    const int64_t t0r = t - lane;
+    if (g != nullptr && t0r < gr.all) {
+      const int m = __reduce_max_sync(FULL_MASK, dm);
+      if (lane == 0 && growth_look(n, t0r, m, g, gr)) {
+        atomicExch(fail, 3);
+        atomicExch(other, 3);
       }
     }
   }
@@ -183,14 +213,14 @@ __global__ void __launch_bounds__(kDepthThreads)
 k_depth_pair(int64_t n, const int64_t *__restrict__ rp, const int32_t *__restrict__ ci,
              const int64_t *__restrict__ dg, int32_t *depth_f, int32_t *depth_b, int32_t *mx,
              DevErr *err, unsigned long long *ctl, int64_t limit_ns, int cap, int cap_b,
-             DepthGrowth *g) {
+             DepthGrowth *g, GrowthRows gr) {
   int *fail = reinterpret_cast<int *>(ctl + 4);
   if ((blockIdx.x & 1) == 0)
     depth_rows<true>(n, rp, ci, dg, depth_f, mx, mx + 2, ctl + 2, err, limit_ns, ctl, fail,
-                     fail + 1, cap, g);
+                     fail + 1, cap, g, gr);
   else
     depth_rows<false>(n, rp, ci, dg, depth_b, mx + 1, mx + 3, ctl + 3, err + 1, limit_ns, ctl + 1,
-                      fail + 1, fail, cap_b, nullptr);
+                      fail + 1, fail, cap_b, nullptr, gr);
 }
 
 __global__ void k_level_count(int64_t n, const int32_t *__restrict__ depth, int32_t *cnt) {
@@ -283,7 +313,9 @@ static int order_from_depth(int64_t n, const int32_t *depth, int32_t nlev, Level
 // level orders.  On success fwd->order / bwd->order (and their level starts)
 // are new device allocations.  kLevelsTooDeep (and no orders) when the forward
 // DAG is deeper than cap or the backward one than cap_b; kLevelsLinear (and none)
-// when `growth` asks and the forward depth grows with the row index.
+// when `growth` asks and rows in index order do not need them: a DAG of fewer than
+// kLevelOrderRows rows (3D 20^3 k = 2 1.12 ms with the orders first, 0.79 beside the
+// rows), or see index_order_serves.
 int build_levels_pair(int64_t n, const int64_t *rp, const int32_t *ci, const int64_t *dg,
                       LevelOrder *fwd, LevelOrder *bwd, int cap, int cap_b, bool growth,
                       cudaStream_t s) {
@@ -294,10 +326,18 @@ int build_levels_pair(int64_t n, const int64_t *rp, const int32_t *ci, const int
   int32_t *depth = nullptr, *mx = nullptr;
   DevErr *err = nullptr;
   unsigned long long *ctl = nullptr;  // two tickets, two entry counts, two failure flags
-  DepthGrowth *g = nullptr, hg = {};
-  hg.rows = (int)std::min<int64_t>(n / 32, INT32_MAX);
-  hg.half = hg.rows / 2;
-  growth = growth && n >= kGrowthRows;
+  if (growth && n < kLevelOrderRows) return kLevelsLinear;
+  DepthGrowth *g = nullptr;
+  GrowthRows gr = {};
+  auto warps = [](int64_t rows) {
+    return (int)(std::min<int64_t>(rows, INT32_MAX / 2) / 32 * 32);
+  };
+  gr.part128 = warps(n / 128);
+  gr.part64 = warps(n / 64);
+  gr.part32 = warps(n / 32);
+  gr.window = kWindowRows;
+  gr.all = std::max(gr.part32, 2 * kWindowRows);
+  gr.before = warps(gr.all - gr.all / 4);
   auto cleanup = [&]() {
     if (depth) cudaFreeAsync(depth, s);
     if (mx) cudaFreeAsync(mx, s);
@@ -305,8 +345,8 @@ int build_levels_pair(int64_t n, const int64_t *rp, const int32_t *ci, const int
     if (ctl) cudaFreeAsync(ctl, s);
     if (g) cudaFreeAsync(g, s);
   };
-  if (growth && (cudaMallocAsync((void **)&g, sizeof(hg), s) != cudaSuccess ||
-                 cudaMemcpyAsync(g, &hg, sizeof(hg), cudaMemcpyHostToDevice, s) != cudaSuccess)) {
+  if (growth && (cudaMallocAsync((void **)&g, sizeof(*g), s) != cudaSuccess ||
+                 cudaMemsetAsync(g, 0, sizeof(*g), s) != cudaSuccess)) {
     cleanup();
     return ILUK_ECUDA;
   }
@@ -330,7 +370,7 @@ int build_levels_pair(int64_t n, const int64_t *rp, const int32_t *ci, const int
   if (grid > want) grid = want;
   if (grid < 2) grid = 2;
   k_depth_pair<<<(unsigned)grid, kDepthThreads, 0, s>>>(n, rp, ci, dg, depth, depth + n, mx, err,
-                                                        ctl, wait_limit(), cap, cap_b, g);
+                                                        ctl, wait_limit(), cap, cap_b, g, gr);
   note_launch();
   DevErr herr[2];
   int32_t nlev[4] = {0, 0, 0, 0};  // and the longest rows
