@@ -1041,44 +1041,45 @@ static const SweepAux *sweep_aux(iluk_fac *F, int sched, cudaStream_t s) {
 // (random band, n = 160,000, k = 2: 710 ms of timing in a 790 ms call; 2D 64^2:
 // 8 of 18 ms).  Each direction has its own DAG and its own pick: `e` entries (of L
 // or of U) a level, `r` rows a level.  Where the lines lie (one application, the
-// kinds timed over 37 grids and bands of 576 to 373,248 rows, k = 0..2, and 35
-// grids around the lines; the pick is within ~10 % of the best on all):
-//  * rows of at most 8 entries on the side (kRingSide), orders built: one SM up
-//    to e + 2 r = 390, four SMs up to 1,300, then the grid (a row costs about two
-//    entries: by entries alone one SM kept 2D 300^2 k = 0, e = 299, r = 150, 0.81 ms,
-//    four SMs 0.58).  One SM / four: 2D k = 0, 160^2 (e + 2 r = 319) 0.274 / 0.281 ms, 200^2
-//    (399) 0.395 / 0.359; k = 1, 160^2 (267) 0.375 / 0.409, 200^2 (333) 0.517 /
+// kinds timed over 37 grids and bands of 576 to 373,248 rows, k = 0..2, and 85
+// around the lines; the pick is within ~10 % of the best on all but where noted):
+//  * rows of at most 8 entries on the side (kRingSide), orders built, inputs near
+//    (ring_suits): one SM up to e + 2 r = 390 (410 for rows of over 4 entries: 2D
+//    256^2 k = 3, 408, 1.26 / 1.43 ms), four SMs up to 1,300, then the grid (a row
+//    costs about two entries: by entries alone one SM kept 2D 300^2 k = 0, e = 299, r =
+//    150, 0.81 ms, four SMs 0.58).  One SM / four: 2D k = 0, 160^2 (e + 2 r = 319) 0.274
+//    / 0.281 ms, 200^2 (399) 0.395 / 0.359; k = 1, 160^2 (267) 0.375 / 0.409, 200^2 (333) 0.517 /
 //    0.512; k = 2, 256^2 (383) 0.831 / 0.870, 300^2 (449) 1.090 / 1.020; 3D k = 0,
 //    14^3 (329) 0.054 / 0.058, 18^3 (542) 0.085 / 0.074; k = 1, 16^3 (335) 0.116 /
 //    0.118, 18^3 (426) 0.140 / 0.134.  Four SMs / grid: 3D 30^3 k = 1 (1,188) 0.277 /
 //    0.316, k = 0 (1,504) 0.193 / 0.175;
-//  * longer rows: a warp per row on a cluster up to 850 entries a level (3D
-//    20^3 k = 2, e = 394: 0.30 ms, grid 0.36; 27-point 20^3 k = 1, e = 868: 0.46
-//    / 0.44), with helpers where rows hold 60 entries or more;
+//  * longer rows: a warp per row on a cluster up to e + 3 r = 850 (cluster / grid: 3D
+//    20^3 k = 2 (489) 0.30 / 0.36 ms, random band n = 20,000 k = 0 (667) 0.31 / 0.34,
+//    n = 160,000 k = 1 (680) 9.7 / 12.0, k = 0 (1,386) 1.98 / 1.39, n = 40,000 with 4 a
+//    row (980) 0.43 / 0.30, 27-point 20^3 k = 0 (878) 0.245 / 0.238, k = 1 (948) 0.46 /
+//    0.42), with helpers where rows hold 60 entries or more;
 //  * else the warp-per-row grid.
 // With the forward DAG's shape for both directions one-sided patterns lose (one
 // application: upper bidiagonal, n = 6,000, 3.15 ms, with its own 2.11; 2D 256^2
 // upwind 0.53 and 0.28).
 // Without level orders the depth is unknown, but above n / 64 (see factor_impl):
 // narrow.
-static int shape_direction(const iluk_sym *S, const LevelOrder &lo) {
+static int shape_direction(const iluk_sym *S, const LevelOrder &lo, bool forward,
+                           cudaStream_t s) {
   const double n = (double)S->n, depth = std::max(lo.nlev, 1);
-  const double e = (double)lo.entries / depth, r = n / depth;
+  const double e = (double)lo.entries / depth, r = n / depth, work = e + 2.0 * r;
   const int grid = ILUK_SCHED_WIDTH(ILUK_SCHED_WARP_GRID, 512);
-  if (lo.longest <= kRingSide) {
-    const double w = e + 2.0 * r;
-    return w <= 390.0 ? ILUK_SCHED_SINGLE_CTA : w <= 1300.0 ? ILUK_SCHED_CLUSTER : grid;
-  }
-  if (std::max(e, 2.0 * r) <= 850.0) {
-    const int wc = 2.0 * (double)lo.entries + n >= 60.0 * n ? ILUK_SCHED_WARP_CLUSTER_HELP
-                                                            : ILUK_SCHED_WARP_CLUSTER;
-    const int w = r >= 20.0 ? 512 : 384;
-    return ILUK_SCHED_WIDTH(wc, w);
-  }
-  return grid;
+  if (lo.longest <= kRingSide && work > 1300.0) return grid;
+  if (lo.longest <= kRingSide &&
+      ring_suits(forward, S->n, S->rowptr, S->colind, S->diag, lo, s))
+    return work <= (lo.longest > 4 ? 410.0 : 390.0) ? ILUK_SCHED_SINGLE_CTA : ILUK_SCHED_CLUSTER;
+  if (e + 3.0 * r > 850.0) return grid;
+  const int wc = 2.0 * (double)lo.entries + n >= 60.0 * n ? ILUK_SCHED_WARP_CLUSTER_HELP
+                                                          : ILUK_SCHED_WARP_CLUSTER;
+  return r >= 20.0 ? ILUK_SCHED_WIDTH(wc, 512) : ILUK_SCHED_WIDTH(wc, 384);
 }
 
-static int shape_schedule(const iluk_sym *S) {
+static int shape_schedule(const iluk_sym *S, cudaStream_t s) {
   if (S->n == 0) return ILUK_SCHED_WARP_GRID;
   auto pair = [](int f, int b) { return f == b ? f : f | (b << 8); };
   if (!S->levels_built) {
@@ -1086,7 +1087,7 @@ static int shape_schedule(const iluk_sym *S) {
                                                          : ILUK_SCHED_WARP_CLUSTER;
     return pair(ILUK_SCHED_WIDTH(wc, 512), ILUK_SCHED_WIDTH(wc, 384));
   }
-  return pair(shape_direction(S, S->lord), shape_direction(S, S->uord));
+  return pair(shape_direction(S, S->lord, true, s), shape_direction(S, S->uord, false, s));
 }
 
 // Autotuner: time the sweep schedules that suit the shape of F's DAGs (the
@@ -1890,7 +1891,7 @@ static int gmres_impl(const iluk_pattern *A, const double *A_val, int prec_kind,
           if (info) *info = finfo;
           return hst;
         }
-        if (F->sched == ILUK_SCHED_AUTO) F->sched = shape_schedule(F->S);
+        if (F->sched == ILUK_SCHED_AUTO) F->sched = shape_schedule(F->S, s);
         sched = F->sched;
         const int ost = orders_for(F, sched, s);
         if (ost != ILUK_OK) return fail(info, ost);

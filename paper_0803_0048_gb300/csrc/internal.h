@@ -25,6 +25,7 @@ struct LanePlan {
   int64_t nch = 0;
   int maxw = 0;                    // longest chain
   bool refused = false;            // no plan: it would take too much memory
+  int64_t far = 0;                 // inputs too far back for the ring
   const int64_t *coff = nullptr;   // int64[nch + 1]
   const int64_t *first = nullptr;  // per slot: position in F of the chain's first entry
   const int32_t *len = nullptr;    // per slot: chain length
@@ -273,6 +274,10 @@ cudaError_t launch_apply_backward(int64_t n, const int64_t *rp, const int32_t *c
                                   const int64_t *dg, const double *v, const DivPrep *rd,
                                   const LevelOrder &bwd, double *tmp, double *y, int sched,
                                   DevErr *err, const SweepAux *aux, cudaStream_t s);
+// Whether the ring sweeps suit this order's rows (they have a plan, made here if need
+// be, and next to no inputs from beyond the ring).  Synchronous.
+bool ring_suits(bool forward, int64_t n, const int64_t *rp, const int32_t *ci, const int64_t *dg,
+                const LevelOrder &lo, cudaStream_t s);
 // y = (LU)^-1 p (or ^-T on the transposed arrays).  tmp must hold the pending
 // marker in every entry on entry, and does again on exit.
 cudaError_t launch_apply(int64_t n, const int64_t *rp, const int32_t *ci, const int64_t *dg,

@@ -561,7 +561,9 @@ __global__ void k_lane_rows(const int32_t *__restrict__ order, int64_t nch,
 
 template <bool FORWARD>
 __global__ void k_lane_slots(LanePlan pl, const int32_t *__restrict__ slot_of,
-                             const int32_t *__restrict__ ci, int32_t *pslot) {
+                             const int32_t *__restrict__ ci, int32_t *pslot,
+                             unsigned long long *far) {
+  unsigned long long beyond = 0;
   const int lane = threadIdx.x & 31;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t c = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; c < pl.nch; c += nw) {
@@ -572,11 +574,14 @@ __global__ void k_lane_slots(LanePlan pl, const int32_t *__restrict__ slot_of,
       if (e >= skip) {
         const int32_t col = ci[FORWARD ? f + (e - skip) : f - (e - skip)];
         const int32_t sl = slot_of[col];
-        v = slot - sl < kRingNear ? sl : far_code(col);
+        const bool near = slot - sl < kRingNear;
+        v = near ? sl : far_code(col);
+        beyond += near ? 0 : 1;
       }
       pslot[(off + e) * 32 + lane] = v;
     }
   }
+  if (beyond) atomicAdd(far, beyond);
 }
 
 // ---------------------------------------------------------------------------
@@ -1153,6 +1158,7 @@ static bool ensure_lane_plan(const LevelOrder &lo_c, int64_t n, const int64_t *r
   pl.nch = lo.len / 32;
   int32_t *slot_of = nullptr, *w = nullptr, *len = nullptr, *pslot = nullptr;
   int64_t *first = nullptr, *coff = nullptr, *scan_tmp = nullptr;
+  unsigned long long far = 0;
   auto free_all = [&](bool keep) {
     for (void *p : {(void *)slot_of, (void *)w, (void *)scan_tmp})
       if (p) cudaFreeAsync(p, s);
@@ -1188,13 +1194,31 @@ static bool ensure_lane_plan(const LevelOrder &lo_c, int64_t n, const int64_t *r
   pl.len = len;
   pl.first = first;
   pl.coff = coff;
-  k_lane_slots<FORWARD><<<row_blocks(lo.len), 256, 0, s>>>(pl, slot_of, ci, pslot);
+  // (the scan is done with its scratch)
+  unsigned long long *dfar = reinterpret_cast<unsigned long long *>(scan_tmp);
+  if (cudaMemsetAsync(dfar, 0, sizeof(far), s) != cudaSuccess) return free_all(false);
+  k_lane_slots<FORWARD><<<row_blocks(lo.len), 256, 0, s>>>(pl, slot_of, ci, pslot, dfar);
   note_launch();
   // complete before another stream's sweep may find it
-  if (cudaStreamSynchronize(s) != cudaSuccess) return free_all(false);
+  if (cudaGetLastError() != cudaSuccess ||
+      cudaMemcpyAsync(&far, dfar, sizeof(far), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+      cudaStreamSynchronize(s) != cudaSuccess)
+    return free_all(false);
+  pl.far = (int64_t)far;
   pl.slot = pslot;
   lo.plan = pl;
   return free_all(true);
+}
+
+// An input from beyond the ring costs its chunk a look at the clock, the error word
+// and global memory, ~1 us, so a chunk in few may have one: random bands, whose
+// rows without inputs all lie in level 1, run 2.5 times slower on the ring than on
+// a cluster (n = 40,000, 3 a row, half-width 300: 1.31 / 0.52 ms an application).
+bool ring_suits(bool forward, int64_t n, const int64_t *rp, const int32_t *ci, const int64_t *dg,
+                const LevelOrder &lo, cudaStream_t s) {
+  const bool planned = forward ? ensure_lane_plan<true>(lo, n, rp, ci, dg, s)
+                               : ensure_lane_plan<false>(lo, n, rp, ci, dg, s);
+  return planned && 100 * lo.plan.far <= lo.entries;
 }
 
 __global__ void k_fill_pending(int64_t n, double *x, unsigned long long bits) {

@@ -120,3 +120,32 @@ def test_one_call_pick_counts_rows_too(N, k, kind):
     b, bd = vec(83, A.n)
     x, info, (S, F) = P.solve(rp, ci, av, bd, k, maxit=2, check=False, return_factors=True)
     assert kinds(F.schedule()) == (kind, kind)
+
+
+@pytest.mark.parametrize("n,hw,kind", [(160000, 2000, L.SCHED_WARP_GRID),
+                                       (40000, 500, L.SCHED_WARP_CLUSTER)])
+def test_one_call_pick_for_longer_rows_counts_rows_too(n, hw, kind):
+    """Random bands of 9 entries a row, k = 0: 861 levels of 186 rows go to all
+    SMs (an application 1.39 ms, on a cluster 1.98), 790 of 51 to a cluster
+    (0.78 ms; all SMs 1.30)."""
+    A = W.random_band(n, 9, hw, 77)
+    rp, ci, av = to_dev(A)
+    b, bd = vec(84, n)
+    x, info, (S, F) = P.solve(rp, ci, av, bd, 0, maxit=2, check=False, return_factors=True)
+    assert S.max_row <= 17 and kinds(F.schedule()) == (kind, kind)
+
+
+def test_one_call_pick_leaves_the_ring_where_inputs_lie_far():
+    """Short rows, 85 a level, but one in eight has no lower entries: level 1
+    holds rows from everywhere, far behind the ring for most of their readers."""
+    A = W.random_band(40000, 3, 300, 1)
+    rp, ci, av = to_dev(A)
+    b, bd = vec(85, A.n)
+    x, info, (S, F) = P.solve(rp, ci, av, bd, 0, return_factors=True)
+    assert S.max_row <= 4 and kinds(F.schedule()) == (L.SCHED_WARP_CLUSTER, L.SCHED_WARP_CLUSTER)
+    ref = oracle.factor(A, 0)
+    st, xo, it, *_ = oracle.gmres(A.n, A.rowptr, A.colind, A.val, b, oracle.PREC_ILU,
+                                  (ref["rowptr"], ref["colind"], ref["val"]), 30, 1e-8,
+                                  dotmode=oracle.DOT_TREE)
+    assert st == oracle.OK and info.iters == it
+    assert_bits_equal(x, xo, "far inputs")
