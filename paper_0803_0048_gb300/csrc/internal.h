@@ -248,6 +248,7 @@ cudaError_t build_fill_pattern(int64_t n, int64_t nnz, const int64_t *arp, const
                                int64_t max_row, cudaStream_t s);
 
 // Levels (levels.cu): synchronous; allocates both orders on success.
+constexpr int64_t kLevelOrderRows = 20000;  // least rows of a DAG for which orders come first
 constexpr int kLevelsTooDeep = -1, kLevelsLinear = -2;
 int build_levels_pair(int64_t n, const int64_t *rp, const int32_t *ci, const int64_t *dg,
                       LevelOrder *fwd, LevelOrder *bwd, int cap, int cap_b, bool growth,
@@ -259,6 +260,7 @@ cudaError_t launch_pivot_info(int64_t n, const int64_t *frp, const int32_t *fci,
                               const int64_t *fdiag, int64_t *pinfo, cudaStream_t s);
 // v0, xf (may be null): also L x = v0 into xf, which holds the pending marker
 // in every entry, each row's entry as soon as the row is factored.
+void numeric_prepare(const iluk_sym *S, cudaStream_t s);  // what launch_numeric makes once
 cudaError_t launch_numeric(const iluk_sym *S, const double *aval, double *fval, DivPrep *rdiag,
                            unsigned long long *ticket, DevErr *err, const double *v0, double *xf,
                            cudaStream_t s);

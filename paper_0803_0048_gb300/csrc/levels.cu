@@ -15,7 +15,6 @@ namespace iluk {
 
 constexpr int kDepthThreads = 512;
 constexpr int kWindowRows = 2048;          // about the rows in flight of a numeric phase
-constexpr int64_t kLevelOrderRows = 20000;  // least rows of a DAG for which orders come first
 constexpr int kDepthBatch = 4;  // inputs a lane looks at together
 
 // One row per lane: a warp claims the next 32 rows in sweep order through a

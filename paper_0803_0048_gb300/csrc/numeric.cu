@@ -1168,6 +1168,14 @@ static bool ensure_stage_plan(const iluk_sym *Sc, cudaStream_t s) {
   return leave(1);
 }
 
+// Whether the rows go by an update plan, and the plan made ahead of their launch.
+static bool staged_rows(const iluk_sym *S, cudaStream_t s) {
+  return S->levels_built && S->lord.corder != nullptr &&
+         S->n >= kStageLevelRows * (int64_t)S->lord.nlev && ensure_stage_plan(S, s);
+}
+
+void numeric_prepare(const iluk_sym *S, cudaStream_t s) { staged_rows(S, s); }
+
 static cudaError_t launch_numeric_impl(const iluk_sym *S, int64_t nbatch, const double *avals,
                                        double *fvals, DivPrep *rdiag, unsigned long long *ticket,
                                        DevErr *errs, const double *v0, double *xf,
@@ -1176,8 +1184,7 @@ static cudaError_t launch_numeric_impl(const iluk_sym *S, int64_t nbatch, const 
   const int32_t *order = S->levels_built ? S->lord.corder : nullptr;
   ProfScope prof_scope(ILUK_PROF_NUMERIC, s);
   const bool wide = order != nullptr && S->n >= kWideLevelRows * (int64_t)S->lord.nlev;
-  const bool staged = nbatch == 1 && order != nullptr &&
-                      S->n >= kStageLevelRows * (int64_t)S->lord.nlev && ensure_stage_plan(S, s);
+  const bool staged = nbatch == 1 && staged_rows(S, s);
   // rows publish their entries as soon as final (see apply_pivots) where F's
   // rows are long, or where a level holds few entries of L (fewer than
   // kEarlyLevelEntries: the band matrices at k <= 1 gain 15-35 %), or before
