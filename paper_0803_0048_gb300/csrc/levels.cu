@@ -88,13 +88,11 @@ __device__ __noinline__ bool growth_look(int64_t n, int64_t t0r, int m, DepthGro
 template <bool FORWARD>
 __device__ void depth_rows(int64_t n, const int64_t *__restrict__ rp,
                            const int32_t *__restrict__ ci, const int64_t *__restrict__ dg,
-                           int32_t *depth, int32_t *maxdepth, int32_t *longest,
-                           unsigned long long *entries, DevErr *err, int64_t limit_ns,
+                           int32_t *depth, int32_t *maxdepth, DevErr *err, int64_t limit_ns,
                            unsigned long long *ticket, int *fail, int *other, int cap,
                            DepthGrowth *g, const GrowthRows &gr) {
   const int lane = threadIdx.x & 31;
-  int dmax_local = 0, longest_local = 0;
-  int64_t entries_local = 0;
+  int dmax_local = 0;
   for (;;) {
     unsigned long long tk = 0;
     if (lane == 0) tk = atomicAdd(ticket, 32ull);
@@ -110,8 +108,6 @@ __device__ void depth_rows(int64_t n, const int64_t *__restrict__ rp,
       const int64_t d = dg[row];
       first = FORWARD ? rp[row] : rp[row + 1] - 1;
       len = (int)(FORWARD ? d - first : first - d);
-      entries_local += len;
-      if (len > longest_local) longest_local = len;
     }
     int q = 0, dm = 0;
     bool done = !mine;
@@ -196,36 +192,58 @@ __device__ void depth_rows(int64_t n, const int64_t *__restrict__ rp,
     }
   }
   dmax_local = __reduce_max_sync(FULL_MASK, dmax_local);
-#pragma unroll
-  for (int o = 16; o >= 1; o >>= 1)
-    entries_local += __shfl_xor_sync(FULL_MASK, entries_local, o);
-  longest_local = __reduce_max_sync(FULL_MASK, longest_local);
   if (lane == 0 && dmax_local) atomicMax(maxdepth, dmax_local);
-  if (lane == 0 && longest_local) atomicMax(longest, longest_local);
-  if (lane == 0 && entries_local) atomicAdd(entries, (unsigned long long)entries_local);
 }
 
 // Even CTAs compute the forward depths, odd CTAs the backward depths (the two
-// DAGs are independent).  mx: the two depths, the two longest rows; ctl: two
-// tickets, the two DAGs' entries, two failure flags.
+// DAGs are independent).  ctl: two tickets, then two failure flags.
 __global__ void __launch_bounds__(kDepthThreads)
 k_depth_pair(int64_t n, const int64_t *__restrict__ rp, const int32_t *__restrict__ ci,
              const int64_t *__restrict__ dg, int32_t *depth_f, int32_t *depth_b, int32_t *mx,
              DevErr *err, unsigned long long *ctl, int64_t limit_ns, int cap, int cap_b,
              DepthGrowth *g, GrowthRows gr) {
-  int *fail = reinterpret_cast<int *>(ctl + 4);
+  int *fail = reinterpret_cast<int *>(ctl + 2);
   if ((blockIdx.x & 1) == 0)
-    depth_rows<true>(n, rp, ci, dg, depth_f, mx, mx + 2, ctl + 2, err, limit_ns, ctl, fail,
-                     fail + 1, cap, g, gr);
+    depth_rows<true>(n, rp, ci, dg, depth_f, mx, err, limit_ns, ctl, fail, fail + 1, cap, g, gr);
   else
-    depth_rows<false>(n, rp, ci, dg, depth_b, mx + 1, mx + 3, ctl + 3, err + 1, limit_ns, ctl + 1,
-                      fail + 1, fail, cap_b, nullptr, gr);
+    depth_rows<false>(n, rp, ci, dg, depth_b, mx + 1, err + 1, limit_ns, ctl + 1, fail + 1, fail,
+                      cap_b, nullptr, gr);
 }
 
-__global__ void k_level_count(int64_t n, const int32_t *__restrict__ depth, int32_t *cnt) {
+// Rows per level; shape[0], shape[1] (0 before): the entries the sweep reads, and the
+// most of a row.
+template <bool FORWARD>
+__global__ void k_level_count(int64_t n, const int32_t *__restrict__ depth,
+                              const int64_t *__restrict__ rp, const int64_t *__restrict__ dg,
+                              int32_t *cnt, unsigned long long *shape) {
+  __shared__ unsigned long long entries;
+  __shared__ int longest;
+  if (threadIdx.x == 0) {
+    entries = 0;
+    longest = 0;
+  }
+  __syncthreads();
+  unsigned long long e = 0;
+  int mx = 0;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x)
+       i += (int64_t)gridDim.x * blockDim.x) {
     atomicAdd(&cnt[depth[i] - 1], 1);
+    const int len = (int)(FORWARD ? dg[i] - rp[i] : rp[i + 1] - 1 - dg[i]);
+    e += (unsigned long long)len;
+    if (len > mx) mx = len;
+  }
+  mx = __reduce_max_sync(FULL_MASK, mx);
+#pragma unroll
+  for (int o = 16; o >= 1; o >>= 1) e += __shfl_xor_sync(FULL_MASK, e, o);
+  if ((threadIdx.x & 31) == 0) {
+    atomicAdd(&entries, e);
+    atomicMax(&longest, mx);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    if (entries) atomicAdd(&shape[0], entries);
+    if (longest) atomicMax(&shape[1], (unsigned long long)longest);
+  }
 }
 
 __global__ void k_level_pad(int64_t nlev, int32_t *cnt) {
@@ -253,8 +271,9 @@ static unsigned grid_for(int64_t n) {
 
 // Padded level order from depths, and the same order without padding
 // (synchronous).
-static int order_from_depth(int64_t n, const int32_t *depth, int32_t nlev, LevelOrder *lo,
-                            cudaStream_t s) {
+template <bool FORWARD>
+static int order_from_depth(int64_t n, const int32_t *depth, const int64_t *rp, const int64_t *dg,
+                            int32_t nlev, LevelOrder *lo, cudaStream_t s) {
   int32_t *cnt = nullptr, *cursor = nullptr;
   int64_t *lstart = nullptr, *scan_tmp = nullptr, *cstart = nullptr;
   auto cleanup = [&]() {
@@ -276,20 +295,24 @@ static int order_from_depth(int64_t n, const int32_t *depth, int32_t nlev, Level
   } while (0)
   CKL(cudaMallocAsync((void **)&cnt, (size_t)nlev * sizeof(int32_t), s));
   CKL(cudaMallocAsync((void **)&cursor, (size_t)nlev * sizeof(int32_t), s));
-  CKL(cudaMallocAsync((void **)&lstart, ((size_t)nlev + 1) * sizeof(int64_t), s));
+  // the level starts, the order's length, and what k_level_count finds
+  CKL(cudaMallocAsync((void **)&lstart, ((size_t)nlev + 3) * sizeof(int64_t), s));
+  CKL(cudaMemsetAsync(lstart + nlev + 1, 0, 2 * sizeof(int64_t), s));
   CKL(cudaMallocAsync((void **)&scan_tmp, (size_t)scan_tmp_elems(nlev) * sizeof(int64_t), s));
   CKL(cudaMemsetAsync(cnt, 0, (size_t)nlev * sizeof(int32_t), s));
   CKL(cudaMemsetAsync(cursor, 0, (size_t)nlev * sizeof(int32_t), s));
   CKL(cudaMallocAsync((void **)&cstart, ((size_t)nlev + 1) * sizeof(int64_t), s));
-  k_level_count<<<grid_for(n), 256, 0, s>>>(n, depth, cnt);
+  k_level_count<FORWARD><<<grid_for(n), 256, 0, s>>>(
+      n, depth, rp, dg, cnt, reinterpret_cast<unsigned long long *>(lstart + nlev + 1));
   note_launch();
   CKL(launch_scan_lengths(nlev, cnt, cstart, scan_tmp, s));  // unpadded level starts
   k_level_pad<<<grid_for(nlev), 256, 0, s>>>(nlev, cnt);
   note_launch();
   CKL(launch_scan_lengths(nlev, cnt, lstart, scan_tmp, s));
-  int64_t len = 0;
-  CKL(cudaMemcpyAsync(&len, lstart + nlev, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+  int64_t shape[3] = {0, 0, 0};
+  CKL(cudaMemcpyAsync(shape, lstart + nlev, sizeof(shape), cudaMemcpyDeviceToHost, s));
   CKL(cudaStreamSynchronize(s));
+  const int64_t len = shape[0];
   CKL(cudaMallocAsync((void **)&lo->order, (size_t)len * sizeof(int32_t), s));
   CKL(cudaMemsetAsync(lo->order, 0xff, (size_t)len * sizeof(int32_t), s));
   k_level_scatter<<<grid_for(n), 256, 0, s>>>(n, depth, lstart, cursor, lo->order);
@@ -304,6 +327,8 @@ static int order_from_depth(int64_t n, const int32_t *depth, int32_t nlev, Level
   lo->lstart = lstart;
   lo->len = len;
   lo->nlev = nlev;
+  lo->entries = shape[1];
+  lo->longest = (int32_t)shape[2];
   lo->clen = n;
   return ILUK_OK;
 }
@@ -324,7 +349,7 @@ int build_levels_pair(int64_t n, const int64_t *rp, const int32_t *ci, const int
   if (n == 0) return ILUK_OK;
   int32_t *depth = nullptr, *mx = nullptr;
   DevErr *err = nullptr;
-  unsigned long long *ctl = nullptr;  // two tickets, two entry counts, two failure flags
+  unsigned long long *ctl = nullptr;  // two tickets, two failure flags
   if (growth && n < kLevelOrderRows) return kLevelsLinear;
   DepthGrowth *g = nullptr;
   GrowthRows gr = {};
@@ -350,12 +375,12 @@ int build_levels_pair(int64_t n, const int64_t *rp, const int32_t *ci, const int
     return ILUK_ECUDA;
   }
   if (cudaMallocAsync((void **)&depth, 2 * n * sizeof(int32_t), s) != cudaSuccess ||
-      cudaMallocAsync((void **)&mx, 4 * sizeof(int32_t), s) != cudaSuccess ||
+      cudaMallocAsync((void **)&mx, 2 * sizeof(int32_t), s) != cudaSuccess ||
       cudaMallocAsync((void **)&err, 2 * sizeof(DevErr), s) != cudaSuccess ||
-      cudaMallocAsync((void **)&ctl, 5 * sizeof(unsigned long long), s) != cudaSuccess ||
+      cudaMallocAsync((void **)&ctl, 3 * sizeof(unsigned long long), s) != cudaSuccess ||
       cudaMemsetAsync(depth, 0, 2 * n * sizeof(int32_t), s) != cudaSuccess ||
-      cudaMemsetAsync(mx, 0, 4 * sizeof(int32_t), s) != cudaSuccess ||
-      cudaMemsetAsync(ctl, 0, 5 * sizeof(unsigned long long), s) != cudaSuccess ||
+      cudaMemsetAsync(mx, 0, 2 * sizeof(int32_t), s) != cudaSuccess ||
+      cudaMemsetAsync(ctl, 0, 3 * sizeof(unsigned long long), s) != cudaSuccess ||
       launch_fill_err(err, s) != cudaSuccess || launch_fill_err(err + 1, s) != cudaSuccess) {
     cleanup();
     return ILUK_ECUDA;
@@ -372,17 +397,11 @@ int build_levels_pair(int64_t n, const int64_t *rp, const int32_t *ci, const int
                                                         ctl, wait_limit(), cap, cap_b, g, gr);
   note_launch();
   DevErr herr[2];
-  int32_t nlev[4] = {0, 0, 0, 0};  // and the longest rows
-  struct {
-    unsigned long long ticket[2], entries[2];
-    int32_t fail[2];
-  } hctl = {};
-  static_assert(sizeof(hctl) == 5 * sizeof(unsigned long long), "as the kernel lays ctl out");
-  const int32_t *fail = hctl.fail;
+  int32_t nlev[2] = {0, 0}, fail[2] = {0, 0};
   if (cudaGetLastError() != cudaSuccess ||
       cudaMemcpyAsync(herr, err, sizeof(herr), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
       cudaMemcpyAsync(nlev, mx, sizeof(nlev), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-      cudaMemcpyAsync(&hctl, ctl, sizeof(hctl), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+      cudaMemcpyAsync(fail, ctl + 2, sizeof(fail), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess) {
     cleanup();
     return ILUK_ECUDA;
@@ -400,12 +419,8 @@ int build_levels_pair(int64_t n, const int64_t *rp, const int32_t *ci, const int
     cleanup();
     return kLevelsTooDeep;
   }
-  int st = order_from_depth(n, depth, nlev[0], fwd, s);
-  if (st == ILUK_OK) st = order_from_depth(n, depth + n, nlev[1], bwd, s);
-  fwd->entries = (int64_t)hctl.entries[0];
-  bwd->entries = (int64_t)hctl.entries[1];
-  fwd->longest = nlev[2];
-  bwd->longest = nlev[3];
+  int st = order_from_depth<true>(n, depth, rp, dg, nlev[0], fwd, s);
+  if (st == ILUK_OK) st = order_from_depth<false>(n, depth + n, rp, dg, nlev[1], bwd, s);
   // the orders are read on other streams than the one they were built on (beside
   // a numeric phase; another caller's), which nothing else makes wait
   if (st == ILUK_OK && cudaStreamSynchronize(s) != cudaSuccess) st = ILUK_ECUDA;
