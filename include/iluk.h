@@ -168,9 +168,9 @@ int64_t iluk_launch_count(void);
  * those events and fills ms[kind] (total milliseconds) and count[kind]
  * (launches) for kind < nkinds (host arrays).  Enabling clears the records.
  * OVERLAPPED collects the work a call runs on a second stream beside its main
- * kernel (the level orders of a deep, narrow DAG, built beside the first
- * numeric phase of a pattern): its time is hidden, not added, so it is kept
- * apart. */
+ * kernel (the level orders of patterns whose rows index order serves as well,
+ * built beside their first numeric phase): its time is hidden, not added, so it
+ * is kept apart. */
 enum {
   ILUK_PROF_VALIDATE = 0, ILUK_PROF_SYMBOLIC = 1, ILUK_PROF_COMPACT = 2, ILUK_PROF_DEPTH = 3,
   ILUK_PROF_NUMERIC = 4, ILUK_PROF_SWEEP = 5 /* forward sweeps */, ILUK_PROF_TRANSPOSE = 6, ILUK_PROF_IILU_BUILD = 7,
@@ -204,8 +204,9 @@ int iluk_sym_query(const iluk_sym *S, iluk_sym_view *view);
 /* Longest dependency chains of the forward and backward sweeps over F's
  * pattern (the number of rows on the critical path of each sweep).  They come
  * with the sweeps' level orders, which the first iluk_numeric on S builds before
- * its rows, or beside them on a deep, narrow DAG; if none has run yet, this call
- * builds them (synchronous on `stream`).  Cached in S afterwards. */
+ * its rows, or beside them (deep and narrow DAGs, few rows, rows that index order
+ * serves as well); if none has run yet, this call builds them (synchronous on
+ * `stream`).  Cached in S afterwards. */
 int iluk_sym_depth(iluk_sym *S, int32_t *depth_lower, int32_t *depth_upper, void *stream);
 /* Copy S's arrays into caller-owned device buffers (any pointer may be NULL
  * to skip that array).  Asynchronous. */
@@ -235,7 +236,8 @@ int iluk_refactor(iluk_fac *F, const double *A_val, iluk_info *info, void *strea
  * dependency first gives the same bits) until a later iluk_numeric or
  * iluk_refactor on S, or iluk_sym_depth, builds them.
  * The phases run one after the other where rows need not wait for one another's
- * patterns (k <= 1, and k >= 2 on patterns of limited reach).  Else (k >= 2) the
+ * patterns (k <= 1, and k >= 2 on patterns of limited reach, except those that
+ * reach across the matrix at a high k).  Else (k >= 2) the
  * numeric phase runs beside the symbolic one, in one launch in which each row is
  * factored as soon as its pattern is final, its values kept in an arena laid out
  * like the symbolic one until both phases end; that launch falls back to the two

@@ -20,7 +20,8 @@
 // afterwards (Sec. 3.4).
 //
 // This walk takes the patterns of k >= 2 that fill.cu, which needs no waits, does not
-// (fill_window: those that reach too far, or across the matrix at a high k), and those whose general walk is asked for.
+// (fill_window: those that reach too far, or across the matrix at a high k), and
+// those whose general walk is asked for.
 //
 // With k <= 1 rows are independent (Sec. 3.3: only level-0 entries can cause
 // fill), so the warp reads the pivot rows straight from A and never waits;
